@@ -120,6 +120,8 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
   o = align_up(o + sizeof(int32_t) * std::max(B, 1));
   pl->off_gbar = o;   // abort word and one barrier counter per request slot
   o = align_up(o + sizeof(uint32_t) * (1 + kGridMaxReq));
+  pl->off_tile0 = o;
+  o = align_up(o + sizeof(int32_t) * (B + 1));
   const size_t blob_end = o;
   pl->off_stats = o;
   o = align_up(o + sizeof(float) * 4 * (size_t)std::max(pl->L, 0) * std::max(pl->Hq, 0) *
@@ -148,6 +150,31 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
   // the whole-GPU selection's published keys, for launches that may take it
   pl->off_gpub = o;
   if (B <= kGridMaxReq && pl->max_vis >= kGridMinTokens) o = align_up(o + grid_pub_bytes());
+  pl->base_bytes = o;
+  // The greedy from a Gram matrix: N_b rows of gram_ld(N_b) floats for every request
+  // that has a choice to make (1 < k_b < N_b).
+  auto gram_units = [&](int b) -> long long {
+    const int n = p->cu_vis[b + 1] - p->cu_vis[b], kb = p->cu_keep[b + 1] - p->cu_keep[b];
+    return kb > 1 && kb < n ? (long long)n * (gram_ld(n) / 32) : 0;
+  };
+  long long units = 0;
+  if (sel_scratch)
+    for (int b = 0; b < B; ++b) units += gram_units(b);
+  // Used where the contraction (about 1.1 PFLOP/s over the lower triangle) costs less
+  // than the rounds over X that it replaces: those accept about 16 picks a round and
+  // take about 100 us each, and the longest request's rounds set the call's time.
+  // Eight requests of 16384 x 2048: 3.7 ms against 16.6 ms at k = 2048, 8.5 ms at 1024;
+  // the line lies near k = 700.
+  double gram_s = 0.0;
+  if (sel_scratch)
+    for (int b = 0; b < B; ++b) gram_s += (double)gram_units(b) * 32.0 * p->feat_dim / 1.1e15;
+  pl->gram = units > 0 && units * 128 <= kGramMaxBytes && gram_s <= 6e-6 * pl->max_keep;
+  if (pl->gram) {
+    pl->off_rn = o;
+    o = align_up(o + sizeof(float) * (size_t)pl->total_vis);
+    pl->off_gram = o;
+    o = align_up(o + (size_t)units * 128);
+  }
   pl->total_bytes = o;
 
   // ---- host staging: [err words][meta][items][order], one copy ----
@@ -156,10 +183,17 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
   int32_t *meta = pl->host_blob.data() + pl->off_meta / 4;
   int32_t *items = pl->host_blob.data() + pl->off_items / 4;
   int32_t *order = pl->host_blob.data() + pl->off_order / 4;
+  int32_t *tile0 = pl->host_blob.data() + pl->off_tile0 / 4;
   int chunk = 0;
-  long long root_off = 0;
+  long long root_off = 0, gram_off = 0;
   for (int b = 0; b < B; ++b) {
     int32_t *m = meta + b * kMetaFields;
+    tile0[b] = pl->gram_tiles;
+    if (pl->gram) {
+      m[kGramOff] = (int32_t)gram_off;
+      gram_off += gram_units(b);
+      if (gram_units(b) > 0) pl->gram_tiles += gram_tiles(p->cu_vis[b + 1] - p->cu_vis[b]);
+    }
     m[kRootOff] = (int32_t)root_off;
     if (sel_scratch) root_off += root_cap(b);
     m[kVisOff] = p->cu_vis[b];
@@ -179,6 +213,7 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
       chunk += nch;
     }
   }
+  tile0[B] = pl->gram_tiles;
   // selection clusters take the most expensive requests (k_b * N_b) first
   std::vector<int> ord(B);
   std::iota(ord.begin(), ord.end(), 0);
@@ -193,11 +228,12 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
 
 namespace {
 
-last_status check_ws(const Plan &pl, const void *ws, size_t ws_bytes, bool scores_only = false) {
+last_status check_ws(const Plan &pl, const void *ws, size_t ws_bytes, bool scores_only = false,
+                     bool select = false) {
   if (ws == nullptr) return fail(LAST_ERR_INVALID_ARG, "workspace is NULL");
   if ((reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0)
     return fail(LAST_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
-  const size_t need = scores_only ? pl.score_bytes : pl.total_bytes;
+  const size_t need = scores_only ? pl.score_bytes : select ? pl.total_bytes : pl.base_bytes;
   if (ws_bytes < need)
     return fail(LAST_ERR_WORKSPACE_TOO_SMALL, "workspace needs " + std::to_string(need) + " bytes");
   return LAST_OK;
@@ -286,7 +322,7 @@ last_status last_select(const last_problem *p, const float *w, const void *x, in
   last_status st = make_plan(p, false, true, &pl);
   if (st != LAST_OK) return st;
   if ((st = check_select_fits(pl)) != LAST_OK) return st;
-  if ((st = check_ws(pl, ws, ws_bytes)) != LAST_OK) return st;
+  if ((st = check_ws(pl, ws, ws_bytes, false, true)) != LAST_OK) return st;
   if (pl.total_keep > 0 && (w == nullptr || x == nullptr || idx_out == nullptr))
     return fail(LAST_ERR_INVALID_ARG, "w, x and idx_out are required");
   if (!aligned16(x) || !aligned16(x_out))
@@ -355,7 +391,7 @@ last_status last_prune(const last_problem *p, const void *q, const void *k, cons
   last_status st = make_plan(p, true, true, &pl);
   if (st != LAST_OK) return st;
   if ((st = check_select_fits(pl)) != LAST_OK) return st;
-  if ((st = check_ws(pl, ws, ws_bytes)) != LAST_OK) return st;
+  if ((st = check_ws(pl, ws, ws_bytes, false, true)) != LAST_OK) return st;
   if (pl.total_vis > 0 && (q == nullptr || k == nullptr || x == nullptr))
     return fail(LAST_ERR_INVALID_ARG, "q, k and x are required");
   if (pl.total_keep > 0 && idx_out == nullptr)

@@ -22,6 +22,7 @@ enum MetaField : int {
   kNumKeep,        // k_b
   kChunkBase,      // first score chunk of request b
   kRootOff,        // first row of request b in the selection's root rows
+  kGramOff,        // request b's Gram matrix, in units of 32 floats
   kMetaFields
 };
 
@@ -35,6 +36,7 @@ constexpr int kSelectWarps = 8;
 constexpr int kGridMaxReq = 4;      // requests of one whole-GPU selection launch
 constexpr int kGridMaxCtas = 256;   // CTAs of one whole-GPU selection launch at most
 constexpr int kGatherThreads = 256;
+constexpr long long kGramMaxBytes = 12LL << 30;   // Gram matrices of one call at most
 
 // Device error flags (first word of the workspace).
 constexpr unsigned kErrGatherIndex = 1u;
@@ -60,6 +62,11 @@ struct Plan {
   // published keys
   size_t off_gbar = 0, off_gpub = 0;
   long long root_rows = 0;
+  // selection from a Gram matrix: 1/|x| per token, the matrices, first tile per request.
+  // base_bytes excludes the first two (Top-k and the gather do not use them).
+  size_t off_rn = 0, off_gram = 0, off_tile0 = 0, base_bytes = 0;
+  int gram_tiles = 0;
+  bool gram = false;
   // host staging (error word, meta rows, score items, selection order) in ws order
   std::vector<int32_t> host_blob;
   size_t blob_bytes = 0;  // bytes from off_meta to the end of the order array
@@ -85,6 +92,18 @@ cudaError_t launch_gather(const Plan &pl, const void *x, const int32_t *idx, voi
 // The whole-GPU selection of a few long requests (select_grid.cu).
 cudaError_t launch_select_grid(const Plan &pl, const float *w, const void *x, int32_t *idx_out,
                                void *x_out, char *ws, cudaStream_t s);
+// The greedy from a Gram matrix (select_gram.cu); *done stays false, with nothing
+// launched, when the requests do not fit it.
+cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, int32_t *idx_out,
+                               void *x_out, char *ws, cudaStream_t s, bool *done);
+// Tiles of the Gram kernel for one request; floats per row of its matrix.
+int gram_tiles(int n_tokens);
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int gram_ld(int n_tokens) { return (n_tokens + 31) / 32 * 32; }
+// Clusters of `fn` (csize CTAs of `threads`, smem bytes each) resident at once, cached.
+int active_clusters(void *fn, int csize, size_t smem, int threads);
 size_t grid_select_smem(int row_bytes, int tpc);
 size_t grid_pub_bytes();
 // Whether the whole-GPU selection can run the plan's requests on the current device

@@ -323,6 +323,11 @@ __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
+// X as a [rows][dv] bf16 tensor, 64-element x box_rows boxes, 128-byte swizzle.
+bool encode_x_map(CUtensorMap *m, const void *x, long long rows, int dv, int box_rows = kTcBM);
+// Bound on |tensor-core distance - canonical distance|.
+float tc_distance_eps(int dv);
+
 template <typename T, int NCH, int TB, bool TC>
 __global__ void __launch_bounds__(kSelThreads, 1)
 select_kernel(const __grid_constant__ SelectArgs a) {

@@ -61,41 +61,6 @@ DeviceInfo device_info() {
   return d;
 }
 
-// Clusters of `fn` (csize CTAs, smem bytes each) resident at once, cached per
-// (device, kernel, cluster size, shared memory); 0 if it cannot be placed.
-int active_clusters(void *fn, int csize, size_t smem) {
-  static std::mutex mu;
-  static std::map<std::tuple<int, void *, int, size_t>, int> cache;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  const auto key = std::make_tuple(dev, fn, csize, smem);
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    auto hit = cache.find(key);
-    if (hit != cache.end()) return hit->second;
-  }
-  int active = 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
-    cudaLaunchConfig_t q = {};
-    q.gridDim = dim3(csize);
-    q.blockDim = dim3(kSelThreads);
-    q.dynamicSmemBytes = smem;
-    cudaLaunchAttribute qa[1];
-    qa[0].id = cudaLaunchAttributeClusterDimension;
-    qa[0].val.clusterDim.x = csize;
-    qa[0].val.clusterDim.y = 1;
-    qa[0].val.clusterDim.z = 1;
-    q.attrs = qa;
-    q.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&active, fn, &q) != cudaSuccess) active = 0;
-  }
-  cudaGetLastError();
-  std::lock_guard<std::mutex> lock(mu);
-  cache.emplace(key, active);
-  return active;
-}
-
 using EncodeTiledFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                    const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                                    const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -118,8 +83,45 @@ EncodeTiledFn encode_tiled() {
   return fn;
 }
 
+}  // namespace
+
+// Clusters of `fn` (csize CTAs of `threads`, smem bytes each) resident at once, cached per
+// (device, kernel, cluster size, shared memory); 0 if it cannot be placed.
+int active_clusters(void *fn, int csize, size_t smem, int threads) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, void *, int, size_t>, int> cache;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const auto key = std::make_tuple(dev, fn, csize, smem);
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    auto hit = cache.find(key);
+    if (hit != cache.end()) return hit->second;
+  }
+  int active = 0;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
+    cudaLaunchConfig_t q = {};
+    q.gridDim = dim3(csize);
+    q.blockDim = dim3(threads);
+    q.dynamicSmemBytes = smem;
+    cudaLaunchAttribute qa[1];
+    qa[0].id = cudaLaunchAttributeClusterDimension;
+    qa[0].val.clusterDim.x = csize;
+    qa[0].val.clusterDim.y = 1;
+    qa[0].val.clusterDim.z = 1;
+    q.attrs = qa;
+    q.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&active, fn, &q) != cudaSuccess) active = 0;
+  }
+  cudaGetLastError();
+  std::lock_guard<std::mutex> lock(mu);
+  cache.emplace(key, active);
+  return active;
+}
+
 // X as a [rows][dv] bf16 tensor, 64-element x box_rows boxes, 128-byte swizzle.
-bool encode_x_map(CUtensorMap *m, const void *x, long long rows, int dv, int box_rows = kTcBM) {
+bool encode_x_map(CUtensorMap *m, const void *x, long long rows, int dv, int box_rows) {
   EncodeTiledFn fn = encode_tiled();
   if (fn == nullptr || rows <= 0) return false;
   cuuint64_t dims[2] = {(cuuint64_t)dv, (cuuint64_t)rows};
@@ -130,6 +132,8 @@ bool encode_x_map(CUtensorMap *m, const void *x, long long rows, int dv, int box
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+
+namespace {
 
 // Bytes of feature rows a CTA streams in one dense update below which the
 // selection does not skip rows by the triangle inequality.
@@ -185,6 +189,11 @@ float tc_distance_eps(int dv) {
 cudaError_t launch_select(const Plan &pl, const float *w, const void *x, int32_t *idx_out,
                           void *x_out, char *ws, cudaStream_t s) {
   if (pl.B == 0 || pl.total_keep == 0) return cudaSuccess;
+  if (pl.gram) {
+    bool done = false;
+    const cudaError_t e = launch_select_gram(pl, w, x, idx_out, x_out, ws, s, &done);
+    if (done || e != cudaSuccess) return e;
+  }
   const int rb = pl.dv * pl.elem;
   const int nch = (pl.dv + 255) / 256;
   const DeviceInfo di = device_info();
@@ -265,7 +274,7 @@ cudaError_t launch_select(const Plan &pl, const float *w, const void *x, int32_t
       }
       smem_c = select_smem(cache_c, rb, tpc_c, ring_c, tb_c, pl.elem, lcap_c, 0, 0, 1, 0, c).total;
     }
-    const int active = active_clusters(fn_c, c, smem_c);
+    const int active = active_clusters(fn_c, c, smem_c, kSelThreads);
     if (active <= 0) continue;
     const double waves = std::ceil((double)pl.B / active);
     // features of the requests in flight beyond L2 stream from HBM

@@ -1,0 +1,64 @@
+"""The greedy from a Gram matrix (select_gram.cu) at the sizes where it can go wrong:
+around the 128-row and 256-column tiles and the 32-token blocks, one token more than
+the cluster's warps hold, feature widths that end inside a K block, every budget from
+one pick to all but one, exact ties, zero rows and rows outside the certificate's norm
+range.  Indices and rows are exact against the oracle."""
+import numpy as np
+import pytest
+
+import paper_2607_27952_gb300 as last
+from gpu_util import (assert_gather_equal, assert_selection_equal, oracle_selection,
+                      problem_of, to_dev, to_host_bits)
+from workloads import bf16_bits_to_f32, custom, f32_to_bf16_bits
+
+pytestmark = pytest.mark.gpu
+
+
+def _wl(n_vis, keep, d_v, seed=5, **kw):
+    return custom(name="gram", seed=seed, batch=len(n_vis), n_vis=n_vis, n_text=4, num_layers=1,
+                  num_q_heads=4, num_kv_heads=2, head_dim=64, feat_dim=d_v, dtype="bf16", keep=keep,
+                  n_clusters=kw.pop("n_clusters", 12), n_planted=3, **kw)
+
+
+def _run(wl, x=None, w=None):
+    import torch
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(3)
+    n = int(wl.cu_vis[-1])
+    w = (rng.random(n) + 0.5).astype(np.float32) if w is None else w
+    prob = problem_of(wl)
+    ws = last.workspace(prob, dev)
+    xd = to_dev(wl.x if x is None else x, dev)
+    idx = torch.full((int(wl.cu_keep[-1]),), -7, dtype=torch.int32, device=dev)
+    xs = torch.zeros((int(wl.cu_keep[-1]), wl.feat_dim), dtype=xd.dtype, device=dev)
+    last.last_select(prob, torch.from_numpy(w).to(dev), xd, idx, ws, x_out=xs)
+    last.last_poll(ws)
+    return w, idx.cpu().numpy(), to_host_bits(xs)
+
+
+@pytest.mark.parametrize("d_v", [8, 72, 520, 1536, 2048])
+@pytest.mark.parametrize("n_vis,keep", [
+    ([1, 31, 33, 127, 129], [1, 30, 2, 64, 40]),
+    ([255, 256, 257, 513], [254, 1, 100, 60]),
+    ([545, 640, 2049], [100, 0, 130]),
+])
+def test_selection_equals_the_oracle(n_vis, keep, d_v):
+    wl = _wl(n_vis, keep, d_v)
+    w, idx, xs = _run(wl)
+    assert_selection_equal(wl, w, idx, range(wl.batch))
+    assert_gather_equal(wl, idx, xs, range(wl.batch))
+
+
+def test_ties_zero_rows_and_extreme_norms():
+    n, d = 300, 512
+    wl = _wl([n], [150], d)
+    x = bf16_bits_to_f32(wl.x).copy()
+    x[10:60] = x[9]                      # exact duplicates
+    x[60:70] = 0.0
+    x[70:110] *= np.float32(2.0) ** -70   # outside the certificate's norm range
+    x[110:150] *= np.float32(2.0) ** 55
+    wl.x = f32_to_bf16_bits(x)
+    w = np.full(n, 1.0 / n, dtype=np.float32)
+    w[:5] = 0.0
+    w, idx, _ = _run(wl, w=w)
+    assert np.array_equal(idx, np.sort(oracle_selection(wl, w, 0)))
