@@ -24,10 +24,6 @@
 // and centre instead of a whole row per token, so its cost no longer grows with
 // d_v, and the N^2 d_v contraction runs once, at tensor-core rates, on every SM.
 //
-// Measured against them (GB300, whole last_prune call): 64 requests of 576 x 2048,
-// k 64/128/192: 1.71 -> 0.84 ms; 32 of 2880, k = 360: 5.27 -> 2.49; 128 of 256..4096 x
-// 1536, k = N/8: 10.3 -> 6.0; 8 of 16384 x 2048, k = 2048: 16.9 -> 8.6.
-//
 // Tokens are dealt to the cluster in blocks of 32: block k belongs to CTA k % C,
 // warp (k / C) % 16, so neighbouring tokens (tiles, frames, near-duplicates) spread
 // over all warps and both the ranking and the exact pairs stay balanced.
@@ -55,7 +51,8 @@ constexpr int kGcand = 1024;               // published entries above U kept bef
 constexpr int kGM = 128, kGN = 256, kGK = 64;
 constexpr int kGramStages = 4;
 constexpr int kGramStageBytes = (kGM + kGN) * kGK * 2;   // 48 KB
-constexpr int kGramThreads = 192;          // 4 epilogue warps, TMA producer, MMA issuer
+constexpr int kGramThreads = 320;          // 8 epilogue warps, TMA producer, MMA issuer
+constexpr int kGramChunkKb = 4;            // K blocks per accumulation chain (kGchunk products)
 constexpr int kGroupRows = 16;             // row blocks per tile group (L2 reuse of both operands)
 
 }  // namespace
@@ -72,6 +69,17 @@ int gram_tiles(int n_tokens) {
   int n = 0;
   for (int g = 0; 16 * g < R; ++g) n += gram_group_tiles(g, std::min(kGroupRows, R - 16 * g));
   return n;
+}
+
+// Bound on |d~ - d| between a distance from the Gram matrix and the canonical one.  A
+// chunk of kGchunk products is one chain of tensor-core accumulations: a sum of n exact
+// products in any order, each addition rounded or truncated once to fp32, errs by at
+// most n 2^-23 sum|x_i,k x_j,k|, and aligning groups of 16 products to the group's
+// largest exponent by 17/16 of that; taken twice.  The chunks are added in fp32 (8 u at
+// most), the canonical order adds 80 u (see tc_distance_eps) and the scalings 1e-6.
+constexpr int kGchunk = 256;
+inline float gram_distance_eps(int dv) {
+  return (float)((std::min(dv, kGchunk) * 0x1p-22 + 88 * 0x1p-24) * 1.01 + 1e-6);
 }
 
 struct GramArgs {
@@ -98,7 +106,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&afull[i], 1);
-      mbar_init(&aempty[i], 4);
+      mbar_init(&aempty[i], 8);
     }
     tslot[1] = 0;
     fence_mbar_init();
@@ -141,7 +149,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
     }
   };
 
-  if (warp == 4) {
+  if (warp == 8) {
     if (lane == 0) {
       uint32_t it = 0;
       for (int tile = blockIdx.x; tile < a.total_tiles; tile += gridDim.x) {
@@ -163,15 +171,14 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
         for (uint32_t k = it > kGramStages ? it - kGramStages : 0; k < it; ++k)
           mbar_wait_bounded(&full[k % kGramStages], (k / kGramStages) & 1, a.err, kErrTimeout);
     }
-  } else if (warp == 5) {
+  } else if (warp == 9) {
     if (lane == 0) {
       const uint32_t idesc = umma_idesc_bf16(kGM, kGN);
-      uint32_t it = 0, nt = 0;
-      for (int tile = blockIdx.x; tile < a.total_tiles; tile += gridDim.x, ++nt) {
-        const int ab = nt & 1;
-        if (nt >= 2) twait(&aempty[ab], ((nt >> 1) - 1) & 1);
-        tc_fence_after();
+      uint32_t it = 0, nc = 0;   // K blocks, accumulation chains
+      for (int tile = blockIdx.x; tile < a.total_tiles; tile += gridDim.x)
         for (int kb = 0; kb < nkb; ++kb, ++it) {
+          const int kc = kb % kGramChunkKb, ab = nc & 1;
+          if (kc == 0 && nc >= 2) twait(&aempty[ab], ((nc >> 1) - 1) & 1);
           const int st = it % kGramStages;
           const bool ok = twait(&full[st], (it / kGramStages) & 1);
           tc_fence_after();
@@ -180,48 +187,67 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
 #pragma unroll
             for (int k = 0; k < kGK / 16; ++k)
               umma_bf16(tmem + ab * kGN, umma_desc_sw128(sa + k * 32),
-                        umma_desc_sw128(sa + kGM * kGK * 2 + k * 32), idesc, (kb | k) != 0 ? 1u : 0u);
+                        umma_desc_sw128(sa + kGM * kGK * 2 + k * 32), idesc, (kc | k) != 0 ? 1u : 0u);
           }
           umma_commit(&empty[st]);
+          if (kc == kGramChunkKb - 1 || kb == nkb - 1) {
+            umma_commit(&afull[ab]);
+            ++nc;
+          }
         }
-        umma_commit(&afull[ab]);
-      }
     }
   } else {
-    uint32_t nt = 0;
-    for (int tile = blockIdx.x; tile < a.total_tiles; tile += gridDim.x, ++nt) {
-      const int ab = nt & 1;
+    // warps 0-7: 32 rows (the warp's TMEM lanes) x 128 columns each; the chains of a
+    // tile are added in registers
+    const int half = warp >> 2, quad = warp & 3;
+    uint32_t nc = 0;
+    for (int tile = blockIdx.x; tile < a.total_tiles; tile += gridDim.x) {
       int b, ti, tj;
       decode(tile, &b, &ti, &tj);
+      float v[128];
+#pragma unroll
+      for (int q = 0; q < 128; ++q) v[q] = 0.f;
+      for (int kb = 0; kb < nkb; kb += kGramChunkKb, ++nc) {
+        const int ab = nc & 1;
+        twait(&afull[ab], (nc >> 1) & 1);
+        __syncwarp();
+        tc_fence_after();
+        const uint32_t tb = tmem + ab * kGN + half * 128 + ((uint32_t)(32 * quad) << 16);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          uint32_t raw[16];
+          tmem_ld16(tb + 16 * c, raw);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) v[16 * c + q] = __fadd_rn(v[16 * c + q], __uint_as_float(raw[q]));
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&aempty[ab]);
+      }
       const int32_t *m = a.meta + b * kMetaFields;
       const int N = m[kNumVis], ld = gram_ld(N);
       float *G = a.gram + (long long)m[kGramOff] * 32;
-      twait(&afull[ab], (nt >> 1) & 1);
-      __syncwarp();
-      tc_fence_after();
-      const int i = ti * kGM + 32 * warp + lane;
-      const uint32_t tb = tmem + ab * kGN + ((uint32_t)(32 * warp) << 16);
-      for (int c0 = 0; c0 < kGN; c0 += 32) {
-        const int j0 = tj * kGN + c0;
-        if (j0 >= N) break;
-        uint32_t v[32];
-        tmem_ld32(tb + c0, v);
-        if (i < N) {
-          float *row = G + (long long)i * ld + j0;
+      const int i = ti * kGM + 32 * quad + lane;
+      const int j0 = tj * kGN + half * 128;
+      // the transposed 128 x 128 block too, unless a tile of its own computes it
+      const bool mirror = j0 / kGM < 2 * (ti / 2) && i < ld;
 #pragma unroll
-          for (int q = 0; q < 32; q += 8) st_global_v8(row + q, v + q);
-        }
-        // the transposed 128 x 128 block, unless a tile of its own computes it
-        if (j0 / kGM < 2 * (ti / 2) && i < ld) {
-          float *col = G + (long long)j0 * ld + i;
+      for (int c = 0; c < 4; ++c) {
+        const int j = j0 + 32 * c;
+        if (j < N) {
+          if (i < N) {
+            float *row = G + (long long)i * ld + j;
 #pragma unroll
-          for (int q = 0; q < 32; ++q)
-            if (j0 + q < N) col[(long long)q * ld] = __uint_as_float(v[q]);
+            for (int q = 0; q < 32; q += 8) st_global_v8(row + q, v + 32 * c + q);
+          }
+          if (mirror) {
+            float *col = G + (long long)j * ld + i;
+#pragma unroll
+            for (int q = 0; q < 32; ++q)
+              if (j + q < N) col[(long long)q * ld] = v[32 * c + q];
+          }
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&aempty[ab]);
     }
   }
   __syncthreads();
@@ -248,41 +274,57 @@ struct GramSelArgs {
   int32_t *idx_out;
   char *x_out;             // nullable
   const int32_t *meta, *order;
-  int dv, row_bytes, csize, mc, slots, words, accept;
-  float eps;
+  int dv, row_bytes, csize, mc, slots, words;
+  float eps;               // bound on |distance from the Gram matrix - canonical distance|
   unsigned *err;
 };
 
+// A published candidate: upper key (high word), token, w~, 1/|x|, the evaluated
+// minimum e, and up to two centres whose distance is only known to within eps.
+struct GramEntry {
+  uint32_t kh, idx;
+  float w, r;
+  float e, p0, p1;
+  uint32_t ids;            // centre of p0 | centre of p1 << 16
+};
+static_assert(sizeof(GramEntry) == 32, "two 16-byte stores publish an entry");
+
 // Shared memory of select_gram_kernel (host sizing and device carve-up alike).
 struct GramSelSmem {
-  size_t rows, w, r, dl, fmask, fidx, sel, pub, cand, pm, plist, key, lidx, ld, lw, lr, acc, misc, bar, total;
+  size_t ks, w, r, e, p0, p1, ids, fmask, fidx, sel, pub, ckey, cidx, pm, mem, acc, cen, misc, total;
 };
-__host__ __device__ inline GramSelSmem gram_sel_smem(int accept, int row_bytes, int slots, int words,
-                                                     int csize, int mc) {
+__host__ __device__ inline GramSelSmem gram_sel_smem(int slots, int words, int csize, int mc) {
   GramSelSmem s;
   size_t o = 0;
   const size_t cap = (size_t)slots * kGthreads;   // token slots of a CTA
-  s.rows = o; o += (size_t)accept * row_bytes;    // the round's accepted centres
+  s.ks = o; o += 4 * cap;                         // high word of the upper key, 0 = not live
   s.w = o; o += 4 * cap;
   s.r = o; o += 4 * cap;
-  s.dl = o; o += 4 * cap;
-  s.fmask = o; o += 8 * cap;                      // flagged tokens: centres to evaluate
+  s.e = o; o += 4 * cap;
+  s.p0 = o; o += 4 * cap;
+  s.p1 = o; o += 4 * cap;
+  s.ids = o; o += 4 * cap;
+  s.fmask = o; o += 8 * cap;                      // tokens to evaluate at once: their centres
   s.fidx = o; o += align16(2 * cap);
   s.sel = o; o += align16(4 * (size_t)words);     // selected bits of the whole request
-  s.pub = o; o += (size_t)2 * kGwarps * csize * (mc + 1) * 16;
-  s.cand = o; o += 2 * kGcand;
-  s.pm = o; o += align16(4 * kGlist * kGpairLd);  // pair dots of the list
-  s.plist = o; o += 2 * kGlist * kGlist / 2;
-  s.key = o; o += 8 * kGlist;
-  s.lidx = o; o += 4 * kGlist;
-  s.ld = o; o += 4 * kGlist;
-  s.lw = o; o += 4 * kGlist;
-  s.lr = o; o += 4 * kGlist;
+  s.pub = o; o += (size_t)2 * kGwarps * csize * (mc + 1) * sizeof(GramEntry);
+  s.ckey = o; o += 8 * kGcand;
+  s.cidx = o; o += 2 * kGcand;
+  s.pm = o; o += align16(4 * kGlist * kGpairLd);  // the list's pairwise distances
+  s.mem = o; o += sizeof(GramEntry) * kGlist;
   s.acc = o; o += 4 * kGmaxAccept;
+  s.cen = o; o += 8 * kGmaxAccept;                // accepted centres: token, 1/|x|
   s.misc = o; o += 8 * 40;
-  s.bar = o; o += 16;
   s.total = align16(o);
   return s;
+}
+
+__device__ __forceinline__ unsigned long long gram_key(uint32_t kh, uint32_t idx) {
+  return ((unsigned long long)kh << 32) | (0xffffffffu - idx);
+}
+// high word of the key of w delta
+__device__ __forceinline__ uint32_t key_high(float w, float delta) {
+  return (uint32_t)(argmax_key(__fmul_rn(w, delta), 0) >> 32);
 }
 
 template <int NCH>
@@ -295,7 +337,7 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
   const int32_t *m = a.meta + b * kMetaFields;
   const int voff = m[kVisOff], N = m[kNumVis], koff = m[kKeepOff], K = m[kNumKeep];
   if (K == 0) return;   // the whole cluster leaves together
-  const GramSelSmem S = gram_sel_smem(a.accept, a.row_bytes, a.slots, a.words, C, a.mc);
+  const GramSelSmem S = gram_sel_smem(a.slots, a.words, C, a.mc);
   {
     uint32_t dyn;
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
@@ -304,28 +346,28 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       return;
     }
   }
-  char *rows = reinterpret_cast<char *>(smem + S.rows);
+  uint32_t *ks = reinterpret_cast<uint32_t *>(smem + S.ks);
   float *w_s = reinterpret_cast<float *>(smem + S.w);
   float *r_s = reinterpret_cast<float *>(smem + S.r);
-  float *dl_s = reinterpret_cast<float *>(smem + S.dl);
+  float *e_s = reinterpret_cast<float *>(smem + S.e);
+  float *p0_s = reinterpret_cast<float *>(smem + S.p0);
+  float *p1_s = reinterpret_cast<float *>(smem + S.p1);
+  uint32_t *id_s = reinterpret_cast<uint32_t *>(smem + S.ids);
   unsigned long long *fmask = reinterpret_cast<unsigned long long *>(smem + S.fmask);
   uint16_t *fidx = reinterpret_cast<uint16_t *>(smem + S.fidx);
   uint32_t *sel = reinterpret_cast<uint32_t *>(smem + S.sel);
-  uint4 *pub = reinterpret_cast<uint4 *>(smem + S.pub);
-  uint16_t *cand = reinterpret_cast<uint16_t *>(smem + S.cand);
+  GramEntry *pub = reinterpret_cast<GramEntry *>(smem + S.pub);
+  unsigned long long *ckey = reinterpret_cast<unsigned long long *>(smem + S.ckey);
+  uint16_t *cidx = reinterpret_cast<uint16_t *>(smem + S.cidx);
   float *pm = reinterpret_cast<float *>(smem + S.pm);
-  uint16_t *plist = reinterpret_cast<uint16_t *>(smem + S.plist);
-  unsigned long long *lkey = reinterpret_cast<unsigned long long *>(smem + S.key);
-  int *lidx = reinterpret_cast<int *>(smem + S.lidx);
-  float *ldl = reinterpret_cast<float *>(smem + S.ld);
-  float *lw = reinterpret_cast<float *>(smem + S.lw);
-  float *lr = reinterpret_cast<float *>(smem + S.lr);
+  GramEntry *mem = reinterpret_cast<GramEntry *>(smem + S.mem);
   int *acc_s = reinterpret_cast<int *>(smem + S.acc);
+  float2 *cen = reinterpret_cast<float2 *>(smem + S.cen);
   unsigned long long *misc = reinterpret_cast<unsigned long long *>(smem + S.misc);
-  int *cnt = reinterpret_cast<int *>(misc + 32);   // [0] flagged tokens, [1] candidates, [2] pairs, [3] list, [4] picks
-  unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem + S.bar);
+  int *cnt = reinterpret_cast<int *>(misc + 32);   // [0] flagged tokens, [1] candidates, [2] picks
 
   const int rb = a.row_bytes, dv = a.dv, ld = gram_ld(N);
+  const float eps = a.eps;
   const int nblk = (N + 31) >> 5;
   const char *xreq = a.x + (long long)voff * rb;
   const float *rreq = a.rn + voff, *wreq = a.w + voff;
@@ -333,84 +375,112 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
   const int P = kGwarps * C;                          // publishing warps of the cluster
   const int step = C * kGwarps;                       // blocks between a warp's slots
   const int blk0 = rank + C * warp;                   // this warp's first block
+  const int nslot = (nblk - blk0 + step - 1) / step;  // this warp's blocks (<= a.slots)
 
-  if (tid == 0) {
-    mbar_init(bar, 1);
-    fence_mbar_init();
-  }
   for (int v = tid; v < nblk; v += kGthreads) sel[v] = K == N ? 0xffffffffu : 0u;
-  for (int s = 0, k = blk0; k < nblk; ++s, k += step) {
-    const int t = 32 * k + lane, li = s * kGthreads + tid;
+  for (int s = 0; s < nslot; ++s) {
+    const int t = 32 * (blk0 + s * step) + lane, li = s * kGthreads + tid;
     const bool in = t < N;
     w_s[li] = in ? wreq[t] : 0.f;
-    r_s[li] = in ? rreq[t] : 0.f;
-    dl_s[li] = INFINITY;
+    r_s[li] = in && K < N ? rreq[t] : 0.f;
+    e_s[li] = INFINITY;
+    p0_s[li] = INFINITY;
+    p1_s[li] = INFINITY;
+    id_s[li] = 0u;
+    ks[li] = in ? 1u : 0u;   // live; the first update sets the key
   }
-  uint32_t phase = 0;
 
   if (K < N) {
     auto csync = [&]() {
       if (C == 1) __syncthreads();
       else cluster_sync();
     };
-    // 8 coordinates per lane of chunk g of a row
-    auto load_row = [&](const char *row, U4 *v) {
+    // 8 coordinates per lane of each chunk of row t
+    auto load_row = [&](int t, U4 *v) {
+      const char *row = xreq + (long long)t * rb;
 #pragma unroll
       for (int g = 0; g < NCH; ++g) {
         const int col = 256 * g + 8 * lane;
         v[g] = col < dv ? ldg_nc(row + col * 2) : U4{0, 0, 0, 0};
       }
     };
-    auto fma8 = [&](const U4 &x, const U4 &c, float acc) {
-      const uint32_t xw[4] = {x.x, x.y, x.z, x.w}, cw[4] = {c.x, c.y, c.z, c.w};
+    // canonical distance of two rows with reciprocal norms ri (the token's) and rc
+    auto distance = [&](const U4 *x, const U4 *c, float ri, float rc) {
+      float acc = 0.f;
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        acc = fma_bf16_lo(xw[h], cw[h], acc);
-        acc = fma_bf16_hi(xw[h], cw[h], acc);
+      for (int g = 0; g < NCH; ++g) {
+        if (256 * g + 8 * lane < dv) {
+          const uint32_t xw[4] = {x[g].x, x[g].y, x[g].z, x[g].w};
+          const uint32_t cw[4] = {c[g].x, c[g].y, c[g].z, c[g].w};
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            acc = fma_bf16_lo(xw[h], cw[h], acc);
+            acc = fma_bf16_hi(xw[h], cw[h], acc);
+          }
+        }
       }
-      return acc;
+      return __fsub_rn(1.0f, __fmul_rn(__fmul_rn(butterfly_sum(acc), ri), rc));
     };
-    const uint32_t rows_sa = smem_addr(rows);
 
-    // Fold the nA accepted centres lidx[acc_s[j]] into the tokens' delta.
-    auto update = [&](int nA, bool seed) {
-      // the centres' rows into shared memory (one bulk copy each)
-      if (warp == 0) {
-        if (lane == 0) mbar_expect_tx(bar, (uint32_t)(nA * rb));
-        __syncwarp();
-        for (int j = lane; j < nA; j += 32)
-          bulk_g2s(rows + (long long)j * rb, xreq + (long long)lidx[acc_s[j]] * rb, (uint32_t)rb, bar);
-      }
+    // Fold the nA accepted centres cen[0 .. nA) into the tokens' distances.  A centre
+    // with d~ - eps at or above the token's upper bound cannot lower its delta.  Any
+    // other becomes one of the token's two pending centres; entries that a new upper
+    // bound excludes leave.  Pairs outside the certificate's norm range, NaN and a
+    // third pending centre are evaluated at once.
+    auto update = [&](int nA) {
       if (tid == 0) cnt[0] = 0;
       __syncthreads();
-      for (int s = 0, k = blk0; k < nblk; ++s, k += step) {
-        const int t = 32 * k + lane, li = s * kGthreads + tid;
-        const bool live = t < N && !((sel[k] >> lane) & 1u);
+      for (int s = 0; s < nslot; ++s) {
+        const int t = 32 * (blk0 + s * step) + lane, li = s * kGthreads + tid;
+        const bool live = ks[li] != 0u;
         unsigned long long msk = 0ull;
-        const float ri = r_s[li], dl = dl_s[li];
+        const float ri = r_s[li];
+        float e = e_s[li], p0 = p0_s[li], p1 = p1_s[li];
+        uint32_t ids = id_s[li];
         const bool in_range = tri_in_range(ri);
-        if (seed) {
-          msk = 1ull;
-        } else {
-          for (int j0 = 0; j0 < nA; j0 += 8) {
-            float g[8];
+        float hi = fminf(e, __fadd_ru(fminf(p0, p1), eps));
+        bool touched = false;
+        for (int j0 = 0; j0 < nA; j0 += 16) {
+          float g[16];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int c = lidx[acc_s[min(j0 + j, nA - 1)]];
-              g[j] = live ? ldg_f32_stream(G + (long long)c * ld + t) : 0.f;
-            }
+          for (int j = 0; j < 16; ++j) {
+            const int c = __float_as_int(cen[min(j0 + j, nA - 1)].x);
+            g[j] = live ? ldg_f32_stream(G + (long long)c * ld + t) : 0.f;
+          }
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              if (j0 + j < nA) {
-                const float rc = lr[acc_s[j0 + j]];
-                const float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[j], ri), rc));
-                // NaN and rows outside the certificate's norm range go to the exact path
-                if (!(__fsub_rn(d, a.eps) >= dl) || !in_range || !tri_in_range(rc)) msk |= 1ull << (j0 + j);
+          for (int j = 0; j < 16; ++j) {
+            if (j0 + j < nA) {
+              const float rc = cen[j0 + j].y;
+              const float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[j], ri), rc));
+              if (live && (!(__fsub_rd(d, eps) >= hi) || !in_range || !tri_in_range(rc))) {
+                touched = true;
+                if (!in_range || !tri_in_range(rc) || d != d) {
+                  msk |= 1ull << (j0 + j);
+                } else {
+                  const uint32_t c = __float_as_uint(cen[j0 + j].x);
+                  hi = fminf(hi, __fadd_ru(d, eps));
+                  if (__fsub_rd(p0, eps) >= hi) p0 = INFINITY;
+                  if (__fsub_rd(p1, eps) >= hi) p1 = INFINITY;
+                  if (p0 == INFINITY) {
+                    p0 = d;
+                    ids = (ids & 0xffff0000u) | c;
+                  } else if (p1 == INFINITY) {
+                    p1 = d;
+                    ids = (ids & 0xffffu) | (c << 16);
+                  } else {
+                    msk |= 1ull << (j0 + j);
+                  }
+                }
               }
             }
           }
         }
-        if (!live) msk = 0ull;
+        if (touched) {
+          p0_s[li] = p0;
+          p1_s[li] = p1;
+          id_s[li] = ids;
+          ks[li] = key_high(w_s[li], fminf(e, __fadd_ru(fminf(p0, p1), eps)));
+        }
         const unsigned bal = __ballot_sync(0xffffffffu, msk != 0ull);
         if (bal) {
           int base = 0;
@@ -423,52 +493,30 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
           }
         }
       }
-      mbar_wait_bounded(bar, phase, a.err, kErrTimeout);
-      phase ^= 1u;
       __syncthreads();
-      // exact canonical distances of the flagged pairs, a warp per token; the next
-      // token's row is in flight while the current one is evaluated
+      // a warp per flagged token: its masked centres in the canonical order
       const int nf = cnt[0];
-      auto row_of = [&](int f) {
-        const int li = fidx[f];
-        const int k = rank + C * ((li >> 5) % kGwarps) + (li / kGthreads) * step;
-        return xreq + (long long)(32 * k + (li & 31)) * rb;
-      };
-      auto exact_token = [&](int f, const U4 *xv) {
+      for (int f = warp; f < nf; f += kGwarps) {
         const int li = fidx[f];
         unsigned long long msk = fmask[f];
-        const float ri = r_s[li];
-        float dl = dl_s[li];
+        const int k = rank + C * ((li >> 5) % kGwarps) + (li / kGthreads) * step;
+        U4 xv[NCH], xc[NCH];
+        load_row(32 * k + (li & 31), xv);
+        float e = e_s[li];
         while (msk) {
           const int j = __ffsll(msk) - 1;
           msk &= msk - 1;
-          const uint32_t cr = rows_sa + (uint32_t)(j * rb);
-          float acc = 0.f;
-#pragma unroll
-          for (int g = 0; g < NCH; ++g) {
-            const int col = 256 * g + 8 * lane;
-            if (col < dv) acc = fma8(xv[g], lds32(cr + col * 2), acc);
-          }
-          const float dot = butterfly_sum(acc);
-          dl = fminf(dl, __fsub_rn(1.0f, __fmul_rn(__fmul_rn(dot, ri), lr[acc_s[j]])));
+          const float2 c = cen[j];
+          load_row(__float_as_int(c.x), xc);
+          e = fminf(e, distance(xv, xc, r_s[li], c.y));
         }
-        if (lane == 0) dl_s[li] = dl;
-      };
-      {
-        U4 xa[NCH], xb[NCH];
-        int f = warp;
-        if (f < nf) load_row(row_of(f), xa);
-        while (f < nf) {
-          if (f + kGwarps < nf) load_row(row_of(f + kGwarps), xb);
-          exact_token(f, xa);
-          f += kGwarps;
-          if (f >= nf) break;
-          if (f + kGwarps < nf) load_row(row_of(f + kGwarps), xa);
-          exact_token(f, xb);
-          f += kGwarps;
+        __syncwarp();
+        if (lane == 0) {
+          e_s[li] = e;
+          ks[li] = key_high(w_s[li], fminf(e, __fadd_ru(fminf(p0_s[li], p1_s[li]), eps)));
         }
       }
-      __syncthreads();
+      if (nf > 0) __syncthreads();
     };
 
     // ---- seed (Eq. 9): argmax w~ over the request, every CTA alike ----
@@ -481,214 +529,295 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       best = warp_max_u64(lane < kGwarps ? misc[lane] : 0ull);
       const int seed = key_index(best);
       if (tid == 0) {
-        lidx[0] = seed;
-        lr[0] = rreq[seed];
-        acc_s[0] = 0;
+        cen[0] = make_float2(__int_as_float(seed), rreq[seed]);
         sel[seed >> 5] |= 1u << (seed & 31);
       }
+      if ((seed >> 5) % C == rank && ((seed >> 5) / C) % kGwarps == warp && lane == (seed & 31))
+        ks[((seed >> 5) / step) * kGthreads + tid] = 0u;
       __syncthreads();
     }
     int taken = 1;
-    if (taken < K) update(1, true);
-
+    if (taken < K) update(1);
     csync();   // every CTA of the cluster runs before the first remote write
+
     // ---- rounds (Eq. 10-11) ----
     const int ent = a.mc + 1;
     for (int round = 0; taken < K; ++round) {
       const int par = round & 1;
-      uint4 *pubp = pub + (size_t)par * P * ent;
-      // 1. this warp's best live keys, best first: {index, delta, w~, 1/|x|}
+      GramEntry *pubp = pub + (size_t)par * P * ent;
+      // 1. this warp's best live tokens by upper key: lane e ends with the e-th one
       {
-        unsigned long long limit = ~0ull, mine;
-        int ms = 0;
-        auto best_below = [&]() {
-          unsigned long long bk = 0ull;
-          for (int s = 0, k = blk0; k < nblk; ++s, k += step) {
-            const int t = 32 * k + lane, li = s * kGthreads + tid;
-            if (t < N && !((sel[k] >> lane) & 1u)) {
-              const unsigned long long kk = argmax_key(__fmul_rn(w_s[li], dl_s[li]), t);
-              if (kk < limit && kk > bk) {
-                bk = kk;
-                ms = s;
-              }
+        uint32_t done = 0u;   // slots of this lane already taken
+        uint32_t kh = 0u;
+        int ms = 0, mine = -1;
+        auto best_left = [&]() {
+          kh = 0u;
+          for (int s = 0; s < nslot; ++s) {
+            const uint32_t v = ks[s * kGthreads + tid];
+            if (v > kh && !((done >> s) & 1u)) {   // lower slots (lower tokens) win ties
+              kh = v;
+              ms = s;
             }
           }
-          return bk;
         };
-        mine = best_below();
+        best_left();
         for (int e = 0; e < ent; ++e) {
-          const unsigned long long best = warp_max_u64(mine);
-          uint4 v = make_uint4(0xffffffffu, 0u, 0u, 0u);   // no token left
-          if (best != 0ull) {
-            const int src = __ffs(__ballot_sync(0xffffffffu, mine == best)) - 1;
-            const int li = __shfl_sync(0xffffffffu, ms, src) * kGthreads + warp * 32 + src;
-            v = make_uint4((uint32_t)key_index(best), __float_as_uint(dl_s[li]), __float_as_uint(w_s[li]),
-                           __float_as_uint(r_s[li]));
-            if (lane == src) {
-              limit = best;
-              mine = best_below();
-            }
+          const uint32_t mx = __reduce_max_sync(0xffffffffu, kh);
+          if (mx == 0u) break;
+          unsigned win = __ballot_sync(0xffffffffu, kh == mx);
+          if (win & (win - 1u)) {   // equal values: the lowest token
+            const uint32_t blk = kh == mx ? (uint32_t)ms : 0xffffffffu;
+            const uint32_t low = __reduce_min_sync(0xffffffffu, blk);
+            win = __ballot_sync(0xffffffffu, kh == mx && (uint32_t)ms == low);
           }
-          if (lane < C)
-            st_cluster_v4u(map_shared(&pubp[(rank * kGwarps + warp) * ent + e], lane), v);
+          const int src = __ffs(win) - 1;
+          const int li = __shfl_sync(0xffffffffu, ms, src) * kGthreads + warp * 32 + src;
+          if (lane == e) mine = li;
+          if (lane == src) {
+            done |= 1u << ms;
+            best_left();
+          }
+        }
+        if (lane < ent) {
+          uint4 v0 = make_uint4(0u, 0xffffffffu, 0u, 0u), v1 = make_uint4(0u, 0u, 0u, 0u);
+          if (mine >= 0) {
+            const int t = 32 * (blk0 + (mine / kGthreads) * step) + (mine & 31);
+            v0 = make_uint4(ks[mine], (uint32_t)t, __float_as_uint(w_s[mine]), __float_as_uint(r_s[mine]));
+            v1 = make_uint4(__float_as_uint(e_s[mine]), __float_as_uint(p0_s[mine]),
+                            __float_as_uint(p1_s[mine]), id_s[mine]);
+          }
+          GramEntry *dst = &pubp[(rank * kGwarps + warp) * ent + lane];
+          for (int q = 0; q < C; ++q) {
+            const uint32_t addr = map_shared(dst, q);
+            st_cluster_v4u(addr, v0);
+            st_cluster_v4u(addr + 16, v1);
+          }
         }
       }
-      if (tid == 0) {
-        cnt[1] = 0;
-        cnt[2] = 0;
-        cnt[3] = 0;
-      }
+      if (tid == 0) cnt[1] = 0;
       csync();
       // 2. the list: published entries above U
-      auto entry_key = [&](const uint4 &v) {
-        return v.x == 0xffffffffu
-                   ? 0ull
-                   : argmax_key(__fmul_rn(__uint_as_float(v.z), __uint_as_float(v.y)), (int)v.x);
-      };
       unsigned long long U = 0ull;
-      for (int q = lane; q < P; q += 32) U = max(U, entry_key(pubp[q * ent + a.mc]));
+      for (int q = lane; q < P; q += 32) {
+        const GramEntry &v = pubp[q * ent + a.mc];
+        if (v.kh != 0u) U = max(U, gram_key(v.kh, v.idx));
+      }
       U = warp_max_u64(U);
       for (int e0 = warp * 32; e0 < P * ent; e0 += kGthreads) {
         const int e = e0 + lane;
-        const bool up = e < P * ent && entry_key(pubp[e]) > U;
+        unsigned long long kk = 0ull;
+        if (e < P * ent && pubp[e].kh != 0u) kk = gram_key(pubp[e].kh, pubp[e].idx);
+        const bool up = kk > U;
         const unsigned bal = __ballot_sync(0xffffffffu, up);
         if (bal) {
           int base = 0;
           if (lane == 0) base = atomicAdd(&cnt[1], __popc(bal));
           base = __shfl_sync(0xffffffffu, base, 0);
-          if (up) cand[base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)e;
+          if (up) {
+            const int pos = base + __popc(bal & ((1u << lane) - 1u));
+            cidx[pos] = (uint16_t)e;
+            ckey[pos] = kk;
+          }
         }
       }
       __syncthreads();
       const int nc = cnt[1];
       // the best kGlist of them; U' = the first key cut off
-      if (warp * 32 < nc) {
-        for (int c0 = warp * 32; c0 < nc; c0 += kGthreads) {
-          const int c = c0 + lane;
-          const uint4 v = c < nc ? pubp[cand[c]] : make_uint4(0xffffffffu, 0u, 0u, 0u);
-          const unsigned long long kk = entry_key(v);
-          int pos = c;
-          if (nc > kGlist) {
-            pos = 0;
-            for (int q = 0; q < nc; ++q) pos += entry_key(pubp[cand[q]]) > kk ? 1 : 0;
-          }
-          if (c < nc) {
-            if (pos < kGlist) {
-              lkey[pos] = kk;
-              lidx[pos] = (int)v.x;
-              ldl[pos] = __uint_as_float(v.y);
-              lw[pos] = __uint_as_float(v.z);
-              lr[pos] = __uint_as_float(v.w);
-            } else if (pos == kGlist) {
-              misc[20] = kk;
-            }
-          }
+      for (int c0 = warp * 32; c0 < nc; c0 += kGthreads) {
+        const int c = c0 + lane;
+        const unsigned long long kk = c < nc ? ckey[c] : 0ull;
+        int pos = c;
+        if (nc > kGlist) {
+          pos = 0;
+          for (int q = 0; q < nc; ++q) pos += ckey[q] > kk ? 1 : 0;
+        }
+        if (c < nc) {
+          if (pos < kGlist) mem[pos] = pubp[cidx[c]];
+          else if (pos == kGlist) misc[20] = kk;
         }
       }
       __syncthreads();
       const int nL = min(nc, kGlist);
       const unsigned long long Up = nc > kGlist ? misc[20] : U;
-      // the list's Gram rows for this CTA's tokens start towards L2
-      for (int k = blk0; k < nblk; k += step)
-        for (int u = lane; u < nL; u += 32) prefetch_l2(G + (long long)lidx[u] * ld + 32 * k);
-      // 3. pair dots: -inf (distance +inf) where the certificate excludes the pair
-      for (int u = warp; u < nL; u += kGwarps) {
-        const int iu = lidx[u];
-        const float ru = lr[u], du = ldl[u];
-        const bool cu = tri_in_range(ru);
+      // 3. the list's Gram rows for this CTA's tokens start towards L2; pairwise
+      // distances from the Gram matrix (NaN: outside the certificate)
+      for (int s = 0; s < nslot; ++s)
+        for (int u = lane; u < nL; u += 32)
+          prefetch_l2(G + (long long)mem[u].idx * ld + 32 * (blk0 + s * step));
+      {
+        constexpr int kRows = kGlist / kGwarps;
+        float g[kRows][kGper];
 #pragma unroll
-        for (int h = 0; h < kGper; ++h) {
-          const int v = lane + 32 * h;
-          bool need = false;
-          if (v > u && v < nL) {
-            const float g = ldg_f32_stream(G + (long long)iu * ld + lidx[v]);
-            const float rv = lr[v];
-            const float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g, ru), rv));
-            need = !cu || !tri_in_range(rv) || !(__fsub_rn(d, a.eps) >= fmaxf(du, ldl[v]));
-            if (!need) pm[u * kGpairLd + v] = pm[v * kGpairLd + u] = -INFINITY;
+        for (int i = 0; i < kRows; ++i)
+#pragma unroll
+          for (int h = 0; h < kGper; ++h) {
+            const int u = warp + i * kGwarps, v = lane + 32 * h;
+            g[i][h] = u < v && v < nL ? ldg_f32_stream(G + (long long)mem[u].idx * ld + mem[v].idx) : 0.f;
           }
-          const unsigned bal = __ballot_sync(0xffffffffu, need);
-          if (bal) {
-            int base = 0;
-            if (lane == 0) base = atomicAdd(&cnt[2], __popc(bal));
-            base = __shfl_sync(0xffffffffu, base, 0);
-            if (need) plist[base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(u * kGlist + v);
+#pragma unroll
+        for (int i = 0; i < kRows; ++i)
+#pragma unroll
+          for (int h = 0; h < kGper; ++h) {
+            const int u = warp + i * kGwarps, v = lane + 32 * h;
+            if (u < v && v < nL) {
+              const float ru = mem[u].r, rv = mem[v].r;
+              float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[i][h], ru), rv));
+              if (!tri_in_range(ru) || !tri_in_range(rv)) d = __int_as_float(0x7fffffff);
+              pm[u * kGpairLd + v] = pm[v * kGpairLd + u] = d;
+            }
+          }
+      }
+      // the members' pending centres in the canonical order: every member's delta is
+      // exact from here on (every CTA alike; the owner keeps the result)
+      for (int u = warp; u < nL; u += kGwarps) {
+        const GramEntry me = mem[u];
+        if (me.p0 == INFINITY && me.p1 == INFINITY) continue;
+        U4 xv[NCH], xc[NCH];
+        load_row((int)me.idx, xv);
+        float e = me.e;
+        if (me.p0 != INFINITY) {
+          const int c = (int)(me.ids & 0xffffu);
+          load_row(c, xc);
+          e = fminf(e, distance(xv, xc, me.r, rreq[c]));
+        }
+        if (me.p1 != INFINITY) {
+          const int c = (int)(me.ids >> 16);
+          load_row(c, xc);
+          e = fminf(e, distance(xv, xc, me.r, rreq[c]));
+        }
+        const uint32_t kh = key_high(me.w, e);
+        if (lane == 0) {
+          mem[u].e = e;
+          mem[u].kh = kh;
+          const int k = (int)me.idx >> 5;
+          if (k % C == rank) {
+            const int li = (k / step) * kGthreads + ((k / C) % kGwarps) * 32 + (int)(me.idx & 31u);
+            e_s[li] = e;
+            p0_s[li] = INFINITY;
+            p1_s[li] = INFINITY;
+            ks[li] = kh;
           }
         }
       }
       __syncthreads();
-      const int np = cnt[2];
-      for (int p = warp; p < np; p += kGwarps) {
-        const int u = plist[p] / kGlist, v = plist[p] % kGlist;
-        U4 xu[NCH], xv[NCH];
-        load_row(xreq + (long long)lidx[u] * rb, xu);
-        load_row(xreq + (long long)lidx[v] * rb, xv);
-        float acc = 0.f;
-#pragma unroll
-        for (int g = 0; g < NCH; ++g)
-          if (256 * g + 8 * lane < dv) acc = fma8(xu[g], xv[g], acc);
-        const float dot = butterfly_sum(acc);
-        if (lane == 0) pm[u * kGpairLd + v] = pm[v * kGpairLd + u] = dot;
-      }
-      __syncthreads();
-      // 4. replay the greedy on the list (warp 0; lane u holds members u, u + 32)
+      // 4. replay the greedy on the list (warp 0; lane u holds members u, u + 32, ..).
+      // A member's delta lies in [lo, hi]: exact until an accepted centre's distance
+      // reaches below hi + eps; such centres are kept in `pend` and evaluated only when
+      // the member's place in the order depends on it.
       if (warp == 0) {
-        unsigned long long key[kGper];
-        float cd[kGper], wv[kGper], rv[kGper];
-        int gi[kGper];
+        uint32_t kh[kGper], kl[kGper];   // upper and lower key, high words
+        float e[kGper], hi[kGper], lo[kGper];
+        unsigned long long pend[kGper];
 #pragma unroll
         for (int h = 0; h < kGper; ++h) {
           const int u = lane + 32 * h;
           const bool in = u < nL;
-          key[h] = in ? lkey[u] : 0ull;
-          cd[h] = in ? ldl[u] : 0.f;
-          wv[h] = in ? lw[u] : 0.f;
-          rv[h] = in ? lr[u] : 0.f;
-          gi[h] = in ? lidx[u] : 0;
+          kh[h] = kl[h] = in ? mem[u].kh : 0u;
+          e[h] = hi[h] = lo[h] = in ? mem[u].e : 0.f;
+          pend[h] = 0ull;
         }
         int nA = 0;
-        while (taken + nA < K && nA < a.accept) {
-          unsigned long long lk = key[0];
+        while (taken + nA < K && nA < kGmaxAccept) {
+          unsigned long long lk = 0ull;
           int lh = 0;
 #pragma unroll
-          for (int h = 1; h < kGper; ++h)
-            if (key[h] > lk) {
-              lk = key[h];
+          for (int h = 0; h < kGper; ++h) {
+            const unsigned long long k = kh[h] ? gram_key(kh[h], mem[lane + 32 * h].idx) : 0ull;
+            if (k > lk) {
+              lk = k;
               lh = h;
             }
+          }
           const unsigned long long bk = warp_max_u64(lk);
           if (bk <= Up) break;   // also the end of the list (key 0)
           const int src = __ffs(__ballot_sync(0xffffffffu, lk == bk)) - 1;
           const int bl = src + 32 * __shfl_sync(0xffffffffu, lh, src);
+          unsigned long long bp = 0ull;
+          uint32_t bkl = 0u;
+          float bhi = 0.f, be = 0.f;
+#pragma unroll
+          for (int h = 0; h < kGper; ++h)
+            if (lane + 32 * h == bl) {
+              bp = pend[h];
+              bkl = kl[h];
+              bhi = hi[h];
+              be = e[h];
+            }
+          bp = shfl_u64(bp, src);
+          if (bp != 0ull) {
+            // inexact: accepted as it is only if its lower key leads every other upper key
+            bkl = __shfl_sync(0xffffffffu, bkl, src);
+            const unsigned long long low = gram_key(bkl, mem[bl].idx);
+            unsigned long long second = 0ull;
+#pragma unroll
+            for (int h = 0; h < kGper; ++h)
+              if (lane + 32 * h != bl && kh[h] != 0u)
+                second = max(second, gram_key(kh[h], mem[lane + 32 * h].idx));
+            second = warp_max_u64(second);
+            if (!(bkl != 0u && low > Up && low > second)) {
+              bhi = __shfl_sync(0xffffffffu, bhi, src);
+              be = __shfl_sync(0xffffffffu, be, src);
+              U4 xv[NCH], xc[NCH];
+              load_row((int)mem[bl].idx, xv);
+              while (bp) {
+                const int j = __ffsll((long long)bp) - 1;
+                bp &= bp - 1;
+                const int cj = acc_s[j];
+                if (__fsub_rd(pm[bl * kGpairLd + cj], eps) >= bhi) continue;   // excluded since
+                load_row((int)mem[cj].idx, xc);
+                be = fminf(be, distance(xv, xc, mem[bl].r, mem[cj].r));
+              }
+#pragma unroll
+              for (int h = 0; h < kGper; ++h)
+                if (lane + 32 * h == bl) {
+                  pend[h] = 0ull;
+                  e[h] = hi[h] = lo[h] = be;
+                  kh[h] = kl[h] = key_high(mem[bl].w, be);
+                }
+              continue;
+            }
+          }
           if (lane == 0) acc_s[nA] = bl;
-          ++nA;
-          const float rbv = lr[bl];
+          __syncwarp();
 #pragma unroll
           for (int h = 0; h < kGper; ++h) {
             const int u = lane + 32 * h;
-            if (u == bl) key[h] = 0ull;
-            if (key[h] != 0ull) {
-              cd[h] = fminf(cd[h], __fsub_rn(1.0f, __fmul_rn(__fmul_rn(pm[bl * kGpairLd + u], rv[h]), rbv)));
-              key[h] = argmax_key(__fmul_rn(wv[h], cd[h]), gi[h]);
+            if (u == bl) kh[h] = 0u;
+            if (kh[h] != 0u) {
+              const float d = pm[bl * kGpairLd + u];
+              if (!(__fsub_rd(d, eps) >= hi[h])) {
+                pend[h] |= 1ull << nA;
+                if (d == d) {
+                  hi[h] = fminf(hi[h], __fadd_ru(d, eps));
+                  lo[h] = fminf(lo[h], __fsub_rd(d, eps));
+                } else {
+                  lo[h] = -INFINITY;
+                }
+                kh[h] = key_high(mem[u].w, hi[h]);
+                kl[h] = lo[h] == -INFINITY ? 0u : key_high(mem[u].w, lo[h]);
+              }
             }
           }
+          ++nA;
         }
-        if (lane == 0) cnt[4] = nA;
+        if (lane == 0) cnt[2] = nA;
       }
       __syncthreads();
-      const int nA = cnt[4];
-      if (nA == 0) {   // cannot happen (the best live key is above U): leave rather than loop
+      const int nA = cnt[2];
+      if (nA == 0 && cnt[1] == 0) {   // cannot happen (the best live key is above U): leave, not loop
         if (tid == 0) atomicOr(a.err, kErrConfig);
         break;
       }
       if (tid < nA) {
-        const int gi = lidx[acc_s[tid]];
-        atomicOr(&sel[gi >> 5], 1u << (gi & 31));
+        const int gi = (int)mem[acc_s[tid]].idx, k = gi >> 5;
+        cen[tid] = make_float2(__int_as_float(gi), mem[acc_s[tid]].r);
+        atomicOr(&sel[k], 1u << (gi & 31));
+        if (k % C == rank) ks[(k / step) * kGthreads + ((k / C) % kGwarps) * 32 + (gi & 31)] = 0u;
       }
       taken += nA;
-      __syncthreads();
       // 5. update
-      if (taken < K) update(nA, false);
+      if (taken < K && nA > 0) update(nA);
+      else __syncthreads();
     }
   }
   __syncthreads();
@@ -756,21 +885,19 @@ void pick_nch(int nch, void **sel, void **norm) {
 }
 
 struct SelShape {
-  int C = 0, mc = 0, slots = 0, words = 0, accept = 0;
+  int C = 0, mc = 0, slots = 0, words = 0;
   size_t smem = 0;
 };
 // The shape of one request's cluster for clusters of c CTAs.
-SelShape shape_for(int c, int max_vis, int rb, int optin) {
+SelShape shape_for(int c, int max_vis, int optin) {
   SelShape s;
   s.C = c;
   s.mc = c == 1 ? 8 : c == 2 ? 6 : c <= 4 ? 4 : 3;
   const int nblk = (max_vis + 31) / 32;
   s.slots = (nblk + c * kGwarps - 1) / (c * kGwarps);
   s.words = nblk;
-  const size_t fixed = gram_sel_smem(0, rb, s.slots, s.words, c, s.mc).total;
-  if (fixed + 8 * (size_t)rb > (size_t)optin || s.slots * kGthreads > 65536) return SelShape();
-  s.accept = (int)std::min<size_t>(kGmaxAccept, (optin - fixed) / rb);
-  s.smem = gram_sel_smem(s.accept, rb, s.slots, s.words, c, s.mc).total;
+  s.smem = gram_sel_smem(s.slots, s.words, c, s.mc).total;
+  if (s.smem > (size_t)optin || s.slots > 32) return SelShape();
   return s;
 }
 
@@ -792,14 +919,14 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   SelShape sh;
   const int cmax = std::min(kMaxCluster, std::max(1, (pl.max_vis + kGthreads - 1) / kGthreads));
   for (int c = cmax; c >= 1; --c) {
-    const SelShape t = shape_for(c, pl.max_vis, rb, optin);
+    const SelShape t = shape_for(c, pl.max_vis, optin);
     if (t.C == 0) continue;
     const int active = active_clusters(sel_fn, c, t.smem, kGthreads);
     if (active <= 0) continue;
     sh = t;
     if (active >= pl.B) break;
   }
-  if (sh.C == 0) return cudaSuccess;   // too long for a cluster: the caller's other paths
+  if (sh.C == 0 || pl.max_vis > 0xffff) return cudaSuccess;   // too long for a cluster: the caller's other paths
 
   GramArgs g;
   std::memset(&g, 0, sizeof g);
@@ -836,8 +963,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   a.meta = g.meta;
   a.order = reinterpret_cast<const int32_t *>(ws + pl.off_order);
   a.dv = pl.dv; a.row_bytes = rb; a.csize = sh.C; a.mc = sh.mc; a.slots = sh.slots; a.words = sh.words;
-  a.accept = sh.accept;
-  a.eps = tc_distance_eps(pl.dv);
+  a.eps = gram_distance_eps(pl.dv);
   a.err = g.err;
   e = cudaFuncSetAttribute(sel_fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sel_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
