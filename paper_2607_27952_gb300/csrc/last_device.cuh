@@ -62,12 +62,6 @@ __device__ __forceinline__ U4 ldg_nc(const void *p) {
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
   return r;
 }
-// One fp32 value, not allocated in L1.
-__device__ __forceinline__ float ldg_f32_stream(const float *p) {
-  float v;
-  asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
-  return v;
-}
 __device__ __forceinline__ void prefetch_l2(const void *p) {
   asm volatile("prefetch.global.L2 [%0];" :: "l"(p));
 }

@@ -11,21 +11,34 @@
 //   2. the published entries above U = the largest (mc+1)-th key form the candidate
 //      list (at most kGlist; U rises to the first key cut off).  No token outside
 //      the list has a key above U, and keys never increase;
-//   3. the list's pairwise distances come from the Gram matrix, certified: a pair
-//      whose tensor-core distance is at least eps above both members' delta cannot
-//      matter; the others are evaluated in the canonical order;
-//   4. the greedy is replayed on the list alone while its best key is above U;
-//   5. the accepted centres' Gram rows are folded into the delta of the CTA's
-//      tokens: a centre with d~ - eps >= delta_i cannot lower delta_i, every other
-//      (token, centre) pair is evaluated in the canonical order.
-// Every CTA of a cluster does steps 2-4 alike, so a round has one cluster barrier.
+//   3. the members' pairwise distances come from the Gram matrix;
+//   4. warp 0 replays the greedy on the list alone while its best key is above U;
+//   5. meanwhile the other warps fold the accepted centres' Gram rows into their
+//      tokens, eight centres at a time as the replay posts them.
+// The Gram distances d~ are only known to within eps, the decisions are canonical, so
+// a token carries an interval: the minimum e over the centres evaluated so far, and up
+// to two pending centres whose d~ lies within eps of being the minimum.  Tokens are
+// ranked by the upper end; a member of the list has its pending centres evaluated in
+// the canonical order (by the CTA that owns it; a second cluster barrier), and during
+// the replay a member is evaluated again only when the order of the picks depends on
+// it.  A token far from the lead is never evaluated at all: evaluating every pair that
+// the certificate leaves open, at the moment it appears, took 185K of 400K cycles a
+// round on requests of 4096 tokens.
+// Every CTA of a cluster does the rest of steps 2-4 alike.
 //
 // Against the rounds that stream X (select_impl.cuh) a round reads 4 bytes per token
 // and centre instead of a whole row per token, so its cost no longer grows with
 // d_v, and the N^2 d_v contraction runs once, at tensor-core rates, on every SM.
 //
+// A round is bound by latency: about 30K cycles on a request of 576 tokens (k = 192, 14
+// rounds), of which the replay takes 650 a pick, 40K on 16384 tokens in 12 CTAs (k =
+// 2048, 76 rounds).  Measured against the rounds that stream X (GB300, whole last_prune
+// call): 64 requests of 576 x 2048, k 64/128/192: 1.71 -> 0.40 ms; 32 of 2880, k = 360:
+// 5.27 -> 1.23; 128 of 256..4096 x 1536, k = N/8: 10.3 -> 2.9; 8 of 16384 x 2048, k =
+// 2048: 16.9 -> 6.3 (3.6 of it the Gram matrix).
+//
 // Tokens are dealt to the cluster in blocks of 32: block k belongs to CTA k % C,
-// warp (k / C) % 16, so neighbouring tokens (tiles, frames, near-duplicates) spread
+// worker warp (k / C) % 15, so neighbouring tokens (tiles, frames, near-duplicates) spread
 // over all warps and both the ranking and the exact pairs stay balanced.
 //
 // Arithmetic of every decision is the canonical fp32 of the public header: the kept
@@ -41,6 +54,9 @@ namespace {
 
 constexpr int kGwarps = 16;
 constexpr int kGthreads = kGwarps * 32;
+constexpr int kGwork = kGwarps - 1;        // warps 1.. own the tokens, warp 0 replays the greedy
+constexpr int kGtok = kGwork * 32;
+constexpr int kGbatch = 8;                 // accepted centres handed to the workers at a time
 constexpr int kGlist = 64;                 // candidate list: two members per lane of the replay
 constexpr int kGper = kGlist / 32;
 constexpr int kGmaxAccept = 64;            // one bit per accepted centre
@@ -75,8 +91,10 @@ int gram_tiles(int n_tokens) {
 // chunk of kGchunk products is one chain of tensor-core accumulations: a sum of n exact
 // products in any order, each addition rounded or truncated once to fp32, errs by at
 // most n 2^-23 sum|x_i,k x_j,k|, and aligning groups of 16 products to the group's
-// largest exponent by 17/16 of that; taken twice.  The chunks are added in fp32 (8 u at
-// most), the canonical order adds 80 u (see tc_distance_eps) and the scalings 1e-6.
+// largest exponent by 17/16 of that; taken twice.  The chunks are added in fp32 (8 u
+// at most), the canonical order adds 80 u (see tc_distance_eps) and the scalings 1e-6.
+// Chains of 128 narrow it further (rounds of 4096-token requests 2.47 -> 2.05 M cycles)
+// but bind the Gram kernel to its epilogue: 3.6 -> 4.3 ms on 8 requests of 16384.
 constexpr int kGchunk = 256;
 inline float gram_distance_eps(int dv) {
   return (float)((std::min(dv, kGchunk) * 0x1p-22 + 88 * 0x1p-24) * 1.01 + 1e-6);
@@ -282,21 +300,23 @@ struct GramSelArgs {
 // A published candidate: upper key (high word), token, w~, 1/|x|, the evaluated
 // minimum e, and up to two centres whose distance is only known to within eps.
 struct GramEntry {
-  uint32_t kh, idx;
+  uint32_t idx;
   float w, r;
-  float e, p0, p1;
   uint32_t ids;            // centre of p0 | centre of p1 << 16
+  uint32_t kh;
+  float e, p0, p1;
 };
 static_assert(sizeof(GramEntry) == 32, "two 16-byte stores publish an entry");
 
 // Shared memory of select_gram_kernel (host sizing and device carve-up alike).
 struct GramSelSmem {
-  size_t ks, w, r, e, p0, p1, ids, fmask, fidx, sel, pub, ckey, cidx, pm, mem, acc, cen, misc, total;
+  size_t ks, w, r, e, p0, p1, ids, hot, sel, pkey, pub, ckey, cidx, pm, mem, res, top, acc, cen,
+      crow, bars, misc, total;
 };
 __host__ __device__ inline GramSelSmem gram_sel_smem(int slots, int words, int csize, int mc) {
   GramSelSmem s;
   size_t o = 0;
-  const size_t cap = (size_t)slots * kGthreads;   // token slots of a CTA
+  const size_t cap = (size_t)slots * kGtok;       // token slots of a CTA
   s.ks = o; o += 4 * cap;                         // high word of the upper key, 0 = not live
   s.w = o; o += 4 * cap;
   s.r = o; o += 4 * cap;
@@ -304,17 +324,21 @@ __host__ __device__ inline GramSelSmem gram_sel_smem(int slots, int words, int c
   s.p0 = o; o += 4 * cap;
   s.p1 = o; o += 4 * cap;
   s.ids = o; o += 4 * cap;
-  s.fmask = o; o += 8 * cap;                      // tokens to evaluate at once: their centres
-  s.fidx = o; o += align16(2 * cap);
+  s.hot = o; o += 4 * cap;                        // tokens a batch may lower: slot, centres
   s.sel = o; o += align16(4 * (size_t)words);     // selected bits of the whole request
-  s.pub = o; o += (size_t)2 * kGwarps * csize * (mc + 1) * sizeof(GramEntry);
-  s.ckey = o; o += 8 * kGcand;
+  s.pkey = o; o += (size_t)2 * kGwork * csize * (mc + 1) * 8;   // published keys
+  s.pub = o; o += (size_t)2 * kGwork * csize * (mc + 1) * sizeof(GramEntry);
+  s.ckey = o = align16(o); o += 8 * (kGcand + 2);
   s.cidx = o; o += 2 * kGcand;
   s.pm = o; o += align16(4 * kGlist * kGpairLd);  // the list's pairwise distances
   s.mem = o; o += sizeof(GramEntry) * kGlist;
+  s.res = o; o += 8 * kGlist;                     // members evaluated by their owners: key, delta
+  s.top = o; o += 8 * kGwarps * 16;               // a warp's leading keys
   s.acc = o; o += 4 * kGmaxAccept;
   s.cen = o; o += 8 * kGmaxAccept;                // accepted centres: token, 1/|x|
-  s.misc = o; o += 8 * 40;
+  s.crow = o; o += 4 * kGmaxAccept;               // and their Gram rows' offsets
+  s.bars = o; o += 8 * (kGmaxAccept / kGbatch);   // batch i of the round's centres is posted
+  s.misc = o; o += 8 * 48;
   s.total = align16(o);
   return s;
 }
@@ -353,18 +377,22 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
   float *p0_s = reinterpret_cast<float *>(smem + S.p0);
   float *p1_s = reinterpret_cast<float *>(smem + S.p1);
   uint32_t *id_s = reinterpret_cast<uint32_t *>(smem + S.ids);
-  unsigned long long *fmask = reinterpret_cast<unsigned long long *>(smem + S.fmask);
-  uint16_t *fidx = reinterpret_cast<uint16_t *>(smem + S.fidx);
+  uint32_t *hot = reinterpret_cast<uint32_t *>(smem + S.hot) + (warp - 1) * a.slots * 32;   // workers
   uint32_t *sel = reinterpret_cast<uint32_t *>(smem + S.sel);
   GramEntry *pub = reinterpret_cast<GramEntry *>(smem + S.pub);
+  unsigned long long *pkey = reinterpret_cast<unsigned long long *>(smem + S.pkey);
   unsigned long long *ckey = reinterpret_cast<unsigned long long *>(smem + S.ckey);
   uint16_t *cidx = reinterpret_cast<uint16_t *>(smem + S.cidx);
   float *pm = reinterpret_cast<float *>(smem + S.pm);
   GramEntry *mem = reinterpret_cast<GramEntry *>(smem + S.mem);
+  float2 *res = reinterpret_cast<float2 *>(smem + S.res);
+  unsigned long long *top_s = reinterpret_cast<unsigned long long *>(smem + S.top) + warp * 16;
   int *acc_s = reinterpret_cast<int *>(smem + S.acc);
   float2 *cen = reinterpret_cast<float2 *>(smem + S.cen);
+  uint32_t *crow = reinterpret_cast<uint32_t *>(smem + S.crow);
   unsigned long long *misc = reinterpret_cast<unsigned long long *>(smem + S.misc);
-  int *cnt = reinterpret_cast<int *>(misc + 32);   // [0] flagged tokens, [1] candidates, [2] picks
+  unsigned long long *bars = reinterpret_cast<unsigned long long *>(smem + S.bars);
+  int *cnt = reinterpret_cast<int *>(misc + 32);   // [0] kept tokens, [1] candidates, [2] picks, [4 + i] batch i
 
   const int rb = a.row_bytes, dv = a.dv, ld = gram_ld(N);
   const float eps = a.eps;
@@ -372,14 +400,25 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
   const char *xreq = a.x + (long long)voff * rb;
   const float *rreq = a.rn + voff, *wreq = a.w + voff;
   const float *G = a.gram + (long long)m[kGramOff] * 32;
-  const int P = kGwarps * C;                          // publishing warps of the cluster
-  const int step = C * kGwarps;                       // blocks between a warp's slots
-  const int blk0 = rank + C * warp;                   // this warp's first block
-  const int nslot = (nblk - blk0 + step - 1) / step;  // this warp's blocks (<= a.slots)
+  const int P = kGwork * C;                           // publishing warps of the cluster
+  const int step = C * kGwork;                        // blocks between a warp's slots
+  const int blk0 = rank + C * (warp - 1);             // a worker's first block
+  const int nslot = warp == 0 ? 0 : (nblk - blk0 + step - 1) / step;   // and its blocks (<= a.slots)
+  const int li0 = tid - 32;                           // a worker thread's first token slot
+  // block k (< 2^12): owner CTA and slot in shared memory, by multiplication
+  const uint32_t inv_c = (0xffffffffu / (uint32_t)C) + 1u, inv_step = (0xffffffffu / (uint32_t)step) + 1u;
+  auto over_c = [&](int k) { return C == 1 ? k : (int)__umulhi((uint32_t)k, inv_c); };
+  auto owned = [&](int k) { return k - over_c(k) * C == rank; };
+  auto slot_of = [&](int t) {   // of an owned token
+    const int k = t >> 5, z = (int)__umulhi((uint32_t)k, inv_step);
+    return z * kGtok + (over_c(k) - z * kGwork) * 32 + (t & 31);
+  };
 
+  if (tid < kGmaxAccept / kGbatch) mbar_init(&bars[tid], 1);
+  if (tid == 0) fence_mbar_init();
   for (int v = tid; v < nblk; v += kGthreads) sel[v] = K == N ? 0xffffffffu : 0u;
   for (int s = 0; s < nslot; ++s) {
-    const int t = 32 * (blk0 + s * step) + lane, li = s * kGthreads + tid;
+    const int t = 32 * (blk0 + s * step) + lane, li = s * kGtok + li0;
     const bool in = t < N;
     w_s[li] = in ? wreq[t] : 0.f;
     r_s[li] = in && K < N ? rreq[t] : 0.f;
@@ -422,101 +461,117 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       return __fsub_rn(1.0f, __fmul_rn(__fmul_rn(butterfly_sum(acc), ri), rc));
     };
 
-    // Fold the nA accepted centres cen[0 .. nA) into the tokens' distances.  A centre
-    // with d~ - eps at or above the token's upper bound cannot lower its delta.  Any
-    // other becomes one of the token's two pending centres; entries that a new upper
-    // bound excludes leave.  Pairs outside the certificate's norm range, NaN and a
-    // third pending centre are evaluated at once.
-    auto update = [&](int nA) {
-      if (tid == 0) cnt[0] = 0;
-      __syncthreads();
-      for (int s = 0; s < nslot; ++s) {
-        const int t = 32 * (blk0 + s * step) + lane, li = s * kGthreads + tid;
-        const bool live = ks[li] != 0u;
-        unsigned long long msk = 0ull;
-        const float ri = r_s[li];
-        float e = e_s[li], p0 = p0_s[li], p1 = p1_s[li];
-        uint32_t ids = id_s[li];
-        const bool in_range = tri_in_range(ri);
-        float hi = fminf(e, __fadd_ru(fminf(p0, p1), eps));
-        bool touched = false;
-        for (int j0 = 0; j0 < nA; j0 += 16) {
-          float g[16];
+    // A worker folds the accepted centres cen[j0 .. j0 + n) (n <= kGbatch) into its
+    // tokens.  A centre with d~ - eps at or above the token's upper bound cannot lower
+    // its delta.  Any other becomes one of the token's two pending centres; entries that
+    // a new upper bound excludes leave.  Pairs outside the certificate's norm range, NaN
+    // and a third pending centre are evaluated at once.
+    auto update = [&](int j0, int n) {
+      const uint32_t all = (1u << n) - 1u;
+      // centres whose pairs the certificate does not cover
+      const uint32_t wide = __ballot_sync(0xffffffffu, lane < n && !tri_in_range(cen[j0 + min(lane, n - 1)].y));
+      int nq = 0;
+      // this batch's part of the rows starts towards L2 (a line per block and centre)
+      for (int i = lane; i < kGbatch * nslot; i += 32)
+        if (i % kGbatch < n)
+          prefetch_l2(G + crow[j0 + i % kGbatch] + 32 * (blk0 + (i / kGbatch) * step));
+      // Four blocks at a time, 32 loads in flight per thread.  d~ - eps < hi is tested as
+      // g rc >= (1 - eps - hi) / ri with a slack of 1e-6 for the roundings; what passes
+      // is queued and tested again below.  (Dead tokens load too: a row holds whole blocks.)
+      for (int s0 = 0; s0 < nslot; s0 += 4) {
+        float g[4][kGbatch];
+        const float *gt = G + 32 * (blk0 + s0 * step) + lane;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int c = __float_as_int(cen[min(j0 + j, nA - 1)].x);
-            g[j] = live ? ldg_f32_stream(G + (long long)c * ld + t) : 0.f;
-          }
+        for (int j = 0; j < kGbatch; ++j) {
+          const float *gr = gt + crow[j0 + min(j, n - 1)];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            if (j0 + j < nA) {
-              const float rc = cen[j0 + j].y;
-              const float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[j], ri), rc));
-              if (live && (!(__fsub_rd(d, eps) >= hi) || !in_range || !tri_in_range(rc))) {
-                touched = true;
-                if (!in_range || !tri_in_range(rc) || d != d) {
-                  msk |= 1ull << (j0 + j);
-                } else {
-                  const uint32_t c = __float_as_uint(cen[j0 + j].x);
-                  hi = fminf(hi, __fadd_ru(d, eps));
-                  if (__fsub_rd(p0, eps) >= hi) p0 = INFINITY;
-                  if (__fsub_rd(p1, eps) >= hi) p1 = INFINITY;
-                  if (p0 == INFINITY) {
-                    p0 = d;
-                    ids = (ids & 0xffff0000u) | c;
-                  } else if (p1 == INFINITY) {
-                    p1 = d;
-                    ids = (ids & 0xffffu) | (c << 16);
-                  } else {
-                    msk |= 1ull << (j0 + j);
-                  }
-                }
+          for (int z = 0; z < 4; ++z) g[z][j] = __ldg(gr + (s0 + z < nslot ? 32 * z * step : 0));
+        }
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          if (s0 + z >= nslot) break;
+          const int li = (s0 + z) * kGtok + li0;
+          const float ri = r_s[li], hi = fminf(e_s[li], __fadd_ru(fminf(p0_s[li], p1_s[li]), eps));
+          const float thr = __fdiv_rn(1.0f - eps - hi - 1e-6f, ri);
+          uint32_t low = tri_in_range(ri) ? wide : all;
+#pragma unroll
+          for (int j = 0; j < kGbatch; ++j)
+            if (!(g[z][j] * cen[j0 + min(j, n - 1)].y < thr)) low |= 1u << j;   // NaN: tested again
+          low = ks[li] != 0u ? low & all : 0u;
+          const unsigned bal = __ballot_sync(0xffffffffu, low != 0u);
+          if (low) hot[nq + __popc(bal & ((1u << lane) - 1u))] = (uint32_t)li | (low << 16);
+          nq += __popc(bal);
+        }
+      }
+      __syncwarp();
+      for (int q0 = 0; q0 < nq; q0 += 32) {
+        uint32_t now = 0u;   // centres to evaluate at once
+        int li = 0, t = 0;
+        float ri = 0.f;
+        if (q0 + lane < nq) {
+          const uint32_t h = hot[q0 + lane];
+          uint32_t bt = h >> 16;
+          li = (int)(h & 0xffffu);
+          const int z = li / kGtok;   // (a constant divisor)
+          t = 32 * (blk0 + z * step) + (li & 31);
+          ri = r_s[li];
+          const bool in_range = tri_in_range(ri);
+          const float e = e_s[li];
+          float p0 = p0_s[li], p1 = p1_s[li], hi = fminf(e, __fadd_ru(fminf(p0, p1), eps));
+          uint32_t ids = id_s[li];
+          while (bt) {
+            const int j = __ffs(bt) - 1;
+            bt &= bt - 1;
+            const float2 cc = cen[j0 + j];
+            const float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(__ldg(G + crow[j0 + j] + t), ri), cc.y));
+            if (!in_range || ((wide >> j) & 1u) || d != d) {
+              now |= 1u << j;
+            } else if (!(__fsub_rd(d, eps) >= hi)) {
+              const uint32_t c = __float_as_uint(cc.x);
+              hi = fminf(hi, __fadd_ru(d, eps));
+              if (__fsub_rd(p0, eps) >= hi) p0 = INFINITY;
+              if (__fsub_rd(p1, eps) >= hi) p1 = INFINITY;
+              if (p0 == INFINITY) {
+                p0 = d;
+                ids = (ids & 0xffff0000u) | c;
+              } else if (p1 == INFINITY) {
+                p1 = d;
+                ids = (ids & 0xffffu) | (c << 16);
+              } else {
+                now |= 1u << j;
               }
             }
           }
-        }
-        if (touched) {
           p0_s[li] = p0;
           p1_s[li] = p1;
           id_s[li] = ids;
           ks[li] = key_high(w_s[li], fminf(e, __fadd_ru(fminf(p0, p1), eps)));
         }
-        const unsigned bal = __ballot_sync(0xffffffffu, msk != 0ull);
-        if (bal) {
-          int base = 0;
-          if (lane == 0) base = atomicAdd(&cnt[0], __popc(bal));
-          base = __shfl_sync(0xffffffffu, base, 0);
-          if (msk) {
-            const int pos = base + __popc(bal & ((1u << lane) - 1u));
-            fidx[pos] = (uint16_t)li;
-            fmask[pos] = msk;
-          }
-        }
-      }
-      __syncthreads();
-      // a warp per flagged token: its masked centres in the canonical order
-      const int nf = cnt[0];
-      for (int f = warp; f < nf; f += kGwarps) {
-        const int li = fidx[f];
-        unsigned long long msk = fmask[f];
-        const int k = rank + C * ((li >> 5) % kGwarps) + (li / kGthreads) * step;
-        U4 xv[NCH], xc[NCH];
-        load_row(32 * k + (li & 31), xv);
-        float e = e_s[li];
-        while (msk) {
-          const int j = __ffsll(msk) - 1;
-          msk &= msk - 1;
-          const float2 c = cen[j];
-          load_row(__float_as_int(c.x), xc);
-          e = fminf(e, distance(xv, xc, r_s[li], c.y));
-        }
         __syncwarp();
-        if (lane == 0) {
-          e_s[li] = e;
-          ks[li] = key_high(w_s[li], fminf(e, __fadd_ru(fminf(p0_s[li], p1_s[li]), eps)));
+        // the whole warp per token to evaluate
+        for (unsigned todo = __ballot_sync(0xffffffffu, now != 0u); todo != 0u; todo &= todo - 1) {
+          const int src = __ffs(todo) - 1;
+          const int lt = __shfl_sync(0xffffffffu, li, src);
+          uint32_t bt = __shfl_sync(0xffffffffu, now, src);
+          U4 xv[NCH], xc[NCH];
+          load_row(__shfl_sync(0xffffffffu, t, src), xv);
+          const float rt = __shfl_sync(0xffffffffu, ri, src);
+          float e = e_s[lt];
+          while (bt) {
+            const int j = __ffs(bt) - 1;
+            bt &= bt - 1;
+            const float2 cc = cen[j0 + j];
+            load_row(__float_as_int(cc.x), xc);
+            e = fminf(e, distance(xv, xc, rt, cc.y));
+          }
+          __syncwarp();
+          if (lane == 0) {
+            e_s[lt] = e;
+            ks[lt] = key_high(w_s[lt], fminf(e, __fadd_ru(fminf(p0_s[lt], p1_s[lt]), eps)));
+          }
+          __syncwarp();
         }
       }
-      if (nf > 0) __syncthreads();
     };
 
     // ---- seed (Eq. 9): argmax w~ over the request, every CTA alike ----
@@ -530,14 +585,14 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       const int seed = key_index(best);
       if (tid == 0) {
         cen[0] = make_float2(__int_as_float(seed), rreq[seed]);
+        crow[0] = (uint32_t)seed * (uint32_t)ld;
         sel[seed >> 5] |= 1u << (seed & 31);
       }
-      if ((seed >> 5) % C == rank && ((seed >> 5) / C) % kGwarps == warp && lane == (seed & 31))
-        ks[((seed >> 5) / step) * kGthreads + tid] = 0u;
+      if (tid == 0 && owned(seed >> 5)) ks[slot_of(seed)] = 0u;
       __syncthreads();
     }
     int taken = 1;
-    if (taken < K) update(1);
+    if (taken < K && warp > 0) update(0, 1);
     csync();   // every CTA of the cluster runs before the first remote write
 
     // ---- rounds (Eq. 10-11) ----
@@ -545,50 +600,60 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
     for (int round = 0; taken < K; ++round) {
       const int par = round & 1;
       GramEntry *pubp = pub + (size_t)par * P * ent;
-      // 1. this warp's best live tokens by upper key: lane e ends with the e-th one
-      {
-        uint32_t done = 0u;   // slots of this lane already taken
-        uint32_t kh = 0u;
-        int ms = 0, mine = -1;
-        auto best_left = [&]() {
-          kh = 0u;
-          for (int s = 0; s < nslot; ++s) {
-            const uint32_t v = ks[s * kGthreads + tid];
-            if (v > kh && !((done >> s) & 1u)) {   // lower slots (lower tokens) win ties
-              kh = v;
-              ms = s;
-            }
-          }
-        };
-        best_left();
+      unsigned long long *keyp = pkey + (size_t)par * P * ent;
+      // 1. this warp's best live tokens by upper key, best first, into top_s: each lane
+      // queues its three best.  A lane whose third is taken may hide a fourth, which is
+      // below it: the third then becomes the bound.
+      if (warp > 0) {
+        unsigned long long k1 = 0ull, k2 = 0ull, k3 = 0ull, bound = 0ull;
+        for (int s = 0; s < nslot; ++s) {
+          const uint32_t v = ks[s * kGtok + li0];
+          const unsigned long long k = v ? gram_key(v, (uint32_t)(32 * (blk0 + s * step) + lane)) : 0ull;
+          const unsigned long long m1 = min(k, k1), m2 = min(m1, k2);
+          k1 = max(k, k1);
+          k2 = max(m1, k2);
+          k3 = max(m2, k3);
+        }
+        int left = 3;
+        if (lane < ent) top_s[lane] = 0ull;
+        __syncwarp();
         for (int e = 0; e < ent; ++e) {
-          const uint32_t mx = __reduce_max_sync(0xffffffffu, kh);
+          const uint32_t mx = __reduce_max_sync(0xffffffffu, (uint32_t)(k1 >> 32));
           if (mx == 0u) break;
-          unsigned win = __ballot_sync(0xffffffffu, kh == mx);
-          if (win & (win - 1u)) {   // equal values: the lowest token
-            const uint32_t blk = kh == mx ? (uint32_t)ms : 0xffffffffu;
-            const uint32_t low = __reduce_min_sync(0xffffffffu, blk);
-            win = __ballot_sync(0xffffffffu, kh == mx && (uint32_t)ms == low);
+          bool win = (uint32_t)(k1 >> 32) == mx;
+          const unsigned bal = __ballot_sync(0xffffffffu, win);
+          if (bal & (bal - 1u)) {   // equal values: the lowest token
+            const uint32_t lo = __reduce_max_sync(0xffffffffu, win ? (uint32_t)k1 : 0u);
+            win = win && (uint32_t)k1 == lo;
           }
-          const int src = __ffs(win) - 1;
-          const int li = __shfl_sync(0xffffffffu, ms, src) * kGthreads + warp * 32 + src;
-          if (lane == e) mine = li;
-          if (lane == src) {
-            done |= 1u << ms;
-            best_left();
+          if (win) {
+            top_s[e] = k1;
+            if (--left == 0) bound = k1;
+            k1 = k2;
+            k2 = k3;
+            k3 = 0ull;
           }
         }
-        if (lane < ent) {
-          uint4 v0 = make_uint4(0u, 0xffffffffu, 0u, 0u), v1 = make_uint4(0u, 0u, 0u, 0u);
-          if (mine >= 0) {
-            const int t = 32 * (blk0 + (mine / kGthreads) * step) + (mine & 31);
-            v0 = make_uint4(ks[mine], (uint32_t)t, __float_as_uint(w_s[mine]), __float_as_uint(r_s[mine]));
-            v1 = make_uint4(__float_as_uint(e_s[mine]), __float_as_uint(p0_s[mine]),
-                            __float_as_uint(p1_s[mine]), id_s[mine]);
+        if (nslot > 3 && __any_sync(0xffffffffu, left == 0)) {
+          bound = warp_max_u64(bound);
+          if (lane == 0) top_s[a.mc] = max(top_s[a.mc], bound);
+        }
+        __syncwarp();
+        // entry lane % 4, 8 or 16 to CTAs lane / 4, 8 or 16, ..
+        const int esh = ent <= 4 ? 2 : ent <= 8 ? 3 : 4, e = lane & ((1 << esh) - 1);
+        if (e < ent) {
+          const unsigned long long kk = top_s[e];
+          uint4 v0 = make_uint4(0u, 0u, 0u, 0u), v1 = v0;
+          if (kk != 0ull) {
+            const int t = key_index(kk), li = slot_of(t);
+            v0 = make_uint4((uint32_t)t, __float_as_uint(w_s[li]), __float_as_uint(r_s[li]), id_s[li]);
+            v1 = make_uint4(ks[li], __float_as_uint(e_s[li]), __float_as_uint(p0_s[li]),
+                            __float_as_uint(p1_s[li]));
           }
-          GramEntry *dst = &pubp[(rank * kGwarps + warp) * ent + lane];
-          for (int q = 0; q < C; ++q) {
-            const uint32_t addr = map_shared(dst, q);
+          const int slot = (rank * kGwork + warp - 1) * ent + e;
+          for (int q = lane >> esh; q < C; q += 32 >> esh) {
+            st_cluster_u64(map_shared(&keyp[slot], q), kk);
+            const uint32_t addr = map_shared(&pubp[slot], q);
             st_cluster_v4u(addr, v0);
             st_cluster_v4u(addr + 16, v1);
           }
@@ -598,15 +663,11 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       csync();
       // 2. the list: published entries above U
       unsigned long long U = 0ull;
-      for (int q = lane; q < P; q += 32) {
-        const GramEntry &v = pubp[q * ent + a.mc];
-        if (v.kh != 0u) U = max(U, gram_key(v.kh, v.idx));
-      }
+      for (int q = lane; q < P; q += 32) U = max(U, keyp[q * ent + a.mc]);
       U = warp_max_u64(U);
       for (int e0 = warp * 32; e0 < P * ent; e0 += kGthreads) {
         const int e = e0 + lane;
-        unsigned long long kk = 0ull;
-        if (e < P * ent && pubp[e].kh != 0u) kk = gram_key(pubp[e].kh, pubp[e].idx);
+        const unsigned long long kk = e < P * ent ? keyp[e] : 0ull;
         const bool up = kk > U;
         const unsigned bal = __ballot_sync(0xffffffffu, up);
         if (bal) {
@@ -622,14 +683,18 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       }
       __syncthreads();
       const int nc = cnt[1];
-      // the best kGlist of them; U' = the first key cut off
+      if (warp == 0) ckey[nc] = 0ull;
+      __syncthreads();
+      // the best kGlist of them in key order (the same in every CTA); U' = the first
+      // key cut off
       for (int c0 = warp * 32; c0 < nc; c0 += kGthreads) {
         const int c = c0 + lane;
         const unsigned long long kk = c < nc ? ckey[c] : 0ull;
-        int pos = c;
-        if (nc > kGlist) {
-          pos = 0;
-          for (int q = 0; q < nc; ++q) pos += ckey[q] > kk ? 1 : 0;
+        int pos = 0;
+#pragma unroll 4
+        for (int q = 0; q < nc; q += 2) {   // (ckey[nc] is zero)
+          const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(&ckey[q]);
+          pos += (x.x > kk ? 1 : 0) + (x.y > kk ? 1 : 0);
         }
         if (c < nc) {
           if (pos < kGlist) mem[pos] = pubp[cidx[c]];
@@ -637,28 +702,54 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
         }
       }
       __syncthreads();
+      if (nc == 0) {   // cannot happen (the best live key is above U): every CTA leaves alike
+        if (tid == 0) atomicOr(a.err, kErrConfig);
+        break;
+      }
       const int nL = min(nc, kGlist);
       const unsigned long long Up = nc > kGlist ? misc[20] : U;
-      // 3. the list's Gram rows for this CTA's tokens start towards L2; pairwise
-      // distances from the Gram matrix (NaN: outside the certificate)
-      for (int s = 0; s < nslot; ++s)
-        for (int u = lane; u < nL; u += 32)
-          prefetch_l2(G + (long long)mem[u].idx * ld + 32 * (blk0 + s * step));
+      unsigned long long need = 0ull;   // this warp's share of the CTA's members
+      int before = 0;
+#pragma unroll
+      for (int h = 0; h < kGper; ++h) {
+        const int u = lane + 32 * h;
+        const bool mine = u < nL && owned((int)(mem[u].idx >> 5)) &&
+                          !(mem[u].p0 == INFINITY && mem[u].p1 == INFINITY);
+        const unsigned bal = __ballot_sync(0xffffffffu, mine);
+        const int at = before + __popc(bal & ((1u << lane) - 1u));
+        need |= (unsigned long long)__ballot_sync(0xffffffffu, mine && at % kGwarps == warp) << (32 * h);
+        before += __popc(bal);
+      }
+      // their rows start towards L2
+      for (unsigned long long n = need; n != 0ull; n &= n - 1) {
+        const GramEntry &me = mem[__ffsll((long long)n) - 1];
+        if (lane * 128 < rb) {
+          prefetch_l2(xreq + (long long)me.idx * rb + lane * 128);
+          if (me.p0 != INFINITY) prefetch_l2(xreq + (long long)(me.ids & 0xffffu) * rb + lane * 128);
+        }
+      }
+      // 3. pairwise distances from the Gram matrix (NaN: outside the certificate): a warp
+      // takes rows u and kGlist - 1 - u together, 63 pairs
       {
-        constexpr int kRows = kGlist / kGwarps;
+        constexpr int kRows = kGlist / 2 / kGwarps;
         float g[kRows][kGper];
+        int pu[kRows][kGper], pv[kRows][kGper];
 #pragma unroll
         for (int i = 0; i < kRows; ++i)
 #pragma unroll
           for (int h = 0; h < kGper; ++h) {
-            const int u = warp + i * kGwarps, v = lane + 32 * h;
-            g[i][h] = u < v && v < nL ? ldg_f32_stream(G + (long long)mem[u].idx * ld + mem[v].idx) : 0.f;
+            const int u = warp + i * kGwarps, x = lane + 32 * h, len = kGlist - 1 - u;
+            pu[i][h] = x < len ? u : len;
+            pv[i][h] = x < len ? u + 1 + x : x + 1;
+            g[i][h] = 0.f;
+            if (pv[i][h] < nL && pu[i][h] < pv[i][h])
+              g[i][h] = __ldg(G + (long long)mem[pu[i][h]].idx * ld + mem[pv[i][h]].idx);
           }
 #pragma unroll
         for (int i = 0; i < kRows; ++i)
 #pragma unroll
           for (int h = 0; h < kGper; ++h) {
-            const int u = warp + i * kGwarps, v = lane + 32 * h;
+            const int u = pu[i][h], v = pv[i][h];
             if (u < v && v < nL) {
               const float ru = mem[u].r, rv = mem[v].r;
               float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[i][h], ru), rv));
@@ -667,98 +758,128 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
             }
           }
       }
-      // the members' pending centres in the canonical order: every member's delta is
-      // exact from here on (every CTA alike; the owner keeps the result)
-      for (int u = warp; u < nL; u += kGwarps) {
-        const GramEntry me = mem[u];
-        if (me.p0 == INFINITY && me.p1 == INFINITY) continue;
-        U4 xv[NCH], xc[NCH];
-        load_row((int)me.idx, xv);
-        float e = me.e;
-        if (me.p0 != INFINITY) {
-          const int c = (int)(me.ids & 0xffffu);
-          load_row(c, xc);
-          e = fminf(e, distance(xv, xc, me.r, rreq[c]));
-        }
-        if (me.p1 != INFINITY) {
-          const int c = (int)(me.ids >> 16);
-          load_row(c, xc);
-          e = fminf(e, distance(xv, xc, me.r, rreq[c]));
-        }
-        const uint32_t kh = key_high(me.w, e);
-        if (lane == 0) {
-          mem[u].e = e;
-          mem[u].kh = kh;
-          const int k = (int)me.idx >> 5;
-          if (k % C == rank) {
-            const int li = (k / step) * kGthreads + ((k / C) % kGwarps) * 32 + (int)(me.idx & 31u);
+      // the members' pending centres in the canonical order, by the CTA that owns the
+      // member, which keeps the result and sends it to every CTA: every member's delta
+      // is exact from here on
+      {
+        for (; need != 0ull; need &= need - 1) {
+          const int u = __ffsll((long long)need) - 1;
+          const GramEntry me = mem[u];
+          const int c0 = (int)(me.ids & 0xffffu), c1 = (int)(me.ids >> 16);
+          const float rc0 = me.p0 != INFINITY ? rreq[c0] : 0.f, rc1 = me.p1 != INFINITY ? rreq[c1] : 0.f;
+          U4 xv[NCH], xc[NCH];
+          load_row((int)me.idx, xv);
+          float e = me.e;
+          if (me.p0 != INFINITY) {
+            load_row(c0, xc);
+            e = fminf(e, distance(xv, xc, me.r, rc0));
+          }
+          if (me.p1 != INFINITY) {
+            load_row(c1, xc);
+            e = fminf(e, distance(xv, xc, me.r, rc1));
+          }
+          const uint32_t kh = key_high(me.w, e);
+          if (lane == 0) {
+            const int li = slot_of((int)me.idx);
             e_s[li] = e;
             p0_s[li] = INFINITY;
             p1_s[li] = INFINITY;
             ks[li] = kh;
           }
+          if (lane < C) st_cluster_v2f(map_shared(&res[u], lane), make_float2(__uint_as_float(kh), e));
         }
       }
-      __syncthreads();
+      csync();
       // 4. replay the greedy on the list (warp 0; lane u holds members u, u + 32, ..).
       // A member's delta lies in [lo, hi]: exact until an accepted centre's distance
       // reaches below hi + eps; such centres are kept in `pend` and evaluated only when
       // the member's place in the order depends on it.
       if (warp == 0) {
-        uint32_t kh[kGper], kl[kGper];   // upper and lower key, high words
-        float e[kGper], hi[kGper], lo[kGper];
+        uint32_t kh[kGper], id[kGper];   // upper key (high word), token
+        float e[kGper], hi[kGper], lo[kGper], wv[kGper];
         unsigned long long pend[kGper];
 #pragma unroll
         for (int h = 0; h < kGper; ++h) {
           const int u = lane + 32 * h;
-          const bool in = u < nL;
-          kh[h] = kl[h] = in ? mem[u].kh : 0u;
-          e[h] = hi[h] = lo[h] = in ? mem[u].e : 0.f;
+          kh[h] = 0u;
+          id[h] = 0u;
+          e[h] = wv[h] = 0.f;
+          if (u < nL) {
+            const bool was = mem[u].p0 != INFINITY || mem[u].p1 != INFINITY;   // evaluated just now
+            const float2 rv = res[u];
+            kh[h] = was ? __float_as_uint(rv.x) : mem[u].kh;
+            e[h] = was ? rv.y : mem[u].e;
+            id[h] = mem[u].idx;
+            wv[h] = mem[u].w;
+          }
+          hi[h] = lo[h] = e[h];
           pend[h] = 0ull;
         }
+        const uint32_t up_hi = (uint32_t)(Up >> 32);
         int nA = 0;
-        while (taken + nA < K && nA < kGmaxAccept) {
-          unsigned long long lk = 0ull;
-          int lh = 0;
+        const int most = min(K - taken, kGmaxAccept);
+        while (nA < most) {
+          // the member with the largest upper key (equal values: the lowest token)
+          uint32_t lk = kh[0];
 #pragma unroll
-          for (int h = 0; h < kGper; ++h) {
-            const unsigned long long k = kh[h] ? gram_key(kh[h], mem[lane + 32 * h].idx) : 0ull;
-            if (k > lk) {
-              lk = k;
-              lh = h;
+          for (int h = 1; h < kGper; ++h) lk = max(lk, kh[h]);
+          const uint32_t mx = __reduce_max_sync(0xffffffffu, lk);
+          unsigned win[kGper];
+          int leads = 0, bl = 0;
+          bool inexact = false;
+#pragma unroll
+          for (int h = kGper - 1; h >= 0; --h) {
+            win[h] = __ballot_sync(0xffffffffu, kh[h] == mx);
+            leads += __popc(win[h]);
+            const unsigned open = __ballot_sync(0xffffffffu, kh[h] == mx && pend[h] != 0ull);
+            bl = win[h] ? __ffs(win[h]) - 1 + 32 * h : bl;
+            inexact = win[h] ? open != 0u : inexact;
+          }
+          if (mx <= up_hi || leads > 1) {
+            if (mx < up_hi || mx == 0u) break;   // also the end of the list
+            uint32_t lid = 0xffffffffu;
+#pragma unroll
+            for (int h = 0; h < kGper; ++h) lid = kh[h] == mx ? min(lid, id[h]) : lid;
+            const uint32_t low = __reduce_min_sync(0xffffffffu, lid);
+            if (gram_key(mx, low) <= Up) break;
+#pragma unroll
+            for (int h = 0; h < kGper; ++h) {
+              const unsigned w = __ballot_sync(0xffffffffu, kh[h] == mx && id[h] == low);
+              const unsigned open = __ballot_sync(0xffffffffu, kh[h] == mx && id[h] == low && pend[h] != 0ull);
+              if (w) {
+                bl = __ffs(w) - 1 + 32 * h;
+                inexact = open != 0u;
+              }
             }
           }
-          const unsigned long long bk = warp_max_u64(lk);
-          if (bk <= Up) break;   // also the end of the list (key 0)
-          const int src = __ffs(__ballot_sync(0xffffffffu, lk == bk)) - 1;
-          const int bl = src + 32 * __shfl_sync(0xffffffffu, lh, src);
-          unsigned long long bp = 0ull;
-          uint32_t bkl = 0u;
-          float bhi = 0.f, be = 0.f;
+          if (inexact) {
+            // accepted as it is only if its lower key leads every other upper key
+            const int src = bl & 31;
+            unsigned long long bp = 0ull;
+            uint32_t bkl = 0u, bid = 0u;
+            float bhi = 0.f, be = 0.f;
+            uint32_t second = 0u;   // best other upper key (high word)
 #pragma unroll
-          for (int h = 0; h < kGper; ++h)
-            if (lane + 32 * h == bl) {
-              bp = pend[h];
-              bkl = kl[h];
-              bhi = hi[h];
-              be = e[h];
+            for (int h = 0; h < kGper; ++h) {
+              if (lane + 32 * h == bl) {
+                bp = pend[h];
+                bkl = lo[h] == -INFINITY ? 0u : key_high(wv[h], lo[h]);
+                bhi = hi[h];
+                be = e[h];
+                bid = id[h];
+              } else {
+                second = max(second, kh[h]);
+              }
             }
-          bp = shfl_u64(bp, src);
-          if (bp != 0ull) {
-            // inexact: accepted as it is only if its lower key leads every other upper key
             bkl = __shfl_sync(0xffffffffu, bkl, src);
-            const unsigned long long low = gram_key(bkl, mem[bl].idx);
-            unsigned long long second = 0ull;
-#pragma unroll
-            for (int h = 0; h < kGper; ++h)
-              if (lane + 32 * h != bl && kh[h] != 0u)
-                second = max(second, gram_key(kh[h], mem[lane + 32 * h].idx));
-            second = warp_max_u64(second);
-            if (!(bkl != 0u && low > Up && low > second)) {
+            second = __reduce_max_sync(0xffffffffu, second);
+            if (!(bkl > up_hi && bkl > second)) {
+              bp = shfl_u64(bp, src);
+              bid = __shfl_sync(0xffffffffu, bid, src);
               bhi = __shfl_sync(0xffffffffu, bhi, src);
               be = __shfl_sync(0xffffffffu, be, src);
               U4 xv[NCH], xc[NCH];
-              load_row((int)mem[bl].idx, xv);
+              load_row((int)bid, xv);
               while (bp) {
                 const int j = __ffsll((long long)bp) - 1;
                 bp &= bp - 1;
@@ -769,62 +890,73 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
               }
 #pragma unroll
               for (int h = 0; h < kGper; ++h)
-                if (lane + 32 * h == bl) {
-                  pend[h] = 0ull;
-                  e[h] = hi[h] = lo[h] = be;
-                  kh[h] = kl[h] = key_high(mem[bl].w, be);
+                if (32 * h <= bl && bl < 32 * (h + 1)) {
+                  if (lane == src) {
+                    pend[h] = 0ull;
+                    e[h] = hi[h] = lo[h] = be;
+                    kh[h] = key_high(wv[h], be);
+                  }
                 }
               continue;
             }
           }
-          if (lane == 0) acc_s[nA] = bl;
-          __syncwarp();
+          const uint32_t bidx = mem[bl].idx;
+          const float brn = mem[bl].r;
+          const unsigned long long bit = 1ull << nA;
 #pragma unroll
           for (int h = 0; h < kGper; ++h) {
             const int u = lane + 32 * h;
-            if (u == bl) kh[h] = 0u;
-            if (kh[h] != 0u) {
-              const float d = pm[bl * kGpairLd + u];
-              if (!(__fsub_rd(d, eps) >= hi[h])) {
-                pend[h] |= 1ull << nA;
-                if (d == d) {
-                  hi[h] = fminf(hi[h], __fadd_ru(d, eps));
-                  lo[h] = fminf(lo[h], __fsub_rd(d, eps));
-                } else {
-                  lo[h] = -INFINITY;
-                }
-                kh[h] = key_high(mem[u].w, hi[h]);
-                kl[h] = lo[h] == -INFINITY ? 0u : key_high(mem[u].w, lo[h]);
-              }
+            const float d = pm[bl * kGpairLd + u];
+            const float dlo = __fsub_rd(d, eps), dhi = __fadd_ru(d, eps);
+            const bool hit = !(dlo >= hi[h]);   // NaN too
+            pend[h] |= hit ? bit : 0ull;
+            lo[h] = hit ? (d == d ? fminf(lo[h], dlo) : -INFINITY) : lo[h];
+            hi[h] = hit ? fminf(hi[h], dhi) : hi[h];   // NaN keeps hi
+            kh[h] = kh[h] == 0u || u == bl ? 0u : key_high(wv[h], hi[h]);
+          }
+          // posted; every eighth centre releases a batch to the workers
+          if (lane == 0) {
+            acc_s[nA] = bl;
+            cen[nA] = make_float2(__uint_as_float(bidx), brn);
+            crow[nA] = bidx * (uint32_t)ld;   // N^2 < 2^32 (the matrix is at most 12 GiB)
+            if (nA % kGbatch == kGbatch - 1) {
+              cnt[4 + nA / kGbatch] = kGbatch;
+              mbar_arrive(&bars[nA / kGbatch]);
             }
           }
+          __syncwarp();
           ++nA;
         }
         if (lane == 0) cnt[2] = nA;
+        if (lane >= nA / kGbatch && lane < kGmaxAccept / kGbatch) {
+          cnt[4 + lane] = lane == nA / kGbatch ? nA % kGbatch : 0;
+          mbar_arrive(&bars[lane]);
+        }
+      } else {
+        // 5. meanwhile the workers fold the accepted centres into their tokens
+        for (int i = 0; i < kGmaxAccept / kGbatch; ++i) {
+          mbar_wait_bounded(&bars[i], par, a.err, kErrTimeout);
+          const int n = cnt[4 + i];
+          if (n > 0) update(i * kGbatch, n);
+          if (n < kGbatch) break;
+        }
       }
       __syncthreads();
       const int nA = cnt[2];
-      if (nA == 0 && cnt[1] == 0) {   // cannot happen (the best live key is above U): leave, not loop
-        if (tid == 0) atomicOr(a.err, kErrConfig);
-        break;
-      }
       if (tid < nA) {
         const int gi = (int)mem[acc_s[tid]].idx, k = gi >> 5;
-        cen[tid] = make_float2(__int_as_float(gi), mem[acc_s[tid]].r);
         atomicOr(&sel[k], 1u << (gi & 31));
-        if (k % C == rank) ks[(k / step) * kGthreads + ((k / C) % kGwarps) * 32 + (gi & 31)] = 0u;
+        if (owned(k)) ks[slot_of(gi)] = 0u;
       }
       taken += nA;
-      // 5. update
-      if (taken < K && nA > 0) update(nA);
-      else __syncthreads();
+      __syncthreads();
     }
   }
   __syncthreads();
 
   // ---- Eq. 12: ascending positions from the request's selected bits; every CTA
   // writes the indices and rows of its own blocks ----
-  int2 *out = reinterpret_cast<int2 *>(smem + S.fmask);   // (token, position) of the kept tokens
+  int2 *out = reinterpret_cast<int2 *>(smem + S.e);   // (token, position) of the kept tokens, over e and p0
   int *wsum = reinterpret_cast<int *>(misc);
   if (tid == 0) cnt[0] = 0;
   int run = 0;
@@ -894,10 +1026,10 @@ SelShape shape_for(int c, int max_vis, int optin) {
   s.C = c;
   s.mc = c == 1 ? 8 : c == 2 ? 6 : c <= 4 ? 4 : 3;
   const int nblk = (max_vis + 31) / 32;
-  s.slots = (nblk + c * kGwarps - 1) / (c * kGwarps);
+  s.slots = (nblk + c * kGwork - 1) / (c * kGwork);
   s.words = nblk;
   s.smem = gram_sel_smem(s.slots, s.words, c, s.mc).total;
-  if (s.smem > (size_t)optin || s.slots > 32) return SelShape();
+  if (s.smem > (size_t)optin || s.slots * kGtok > 0xffff) return SelShape();
   return s;
 }
 
@@ -917,7 +1049,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   // The largest clusters that still run every request at once, but no more CTAs than
   // give each warp a block of tokens; when none does, the smallest that fits.
   SelShape sh;
-  const int cmax = std::min(kMaxCluster, std::max(1, (pl.max_vis + kGthreads - 1) / kGthreads));
+  const int cmax = std::min(kMaxCluster, std::max(1, (pl.max_vis + kGtok - 1) / kGtok));
   for (int c = cmax; c >= 1; --c) {
     const SelShape t = shape_for(c, pl.max_vis, optin);
     if (t.C == 0) continue;
