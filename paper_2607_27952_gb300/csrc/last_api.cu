@@ -192,7 +192,7 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
     if (pl->gram) {
       m[kGramOff] = (int32_t)gram_off;
       gram_off += gram_units(b);
-      if (gram_units(b) > 0) pl->gram_tiles += gram_tiles(p->cu_vis[b + 1] - p->cu_vis[b]);
+      if (gram_units(b) > 0) pl->gram_tiles += gram_tiles(p->cu_vis[b + 1] - p->cu_vis[b], gram_long(pl->max_vis));
     }
     m[kRootOff] = (int32_t)root_off;
     if (sel_scratch) root_off += root_cap(b);

@@ -97,7 +97,9 @@ cudaError_t launch_select_grid(const Plan &pl, const float *w, const void *x, in
 cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, int32_t *idx_out,
                                void *x_out, char *ws, cudaStream_t s, bool *done);
 // Tiles of the Gram kernel for one request; floats per row of its matrix.
-int gram_tiles(int n_tokens);
+int gram_tiles(int n_tokens, bool pair);
+// Whether CTA pairs compute the matrices (the longest request decides).
+bool gram_long(int max_vis);
 #ifdef __CUDACC__
 __host__ __device__
 #endif

@@ -1,8 +1,8 @@
 // Eq. 9-12 (Sec. 3.4): the greedy selection of bf16 features from a Gram matrix.
 //
 // Three launches.  norms_kernel: 1/|x_i| of every token (canonical order).
-// gram_kernel: every request's dot products x_i . x_j on the tensor cores, fp32, to
-// the workspace (lower triangle computed, mirrored on the way out).
+// gram_kernel or gram_pair_kernel: every request's dot products x_i . x_j on the tensor
+// cores, fp32, to the workspace (lower triangle computed, mirrored on the way out).
 // select_gram_kernel: the greedy, one thread-block cluster of C CTAs per request,
 // in rounds that accept a batch of consecutive picks at once and give exactly the
 // sequential Eq. 10-11 sequence:
@@ -33,9 +33,9 @@
 // A round is bound by latency: about 30K cycles on a request of 576 tokens (k = 192, 14
 // rounds), of which the replay takes 650 a pick, 40K on 16384 tokens in 12 CTAs (k =
 // 2048, 76 rounds).  Measured against the rounds that stream X (GB300, whole last_prune
-// call): 64 requests of 576 x 2048, k 64/128/192: 1.71 -> 0.40 ms; 32 of 2880, k = 360:
-// 5.27 -> 1.23; 128 of 256..4096 x 1536, k = N/8: 10.3 -> 2.9; 8 of 16384 x 2048, k =
-// 2048: 16.9 -> 6.3 (3.6 of it the Gram matrix).
+// call): 64 requests of 576 x 2048, k 64/128/192: 1.71 -> 0.39 ms; 32 of 2880, k = 360:
+// 5.27 -> 1.17; 128 of 256..4096 x 1536, k = N/8: 10.3 -> 2.5; 8 of 16384 x 2048, k =
+// 2048: 16.9 -> 5.0 (3.0 of it the Gram matrix).
 //
 // Tokens are dealt to the cluster in blocks of 32: block k belongs to CTA k % C,
 // worker warp (k / C) % 15, so neighbouring tokens (tiles, frames, near-duplicates) spread
@@ -47,6 +47,8 @@
 
 #include <algorithm>
 #include <cstring>
+#include <functional>
+#include <vector>
 
 namespace last {
 
@@ -67,8 +69,9 @@ constexpr int kGcand = 1024;               // published entries above U kept bef
 constexpr int kGM = 128, kGN = 256, kGK = 64;
 constexpr int kGramStages = 4;
 constexpr int kGramStageBytes = (kGM + kGN) * kGK * 2;   // 48 KB
+constexpr int kPairStages = 3;
+constexpr int kPairStageBytes = 2 * 2 * kGM * kGK * 2;   // two K blocks, 64 KB per CTA of a pair
 constexpr int kGramThreads = 320;          // 8 epilogue warps, TMA producer, MMA issuer
-constexpr int kGramChunkKb = 4;            // K blocks per accumulation chain (kGchunk products)
 constexpr int kGroupRows = 16;             // row blocks per tile group (L2 reuse of both operands)
 
 }  // namespace
@@ -80,7 +83,11 @@ __host__ __device__ inline int gram_group_tiles(int g, int h) {
   for (int c = 0; 2 * c < h; ++c) n += h - 2 * c;
   return n;
 }
-int gram_tiles(int n_tokens) {
+int gram_tiles(int n_tokens, bool pair) {
+  if (pair) {
+    const int R = (n_tokens + kGN - 1) / kGN;
+    return R * (R + 1) / 2;
+  }
   const int R = (n_tokens + kGM - 1) / kGM;
   int n = 0;
   for (int g = 0; 16 * g < R; ++g) n += gram_group_tiles(g, std::min(kGroupRows, R - 16 * g));
@@ -88,33 +95,65 @@ int gram_tiles(int n_tokens) {
 }
 
 // Bound on |d~ - d| between a distance from the Gram matrix and the canonical one.  A
-// chunk of kGchunk products is one chain of tensor-core accumulations: a sum of n exact
+// chunk of products is one chain of tensor-core accumulations: a sum of n exact
 // products in any order, each addition rounded or truncated once to fp32, errs by at
 // most n 2^-23 sum|x_i,k x_j,k|, and aligning groups of 16 products to the group's
-// largest exponent by 17/16 of that; taken twice.  The chunks are added in fp32 (8 u
-// at most), the canonical order adds 80 u (see tc_distance_eps) and the scalings 1e-6.
-// Chains of 128 narrow it further (rounds of 4096-token requests 2.47 -> 2.05 M cycles)
-// but bind the Gram kernel to its epilogue: 3.6 -> 4.3 ms on 8 requests of 16384.
-constexpr int kGchunk = 256;
-inline float gram_distance_eps(int dv) {
-  return (float)((std::min(dv, kGchunk) * 0x1p-22 + 88 * 0x1p-24) * 1.01 + 1e-6);
+// largest exponent by 17/16 of that; taken twice.  The chunks are added in fp32 (8 u at
+// most), the canonical order adds 80 u (see tc_distance_eps) and the scalings 1e-6.
+inline float gram_distance_eps(int dv, int chunk) {
+  return (float)((std::min(dv, chunk) * 0x1p-22 + 88 * 0x1p-24) * 1.01 + 1e-6);
 }
+// Requests of at least this many tokens take CTA pairs; below, the pairs' 256-row tiles
+// waste more than they gain (64 requests of 576: 0.111 against 0.090 ms).
+bool gram_long(int max_vis) { return max_vis >= 2048; }
+// Products per chain.  Short chains narrow the bound, so fewer distances are evaluated
+// in the canonical order, but each costs the Gram kernel a pass over its accumulators,
+// and long requests spend most of their time there.  Whole calls, pairs with chains of
+// 256 / 512 / 1024 / 2048: 32 requests of 2880 1.22 / 1.17 / - / - ms, 128 of 256..4096
+// 2.51 / 2.53, 8 of 16384 - / 5.45 / 5.00 / 5.18.
+int gram_chunk(int max_vis) { return max_vis >= 8192 ? 1024 : max_vis >= 2048 ? 512 : 256; }
 
 struct GramArgs {
   CUtensorMap tmap;        // X as [total_vis][dv] bf16, box 64 x 128, 128-byte swizzle
   float *gram;
   const int32_t *meta;
   const int32_t *tile0;    // [B + 1] first tile of each request
-  int B, dv, total_tiles;
+  int B, dv, total_tiles, chunk_kb;   // chunk_kb: K blocks per accumulation chain
   unsigned *err;
 };
+
+// Row i, columns j0 .. j0 + 127 of a request's matrix, and the same values as a column
+// when `mirror`.
+__device__ __forceinline__ void store_tile(const GramArgs &a, int b, int i, int j0, bool mirror,
+                                           const float *v) {
+  const int32_t *m = a.meta + b * kMetaFields;
+  const int N = m[kNumVis], ld = gram_ld(N);
+  float *G = a.gram + (long long)m[kGramOff] * 32;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int j = j0 + 32 * c;
+    if (j < N) {
+      if (i < N) {
+        float *row = G + (long long)i * ld + j;
+#pragma unroll
+        for (int q = 0; q < 32; q += 8) st_global_v8(row + q, v + 32 * c + q);
+      }
+      if (mirror && i < ld) {
+        float *col = G + (long long)j * ld + i;
+#pragma unroll
+        for (int q = 0; q < 32; ++q)
+          if (j + q < N) col[(long long)q * ld] = v[32 * c + q];
+      }
+    }
+  }
+}
 
 __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_constant__ GramArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  __shared__ unsigned long long full[kGramStages], empty[kGramStages], afull[2], aempty[2];
-  __shared__ uint32_t tslot[2];   // TMEM base, abort word
+  __shared__ unsigned long long full[kGramStages], empty[kGramStages], afull[2], aempty[2], never;
+  __shared__ uint32_t tslot;   // TMEM base
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nkb = tc_kblocks(a.dv);
   if (threadIdx.x == 0) {
@@ -126,21 +165,19 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
       mbar_init(&afull[i], 1);
       mbar_init(&aempty[i], 8);
     }
-    tslot[1] = 0;
+    mbar_init(&never, 1);
     fence_mbar_init();
   }
-  if (warp == 0) tmem_alloc(&tslot[0], 512);
+  if (warp == 0) tmem_alloc(&tslot, 512);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = tslot[0];
-  // after one expired wait every later wait returns at once and the call reports it
+  const uint32_t tmem = tslot;
+  // a role's waits: after one has expired the others return at once and the call reports it
+  bool dead = false;
   auto twait = [&](unsigned long long *bar, uint32_t par) -> bool {
-    volatile uint32_t *abort_w = &tslot[1];
-    if (*abort_w) return false;
-    if (mbar_wait_bounded(bar, par, a.err, kErrTimeout)) return true;
-    *abort_w = 1u;
-    return false;
+    if (!dead && !mbar_wait_bounded(bar, par, a.err, kErrTimeout)) dead = true;
+    return !dead;
   };
   // tile -> (request, row block, column block)
   auto decode = [&](int tile, int *b_, int *ti, int *tj) {
@@ -169,49 +206,58 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
 
   if (warp == 8) {
     if (lane == 0) {
-      uint32_t it = 0;
+      int st = 0;
+      uint32_t ph = 1;   // (the first pass over the ring waits for nothing)
       for (int tile = blockIdx.x; tile < a.total_tiles; tile += gridDim.x) {
         int b, ti, tj;
         decode(tile, &b, &ti, &tj);
         const int row0 = a.meta[b * kMetaFields + kVisOff];
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int st = it % kGramStages;
-          if (it >= kGramStages && !twait(&empty[st], ((it / kGramStages) - 1) & 1)) continue;
+        for (int kb = 0; kb < nkb; ++kb) {
+          if (!twait(&empty[st], ph)) break;
           unsigned char *dst = smem + st * kGramStageBytes;
           mbar_expect_tx(&full[st], kGramStageBytes);
           tma_load_2d(dst, &a.tmap, kb * kGK, row0 + ti * kGM, &full[st]);
           tma_load_2d(dst + kGM * kGK * 2, &a.tmap, kb * kGK, row0 + tj * kGN, &full[st]);
           tma_load_2d(dst + 2 * kGM * kGK * 2, &a.tmap, kb * kGK, row0 + tj * kGN + 128, &full[st]);
+          if (++st == kGramStages) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
       }
-      // an aborted call: the last copies still land before the CTA may exit
-      if (*reinterpret_cast<volatile uint32_t *>(&tslot[1]))
-        for (uint32_t k = it > kGramStages ? it - kGramStages : 0; k < it; ++k)
-          mbar_wait_bounded(&full[k % kGramStages], (k / kGramStages) & 1, a.err, kErrTimeout);
+      // an aborted call: time for the last copies to land before the CTA may exit
+      if (dead)
+        for (int i = 0; i < 1 << 14; ++i) mbar_try_wait(&never, 0);
     }
   } else if (warp == 9) {
     if (lane == 0) {
       const uint32_t idesc = umma_idesc_bf16(kGM, kGN);
-      uint32_t it = 0, nc = 0;   // K blocks, accumulation chains
+      // the operands' descriptors: a stage further is kGramStageBytes, 16 elements 32 bytes
+      const uint64_t da = umma_desc_sw128(smem_addr(smem)), db = umma_desc_sw128(smem_addr(smem) + kGM * kGK * 2);
+      int st = 0;
+      uint32_t ph = 0, ab = 0, aph = 1;
       for (int tile = blockIdx.x; tile < a.total_tiles; tile += gridDim.x)
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int kc = kb % kGramChunkKb, ab = nc & 1;
-          if (kc == 0 && nc >= 2) twait(&aempty[ab], ((nc >> 1) - 1) & 1);
-          const int st = it % kGramStages;
-          const bool ok = twait(&full[st], (it / kGramStages) & 1);
-          tc_fence_after();
-          if (ok) {
-            const uint32_t sa = smem_addr(smem + st * kGramStageBytes);
+        for (int kb = 0; kb < nkb; kb += a.chunk_kb) {
+          const int end = min(kb + a.chunk_kb, nkb);
+          twait(&aempty[ab], aph);
+          for (int k = kb; k < end; ++k) {
+            const bool ok = twait(&full[st], ph);
+            tc_fence_after();
+            const uint64_t off = (uint64_t)(uint32_t)(st * (kGramStageBytes >> 4));
+            if (ok) {
 #pragma unroll
-            for (int k = 0; k < kGK / 16; ++k)
-              umma_bf16(tmem + ab * kGN, umma_desc_sw128(sa + k * 32),
-                        umma_desc_sw128(sa + kGM * kGK * 2 + k * 32), idesc, (kc | k) != 0 ? 1u : 0u);
+              for (int q = 0; q < kGK / 16; ++q)
+                umma_bf16(tmem + ab * kGN, da + off + 2 * q, db + off + 2 * q, idesc, (k != kb || q) ? 1u : 0u);
+            }
+            umma_commit(&empty[st]);
+            if (++st == kGramStages) {
+              st = 0;
+              ph ^= 1u;
+            }
           }
-          umma_commit(&empty[st]);
-          if (kc == kGramChunkKb - 1 || kb == nkb - 1) {
-            umma_commit(&afull[ab]);
-            ++nc;
-          }
+          umma_commit(&afull[ab]);
+          ab ^= 1u;
+          aph ^= ab ^ 1u;   // flips when the first accumulator comes round again
         }
     }
   } else {
@@ -225,7 +271,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
       float v[128];
 #pragma unroll
       for (int q = 0; q < 128; ++q) v[q] = 0.f;
-      for (int kb = 0; kb < nkb; kb += kGramChunkKb, ++nc) {
+      for (int kb = 0; kb < nkb; kb += a.chunk_kb, ++nc) {
         const int ab = nc & 1;
         twait(&afull[ab], (nc >> 1) & 1);
         __syncwarp();
@@ -242,41 +288,188 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
         __syncwarp();
         if (lane == 0) mbar_arrive(&aempty[ab]);
       }
-      const int32_t *m = a.meta + b * kMetaFields;
-      const int N = m[kNumVis], ld = gram_ld(N);
-      float *G = a.gram + (long long)m[kGramOff] * 32;
-      const int i = ti * kGM + 32 * quad + lane;
-      const int j0 = tj * kGN + half * 128;
       // the transposed 128 x 128 block too, unless a tile of its own computes it
-      const bool mirror = j0 / kGM < 2 * (ti / 2) && i < ld;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int j = j0 + 32 * c;
-        if (j < N) {
-          if (i < N) {
-            float *row = G + (long long)i * ld + j;
-#pragma unroll
-            for (int q = 0; q < 32; q += 8) st_global_v8(row + q, v + 32 * c + q);
-          }
-          if (mirror) {
-            float *col = G + (long long)j * ld + i;
-#pragma unroll
-            for (int q = 0; q < 32; ++q)
-              if (j + q < N) col[(long long)q * ld] = v[32 * c + q];
-          }
-        }
-      }
+      const int j0 = tj * kGN + half * 128;
+      store_tile(a, b, ti * kGM + 32 * quad + lane, j0, j0 / kGM < 2 * (ti / 2), v);
     }
   }
   __syncthreads();
   tc_fence_after();
   if (warp == 0) tmem_dealloc(tmem, 512);
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the norms too are done when this grid is
 }
 
-// 1/|x_i| in the canonical order, one warp per token.
+// The same tiles for a pair of CTAs (a cluster of two): 256 rows x 256 columns, each CTA
+// holding 128 rows of the accumulator and loading its half of either operand: 32 KB per
+// K block of 128 x 256 products instead of 48, into and out of a shared memory that the
+// single-CTA kernel saturates.  A stage holds two K blocks: handing a stage over costs
+// about 750 cycles however small it is (copies alone, 2 x 16384 tokens: 0.64 ms with one
+// K block a stage, 0.38 with two).  Copies and MMAs without the epilogue 0.59 ms, 1.86
+// PFLOP/s over the lower triangle (single CTA 0.78); with it 0.79 in chains of 1024
+// products, 0.91 of 512, 1.08 of 256 (single CTA 1.00 in one chain, 1.15 of 256): the
+// epilogue's stores only overlap the chains that fit in tensor memory.  Both kernels'
+// issuing threads keep the stage, its phase and the descriptors in registers: deriving
+// them from a counter took 3.47 instead of 2.99 ms on 8 requests of 16384.
+__global__ void __launch_bounds__(kGramThreads, 1) gram_pair_kernel(const __grid_constant__ GramArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned char *smem = reinterpret_cast<unsigned char *>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  // full, aempty: of the even CTA (its barriers count both CTAs); empty, afull: each CTA's
+  __shared__ unsigned long long full[kPairStages], empty[kPairStages], afull[2], aempty[2], never;
+  __shared__ uint32_t tslot;   // TMEM base
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)cluster_ctarank();
+  const int nkb = tc_kblocks(a.dv);
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kPairStages; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&afull[i], 1);
+      mbar_init(&aempty[i], 16);
+    }
+    mbar_init(&never, 1);
+    fence_mbar_init();
+  }
+  if (warp == 0) tmem_alloc_pair(&tslot, 512);
+  tc_fence_before();
+  cluster_sync();
+  tc_fence_after();
+  const uint32_t tmem = tslot;
+  bool dead = false;
+  auto twait = [&](unsigned long long *bar, uint32_t par) -> bool {
+    if (!dead && !mbar_wait_bounded(bar, par, a.err, kErrTimeout)) dead = true;
+    return !dead;
+  };
+  auto decode = [&](int tile, int *b_, int *ti, int *tj) {
+    int lo = 0, hi = a.B - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (a.tile0[mid] <= tile) lo = mid; else hi = mid - 1;
+    }
+    *b_ = lo;
+    int rem = tile - a.tile0[lo];
+    const int R = (a.meta[lo * kMetaFields + kNumVis] + kGN - 1) / kGN;
+    int g = 0;
+    while (8 * (g + 1) < R && rem >= 64 * g + 36) rem -= 64 * g++ + 36;   // whole groups
+    const int h = min(8, R - 8 * g);
+    if (rem < h * 8 * g) {
+      *tj = rem / h;
+      *ti = 8 * g + rem % h;
+    } else {
+      rem -= h * 8 * g;
+      int c = 0;
+      while (rem >= h - c) rem -= h - c++;
+      *tj = 8 * g + c;
+      *ti = 8 * g + c + rem;
+    }
+  };
+  const int tile_first = blockIdx.x >> 1, tile_step = gridDim.x >> 1;
+
+  if (warp == 8) {
+    if (lane == 0) {
+      int st = 0;
+      uint32_t ph = 1;   // (the first pass over the ring waits for nothing)
+      for (int tile = tile_first; tile < a.total_tiles; tile += tile_step) {
+        int b, ti, tj;
+        decode(tile, &b, &ti, &tj);
+        const int row0 = a.meta[b * kMetaFields + kVisOff] + 128 * rank;
+        for (int kb = 0; kb < nkb; kb += 2) {
+          if (!twait(&empty[st], ph)) break;
+          unsigned char *dst = smem + st * kPairStageBytes;
+          const uint32_t bar = map_shared(&full[st], 0);
+          if (rank == 0) mbar_expect_tx(&full[st], 2 * kPairStageBytes);
+          for (int y = 0; y < 2; ++y) {   // (columns past d_v land as zeros)
+            tma_load_2d_pair(dst + 2 * y * kGM * kGK * 2, &a.tmap, (kb + y) * kGK, row0 + ti * kGN, bar);
+            tma_load_2d_pair(dst + (2 * y + 1) * kGM * kGK * 2, &a.tmap, (kb + y) * kGK, row0 + tj * kGN, bar);
+          }
+          if (++st == kPairStages) {
+            st = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      // an aborted call: time for the last copies to land (their barrier may be the
+      // other CTA's) before the CTA may exit
+      if (dead)
+        for (int i = 0; i < 1 << 14; ++i) mbar_try_wait(&never, 0);
+    }
+  } else if (warp == 9) {
+    if (lane == 0 && rank == 0) {
+      const uint32_t idesc = umma_idesc_bf16(2 * kGM, kGN);
+      const uint64_t da = umma_desc_sw128(smem_addr(smem)), db = umma_desc_sw128(smem_addr(smem) + kGM * kGK * 2);
+      int st = 0;
+      uint32_t ph = 0, ab = 0, aph = 1;
+      for (int tile = tile_first; tile < a.total_tiles; tile += tile_step)
+        for (int kb = 0; kb < nkb; kb += a.chunk_kb) {
+          const int end = min(kb + a.chunk_kb, nkb);
+          twait(&aempty[ab], aph);
+          for (int k = kb; k < end; k += 2) {
+            const bool ok = twait(&full[st], ph);
+            tc_fence_after();
+            const uint64_t off = (uint64_t)(uint32_t)(st * (kPairStageBytes >> 4));
+            if (ok) {
+#pragma unroll
+              for (int q = 0; q < 2 * kGK / 16; ++q) {
+                const int at = (q / 4) * (2 * kGM * kGK * 2 >> 4) + 2 * (q % 4);
+                umma_bf16_pair(tmem + ab * kGN, da + off + at, db + off + at, idesc, (k != kb || q) ? 1u : 0u);
+              }
+            }
+            umma_commit_pair(&empty[st]);
+            if (++st == kPairStages) {
+              st = 0;
+              ph ^= 1u;
+            }
+          }
+          umma_commit_pair(&afull[ab]);
+          ab ^= 1u;
+          aph ^= ab ^ 1u;
+        }
+    }
+  } else {
+    const int half = warp >> 2, quad = warp & 3;
+    uint32_t nc = 0;
+    for (int tile = tile_first; tile < a.total_tiles; tile += tile_step) {
+      int b, ti, tj;
+      decode(tile, &b, &ti, &tj);
+      float v[128];
+#pragma unroll
+      for (int q = 0; q < 128; ++q) v[q] = 0.f;
+      for (int kb = 0; kb < nkb; kb += a.chunk_kb, ++nc) {
+        const int ab = nc & 1;
+        twait(&afull[ab], (nc >> 1) & 1);
+        __syncwarp();
+        tc_fence_after();
+        const uint32_t tb = tmem + ab * kGN + half * 128 + ((uint32_t)(32 * quad) << 16);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          uint32_t raw[16];
+          tmem_ld16(tb + 16 * c, raw);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) v[16 * c + q] = __fadd_rn(v[16 * c + q], __uint_as_float(raw[q]));
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(map_shared(&aempty[ab], 0));
+      }
+      store_tile(a, b, ti * kGN + 128 * rank + 32 * quad + lane, tj * kGN + half * 128, ti != tj, v);
+    }
+  }
+  __syncwarp();
+  tc_fence_before();
+  cluster_sync();   // both CTAs are done with either's barriers, operands and accumulators
+  tc_fence_after();
+  if (warp == 0) tmem_dealloc_pair(tmem, 512);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// 1/|x_i| in the canonical order, one warp per token: one read of X at the copy rate (24
+// us on 64 requests of 576 x 2048).  The Gram kernel starts beside it.
 template <typename T, int NCH>
 __global__ void __launch_bounds__(256) norms_kernel(const char *x, float *rn, int dv, int row_bytes,
                                                     long long total) {
+  asm volatile("griddepcontrol.launch_dependents;");
   const int lane = threadIdx.x & 31;
   const long long nw = (long long)gridDim.x * 8;
   for (long long t = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); t < total; t += nw) {
@@ -1046,17 +1239,35 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   void *sel_fn = nullptr, *norm_fn = nullptr;
   pick_nch<8>((pl.dv + 255) / 256, &sel_fn, &norm_fn);
 
-  // The largest clusters that still run every request at once, but no more CTAs than
-  // give each warp a block of tokens; when none does, the smallest that fits.
+  // The cluster size with the shortest schedule: requests go, most work first, to the
+  // next free cluster; a request takes about k / 16 + 2 rounds of 27K cycles, 4.6K more
+  // per block of 32 tokens that a warp holds and 0.4K per CTA (measured: 32K cycles a
+  // round on 576 tokens in two CTAs, 66K on 4096 in one, 42K on 16384 in twelve).
+  // Clusters of two instead of one: 2.88 -> 2.52 ms on 128 requests of 256..4096.
+  const int32_t *meta = pl.host_blob.data() + pl.off_meta / 4;
+  const int32_t *order = pl.host_blob.data() + pl.off_order / 4;
   SelShape sh;
-  const int cmax = std::min(kMaxCluster, std::max(1, (pl.max_vis + kGtok - 1) / kGtok));
-  for (int c = cmax; c >= 1; --c) {
+  double best = 0.0;
+  std::vector<double> busy;
+  for (int c = 1; c <= kMaxCluster; ++c) {
     const SelShape t = shape_for(c, pl.max_vis, optin);
     if (t.C == 0) continue;
     const int active = active_clusters(sel_fn, c, t.smem, kGthreads);
     if (active <= 0) continue;
-    sh = t;
-    if (active >= pl.B) break;
+    busy.assign(std::min(active, pl.B), 0.0);   // a heap, the next free cluster on top
+    double end = 0.0;
+    for (int i = 0; i < pl.B; ++i) {
+      const int32_t *m = meta + order[i] * kMetaFields;
+      const int slots = ((m[kNumVis] + 31) / 32 + c * kGwork - 1) / (c * kGwork);
+      std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
+      busy.back() += (m[kNumKeep] / 16.0 + 2.0) * (27.0 + 4.6 * slots + 0.4 * c);
+      end = std::max(end, busy.back());
+      std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+    }
+    if (sh.C == 0 || end < best) {
+      sh = t;
+      best = end;
+    }
   }
   if (sh.C == 0 || pl.max_vis > 0xffff) return cudaSuccess;   // too long for a cluster: the caller's other paths
 
@@ -1069,23 +1280,42 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   g.B = pl.B;
   g.dv = pl.dv;
   g.total_tiles = pl.gram_tiles;
+  const bool pair = gram_long(pl.max_vis);
+  const int chunk = gram_chunk(pl.max_vis);
+  g.chunk_kb = chunk / kGK;
   g.err = reinterpret_cast<unsigned *>(ws + pl.off_err);
   float *rn = reinterpret_cast<float *>(ws + pl.off_rn);
-  cudaError_t e;
-  {
+  cudaError_t e = cudaSuccess;
+  if (pl.gram_tiles > 0) {
     const char *xc = static_cast<const char *>(x);
     int dv = pl.dv, row = rb;
     long long total = pl.total_vis;
-    void *args[] = {&xc, &rn, &dv, &row, &total};
-    const int grid = (int)std::min<long long>((pl.total_vis + 7) / 8, (long long)sms * 8);
-    if ((e = cudaLaunchKernel(norm_fn, dim3(grid), dim3(256), args, 0, s)) != cudaSuccess) return e;
-  }
-  if (pl.gram_tiles > 0) {
-    const size_t smem = (size_t)kGramStages * kGramStageBytes + 1024;
-    e = cudaFuncSetAttribute(gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    void *nargs[] = {&xc, &rn, &dv, &row, &total};
+    const int ngrid = (int)std::min<long long>((pl.total_vis + 7) / 8, (long long)sms * 8);
+    if ((e = cudaLaunchKernel(norm_fn, dim3(ngrid), dim3(256), nargs, 0, s)) != cudaSuccess) return e;
+    // the matrix needs no norms: its kernel starts beside the norms' and ends after them
+    void *fn = pair ? (void *)gram_pair_kernel : (void *)gram_kernel;
+    const size_t smem = 192 * 1024 + 1024;
+    static_assert(kGramStages * kGramStageBytes == 192 * 1024 && kPairStages * kPairStageBytes == 192 * 1024,
+                  "the ring of either kernel");
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    gram_kernel<<<std::min(sms, pl.gram_tiles), kGramThreads, smem, s>>>(g);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(pair ? 2 * std::min(sms / 2, pl.gram_tiles) : std::min(sms, pl.gram_tiles));
+    cfg.blockDim = dim3(kGramThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = pair ? 2 : 1;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    void *args[] = {&g};
+    if ((e = cudaLaunchKernelExC(&cfg, fn, args)) != cudaSuccess) return e;
   }
   GramSelArgs a;
   std::memset(&a, 0, sizeof a);
@@ -1095,7 +1325,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   a.meta = g.meta;
   a.order = reinterpret_cast<const int32_t *>(ws + pl.off_order);
   a.dv = pl.dv; a.row_bytes = rb; a.csize = sh.C; a.mc = sh.mc; a.slots = sh.slots; a.words = sh.words;
-  a.eps = gram_distance_eps(pl.dv);
+  a.eps = gram_distance_eps(pl.dv, chunk);
   a.err = g.err;
   e = cudaFuncSetAttribute(sel_fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sel_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);

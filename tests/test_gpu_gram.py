@@ -1,5 +1,5 @@
 """The greedy from a Gram matrix (select_gram.cu) at the sizes where it can go wrong:
-around the 128-row and 256-column tiles and the 32-token blocks, one token more than
+around the 128-row and 256-column tiles (of one CTA and of pairs) and the 32-token blocks, one token more than
 the cluster's warps hold, feature widths that end inside a K block, every budget from
 one pick to all but one, exact ties, zero rows and rows outside the certificate's norm
 range.  Indices and rows are exact against the oracle."""
@@ -41,6 +41,7 @@ def _run(wl, x=None, w=None):
     ([1, 31, 33, 127, 129], [1, 30, 2, 64, 40]),
     ([255, 256, 257, 513], [254, 1, 100, 60]),
     ([545, 640, 2049], [100, 0, 130]),
+    ([8200, 90, 257], [60, 20, 60]),       # CTA pairs
 ])
 def test_selection_equals_the_oracle(n_vis, keep, d_v):
     wl = _wl(n_vis, keep, d_v)
