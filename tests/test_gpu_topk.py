@@ -152,3 +152,23 @@ def test_deterministic():
     a, xa = run_topk(wl, w32)
     b, xb = run_topk(wl, w32)
     assert np.array_equal(a, b) and np.array_equal(xa, xb)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 1025, 49153])
+@pytest.mark.parametrize("kind", ["close", "two_values", "signs"])
+def test_threshold_ties_and_shared_leading_bits(n, kind):
+    """Scores that share their leading bits, that are two values only (the threshold is a
+    long tie spread over the warps' parts) and of both signs with zeros."""
+    import torch
+    import paper_2607_27952_gb300 as last
+    rng = np.random.default_rng(n)
+    w = {"close": (1.0 + rng.integers(0, 4096, n) * 2.0 ** -20), "two_values": rng.integers(0, 2, n) + 1.0,
+         "signs": rng.integers(-3, 4, n) * 0.5}[kind].astype(np.float32)
+    w[w == 0.0] = rng.choice([0.0, -0.0], int((w == 0.0).sum()))
+    for k in sorted({1, max(1, n // 3), max(1, n - 1)}):
+        prob = last.Problem(batch=1, num_layers=0, num_q_heads=0, num_kv_heads=0, head_dim=0, feat_dim=8,
+                            dtype="bf16", cu_seqlens=None, vis_start=None, cu_vis=[0, n], cu_keep=[0, k])
+        idx = torch.full((k,), -7, dtype=torch.int32, device="cuda:0")
+        last.last_select_topk(prob, torch.from_numpy(w).cuda(), idx, last.workspace(prob, "cuda:0"))
+        want = np.sort(np.argsort(-w, kind="stable")[:k])
+        assert np.array_equal(idx.cpu().numpy(), want)
