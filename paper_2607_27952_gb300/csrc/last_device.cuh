@@ -292,6 +292,12 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const void *tmap, int x, 
                :: "r"(smem_addr(dst)), "l"(tmap), "r"(x), "r"(y), "r"(smem_addr(bar)) : "memory");
 }
 
+__device__ __forceinline__ void tma_load_3d(void *dst, const void *tmap, int x, int y, int z,
+                                            unsigned long long *bar) {
+  asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+               :: "r"(smem_addr(dst)), "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar)) : "memory");
+}
+
 // ---- CTA pairs (cta_group::2): both CTAs of a cluster of two run one MMA ----
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t *slot, uint32_t ncols) {   // one warp of each CTA
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"

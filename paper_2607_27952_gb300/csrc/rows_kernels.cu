@@ -6,21 +6,28 @@
 // rows, layers and q-heads at the visual positions and normalised (Eq. 8).  A
 // "column" is one (row, q-head of kv-head g) pair: G = Hq / Hkv columns per row.
 //
-// Four launches, all deterministic (fixed reduction orders, no float atomics):
-// rows_stats_kernel (request, 128-key chunk, layer, kv-head, 128-column tile):
-//   tcgen05.mma with the query columns as M and the chunk's keys as N (bf16, fp32
-//   accumulator in TMEM); thread t owns column t and takes, over its TMEM lane, the
-//   masked max of its logits (log2 domain) and the sums of 2^(z - max) over all and
-//   over the visual keys -- the chunk statistics of Eq. 6's softmax.
-// rows_merge_kernel (request): merges each column's chunk statistics in chunk
-//   order into (max, 1/Z) and the request's visual probability mass.
-// rows_probs_kernel (request, visual 128-key chunk, layer, kv-head): the same
-//   contraction with the keys as M; thread t owns key t and sums the probabilities
-//   2^(z - max) / Z over the columns (every column sees every visual key).
+// Four launches, all deterministic (fixed reduction orders, no float atomics).  The two
+// passes over K are one persistent kernel each (rows_pass_kernel): a TMA thread streams
+// (request, 128-key chunk, layer, kv-head) items, the keys' and the query columns' tiles
+// together, through a ring of stages; one thread issues tcgen05.mma with the keys as M
+// and the columns as N (bf16, fp32 accumulators in TMEM, one buffer per epilogue group);
+// groups of four warps take the finished items in turn, thread = key.
+// pass 1: per column the chunk's masked max of the logits (log2 domain) and the sums of
+//   2^(z - max) over all and over the visual keys (Eq. 6's softmax statistics), reduced
+//   over a warp's 32 keys for 32 columns at once (31 exchanges instead of 160);
+// rows_merge_kernel (request, 32 columns): the chunk statistics of each column into
+//   (max, 1/Z) and the columns' visual probability mass;
+// pass 2 (visual chunks): per key the probabilities 2^(z - max) / Z summed over the
+//   columns (every column sees every visual key);
 // rows_final_kernel (request, 256 visual tokens): adds the (layer, kv-head)
 //   partial sums and divides by the visual mass (Eq. 7-8).
+// The passes are bound by K's bytes and by the exponentials and exchanges of pass 1.
+// One CTA per item, staging by its own loads, spent 19 us of latency on each: 64 requests
+// of 576 tokens and 32 rows 369 us, 8 of 16384 456 us for the whole call; now
+// 140 us (88 + 38 in the passes; K read twice at the copy rate is 52) and 162 us.
 #include "last_device.cuh"
 #include "last_internal.h"
+#include "tensor_map.h"
 
 #include <algorithm>
 #include <cmath>
@@ -40,23 +47,27 @@ enum RowsField : int {
 };
 
 constexpr int kRowsChunk = 128;     // keys per CTA
-constexpr int kRowsThreads = 128;   // one thread per TMEM lane
 constexpr int kRowsMaxN = 256;      // columns (rows x G) per request
 constexpr int kRowsMaxRH = 6144;    // (row, layer, q-head) triples per request
 
+constexpr int kRowsGroups = 4;      // epilogue groups of four warps (two when npad > 128)
+constexpr int kPassThreads = 32 * (4 * kRowsGroups + 2);
+constexpr int kRowsMaxStages = 8;
+
 struct RowsArgs {
-  const __nv_bfloat16 *q, *k;
+  CUtensorMap kmap;      // K as [L * total_keys][Hkv * D], box 64 x 128, 128-byte swizzle
+  CUtensorMap qmap;      // q as [rows][L * Hq][D], box 64 x G x qbox
   const int32_t *meta;
   const int2 *items1, *items2;
   const int32_t *row_pos;
-  float4 *stats;         // per column-layer-head triple x chunk: max, sum, visual sum
-  float2 *coef;          // per triple: max, 1 / Z
-  float *inv_total;      // per request: 1 / visual mass
+  float4 *stats;         // per request [chunk][row, layer, head]: max, sum, visual sum
+  float2 *coef;          // per (row, layer, head): max, 1 / Z
+  float *mass;           // per request and block of 32 such triples: visual mass
   float *partial;        // [L][Hkv][total_vis] probability sums
   float *w;
   long long total_keys, total_vis;
-  int L, Hq, Hkv, D, G, npad;
-  uint32_t tmem_stats, tmem_probs;
+  int L, Hq, Hkv, D, G, npad, qbox, n_items, nstage, ngroup, mass_blocks;
+  uint32_t tmem_cols;    // TMEM columns of one group's accumulator
   float qscale;          // softmax scale * log2(e)
   unsigned *err;
 };
@@ -65,243 +76,309 @@ __device__ __forceinline__ long long stat_base(const int32_t *m) {
   return *reinterpret_cast<const long long *>(m + kRStatBase);
 }
 
-// 16-byte chunk j of row `row` of a K-major operand with 128-byte rows and the
-// 128-byte swizzle; K blocks of `rows` rows each.
-__device__ __forceinline__ unsigned char *sw128_chunk(unsigned char *base, int rows, int row, int j) {
-  return base + (j >> 3) * (rows * 128) + row * 128 + (((j & 7) ^ (row & 7)) << 4);
-}
-
-// Keys c*128 .. c*128+127 of kv-head g (zero past P) into a 128-row operand.
-__device__ __forceinline__ void stage_keys(unsigned char *dst, const RowsArgs &a, int seq0, int P,
-                                           int c, int l, int g) {
-  const int t = threadIdx.x, p = c * kRowsChunk + t;
-  const __nv_bfloat16 *src = a.k + (((long long)l * a.total_keys + seq0 + p) * a.Hkv + g) * a.D;
-  for (int j = 0; j < a.D / 8; ++j)
-    *reinterpret_cast<U4 *>(sw128_chunk(dst, kRowsChunk, t, j)) =
-        p < P ? ldg(src + 8 * j) : U4{0, 0, 0, 0};
-}
-
-// Query columns n0 .. n0+rows-1 (row n / G, q-head g*G + n % G; zero past ncol).
-__device__ __forceinline__ void stage_queries(unsigned char *dst, const RowsArgs &a, int rows,
-                                              int n0, int ncol, int row0, int l, int g) {
-  for (int idx = threadIdx.x; idx < rows * (a.D / 8); idx += kRowsThreads) {
-    const int i = idx / (a.D / 8), j = idx - i * (a.D / 8), n = n0 + i;
-    U4 v = U4{0, 0, 0, 0};
-    if (n < ncol) {
-      const int r = n / a.G, gg = n - r * a.G;
-      v = ldg(a.q + (((long long)(row0 + r) * a.L + l) * a.Hq + g * a.G + gg) * a.D + 8 * j);
-    }
-    *reinterpret_cast<U4 *>(sw128_chunk(dst, rows, i, j)) = v;
-  }
-}
-
-// D[tmem] = A[128 x D] * B[n x D]^T over D / 64 K blocks, one thread; completion on bar.
-__device__ __forceinline__ void rows_mma(uint32_t tmem, unsigned char *A, unsigned char *B, int n,
-                                         int nkb, unsigned long long *bar) {
-  const uint32_t idesc = umma_idesc_bf16(kRowsChunk, n);
-  for (int kb = 0; kb < nkb; ++kb)
+// 32 values per lane, one per column, reduced over the warp's lanes: lane c ends with
+// column c.  At each step a lane keeps the half of the columns its bit selects.
+template <typename F>
+__device__ __forceinline__ float warp_columns(float *v, int lane, F op) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      umma_bf16(tmem, umma_desc_sw128(smem_addr(A + kb * (kRowsChunk * 128)) + k * 32),
-                umma_desc_sw128(smem_addr(B + kb * (n * 128)) + k * 32), idesc, (kb | k) != 0 ? 1u : 0u);
-  umma_commit(bar);
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < o; ++q) {
+      const float send = (lane & o) ? v[q] : v[q + o];
+      const float keep = (lane & o) ? v[q + o] : v[q];
+      v[q] = op(keep, __shfl_xor_sync(0xffffffffu, send, o));
+    }
+  return v[0];
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(kRowsThreads)
-rows_stats_kernel(const RowsArgs a) {
-  const int2 item = a.items1[blockIdx.x];
-  const int b = item.x, c = item.y, l = blockIdx.y;
-  const int g = blockIdx.z % a.Hkv, mt = blockIdx.z / a.Hkv;
-  const int32_t *m = a.meta + b * kRowsFields;
-  const int ncol = m[kRNumRows] * a.G;
-  if (mt * kRowsThreads >= ncol) return;   // the whole CTA leaves before any allocation
+template <bool STATS>
+__global__ void __launch_bounds__(kPassThreads, 1) rows_pass_kernel(const __grid_constant__ RowsArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int nkb = a.D / 64;
-  unsigned char *sQ = smem, *sK = smem + nkb * (kRowsChunk * 128);
-  unsigned long long *bar = reinterpret_cast<unsigned long long *>(sK + nkb * (kRowsChunk * 128));
-  uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 1);
-  const int seq0 = m[kRSeqStart], P = m[kRSeqLen], v0 = m[kRVisStart], nvis = m[kRNumVis];
-  const int row0 = m[kRRowOff], nch = m[kRNumChunks];
-  const int t = threadIdx.x, warp = t >> 5;
-
-  if (t == 0) {
-    mbar_init(bar, 1);
+  __shared__ unsigned long long full[kRowsMaxStages], empty[kRowsMaxStages];
+  __shared__ unsigned long long afull[kRowsGroups], aempty[kRowsGroups], never;
+  __shared__ uint32_t tslot;
+  __shared__ float4 part[kRowsGroups][4][32];   // pass 1: the warps' statistics of 32 columns
+  __shared__ float2 cf[kRowsGroups][kRowsMaxN]; // pass 2: the item's (max, 1 / Z)
+  __shared__ float bmax[kRowsGroups * 4][32];   // pass 1: a warp's column maxima
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nkb = a.D / 64, ngroup = a.ngroup;
+  const int kbytes = nkb * kRowsChunk * 128, qbytes = nkb * a.npad * 128, stage_bytes = kbytes + qbytes;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < a.nstage; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
+    }
+    for (int i = 0; i < ngroup; ++i) {
+      mbar_init(&afull[i], 1);
+      mbar_init(&aempty[i], 4);
+    }
+    mbar_init(&never, 1);
     fence_mbar_init();
   }
-  if (warp == 0) tmem_alloc(tslot, a.tmem_stats);
-  stage_queries(sQ, a, kRowsThreads, mt * kRowsThreads, ncol, row0, l, g);
-  stage_keys(sK, a, seq0, P, c, l, g);
-  fence_proxy_async_smem();
+  const uint32_t tmem_total = a.tmem_cols * (uint32_t)ngroup;
+  if (warp == 0) tmem_alloc(&tslot, tmem_total);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot;
-  if (t == 0) rows_mma(tmem, sQ, sK, kRowsChunk, nkb, bar);
-  __syncwarp();
-  mbar_wait_bounded(bar, 0, a.err, kErrTimeout);
-  tc_fence_after();
+  const uint32_t tmem = tslot;
+  bool dead = false;   // after one expired wait a role's others return at once
+  auto twait = [&](unsigned long long *bar, uint32_t par) -> bool {
+    if (!dead && !mbar_wait_bounded(bar, par, a.err, kErrTimeout)) dead = true;
+    return !dead;
+  };
+  const int2 *items = STATS ? a.items1 : a.items2;
+  // item -> (request, chunk), layer, kv-head; heads fastest, so that CTAs running side by
+  // side read neighbouring bytes of the same keys
+  auto decode = [&](int item, int *b, int *c, int *l, int *g) {
+    const int hl = a.Hkv * a.L, it = item / hl, r = item - it * hl;
+    const int2 v = items[it];
+    *b = v.x;
+    *c = v.y;
+    *l = r / a.Hkv;
+    *g = r - *l * a.Hkv;
+  };
 
-  // column n: its row's position bounds the keys it sees
-  const int n = mt * kRowsThreads + t;
-  const bool col_ok = n < ncol;
-  const int r = col_ok ? n / a.G : 0;
-  const int pos = col_ok ? a.row_pos[row0 + r] : -1;
-  const uint32_t lane_addr = tmem + ((uint32_t)(32 * warp) << 16);
-  const int p0 = c * kRowsChunk;
-  float mx = -INFINITY;
-  for (int j0 = 0; j0 < kRowsChunk; j0 += 16) {
-    uint32_t raw[16];
-    tmem_ld16(lane_addr + (uint32_t)j0, raw);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int p = p0 + j0 + j;
-      if (p < P && p <= pos) mx = fmaxf(mx, __uint_as_float(raw[j]) * a.qscale);
+  if (warp == 4 * kRowsGroups) {
+    if (lane == 0) {
+      int st = 0;
+      uint32_t ph = 1;
+      for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
+        int b, c, l, g;
+        decode(item, &b, &c, &l, &g);
+        const int32_t *m = a.meta + b * kRowsFields;
+        const int key0 = (int)((long long)l * a.total_keys) + m[kRSeqStart] + c * kRowsChunk;
+        if (!twait(&empty[st], ph)) break;
+        unsigned char *dst = smem + (size_t)st * stage_bytes;
+        mbar_expect_tx(&full[st], (uint32_t)(kbytes + nkb * a.G * a.qbox * 128));
+        for (int kb = 0; kb < nkb; ++kb) {
+          tma_load_2d(dst + kb * kRowsChunk * 128, &a.kmap, g * a.D + 64 * kb, key0, &full[st]);
+          tma_load_3d(dst + kbytes + kb * a.npad * 128, &a.qmap, 64 * kb, l * a.Hq + g * a.G, m[kRRowOff],
+                      &full[st]);
+        }
+        if (++st == a.nstage) {
+          st = 0;
+          ph ^= 1u;
+        }
+      }
+      // an aborted call: time for the last copies to land before the CTA may exit
+      if (dead)
+        for (int i = 0; i < 1 << 14; ++i) mbar_try_wait(&never, 0);
     }
-  }
-  // (a column with no visible key in this chunk keeps max = -inf and adds nothing;
-  // the TMEM loads stay warp-uniform)
-  float sum = 0.f, vis = 0.f;
-  for (int j0 = 0; j0 < kRowsChunk; j0 += 16) {
-    uint32_t raw[16];
-    tmem_ld16(lane_addr + (uint32_t)j0, raw);
+  } else if (warp == 4 * kRowsGroups + 1) {
+    if (lane == 0) {
+      const uint32_t idesc = umma_idesc_bf16(kRowsChunk, a.npad);
+      int st = 0, gr = 0;
+      uint32_t ph = 0, gph = 1;
+      for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
+        twait(&aempty[gr], gph);
+        const bool ok = twait(&full[st], ph);
+        tc_fence_after();
+        if (ok) {
+          const uint32_t sk = smem_addr(smem + (size_t)st * stage_bytes), sq = sk + kbytes;
+          for (int kb = 0; kb < nkb; ++kb)
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int p = p0 + j0 + j;
-      if (p < P && p <= pos) {
-        const float e = exp2f(__uint_as_float(raw[j]) * a.qscale - mx);
-        sum += e;
-        if (p >= v0 && p < v0 + nvis) vis += e;
+            for (int k = 0; k < 4; ++k)
+              umma_bf16(tmem + gr * a.tmem_cols, umma_desc_sw128(sk + kb * kRowsChunk * 128 + k * 32),
+                        umma_desc_sw128(sq + kb * a.npad * 128 + k * 32), idesc, (kb | k) != 0 ? 1u : 0u);
+        }
+        umma_commit(&empty[st]);
+        umma_commit(&afull[gr]);
+        if (++st == a.nstage) {
+          st = 0;
+          ph ^= 1u;
+        }
+        if (++gr == ngroup) {
+          gr = 0;
+          gph ^= 1u;
+        }
       }
     }
-  }
-  if (col_ok) {
-    const int h = g * a.G + (n - r * a.G);
-    const long long rh = ((long long)r * a.L + l) * a.Hq + h;
-    a.stats[stat_base(m) + rh * nch + c] = make_float4(mx, sum, vis, 0.f);
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, a.tmem_stats);
-}
-
-__global__ void __launch_bounds__(1024)
-rows_merge_kernel(const RowsArgs a) {
-  __shared__ float red[32];
-  const int b = blockIdx.x;
-  const int32_t *m = a.meta + b * kRowsFields;
-  const int RH = m[kRNumRows] * a.L * a.Hq, nch = m[kRNumChunks], cb = m[kRCoefBase];
-  const float4 *stats = a.stats + stat_base(m);
-  float vis_mass = 0.f;
-  for (int rh = threadIdx.x; rh < RH; rh += blockDim.x) {
-    const float4 *st = stats + (long long)rh * nch;
-    float mx = -INFINITY;
-    for (int c = 0; c < nch; ++c) mx = fmaxf(mx, st[c].x);
-    float z = 0.f, vz = 0.f;
-    for (int c = 0; c < nch; ++c) {
-      const float4 v = st[c];
-      const float f = v.x == -INFINITY ? 0.f : exp2f(v.x - mx);   // chunks past the row
-      z += v.y * f;
-      vz += v.z * f;
+  } else if (warp < 4 * ngroup) {
+    const int gr = warp >> 2, quad = warp & 3, gt = threadIdx.x & 127;   // group, its warp, its thread
+    uint32_t ph = 0;
+    for (int item = blockIdx.x + gr * gridDim.x; item < a.n_items; item += ngroup * gridDim.x, ph ^= 1u) {
+      int b, c, l, g;
+      decode(item, &b, &c, &l, &g);
+      const int32_t *m = a.meta + b * kRowsFields;
+      const int P = m[kRSeqLen], v0 = m[kRVisStart], v1 = v0 + m[kRNumVis], row0 = m[kRRowOff];
+      const int ncol = m[kRNumRows] * a.G, p0 = c * kRowsChunk, p = p0 + gt;
+      // rows sit after the visual span: keys up to its end are seen by every row
+      const bool seen = p0 + kRowsChunk <= v1, in_vis = p >= v0 && p < v1;
+      const uint32_t acc = tmem + gr * a.tmem_cols + ((uint32_t)(32 * quad) << 16);
+      const long long rh0 = (long long)l * a.Hq + g * a.G;   // triple of (row 0, l, first head of g)
+      if (!STATS) {
+        for (int n = gt; n < ncol; n += 128) {
+          const int r = n / a.G;
+          cf[gr][n] = a.coef[m[kRCoefBase] + (long long)r * a.L * a.Hq + rh0 + (n - r * a.G)];
+        }
+        asm volatile("bar.sync %0, 128;" :: "r"(1 + gr) : "memory");
+      }
+      twait(&afull[gr], ph);
+      __syncwarp();
+      tc_fence_after();
+      if constexpr (STATS) {
+        float4 *st = a.stats + stat_base(m) + (long long)c * m[kRNumRows] * a.L * a.Hq;
+        for (int n0 = 0; n0 < ncol; n0 += 32) {
+          float z[32], t[32];
+          {
+            uint32_t raw[32];
+            tmem_ld16(acc + n0, raw);
+            if (n0 + 16 < a.npad) tmem_ld16(acc + n0 + 16, raw + 16);
+#pragma unroll
+            for (int q = 0; q < 32; ++q) z[q] = __uint_as_float(raw[q]) * a.qscale;
+          }
+          if (!seen) {   // causal mask of the text rows, keys past the request
+#pragma unroll
+            for (int q = 0; q < 32; ++q) {
+              const int pos = n0 + q < ncol ? a.row_pos[row0 + (n0 + q) / a.G] : -1;
+              if (p >= P || p > pos) z[q] = -INFINITY;
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < 32; ++q) t[q] = z[q];
+          const float mx = warp_columns(t, lane, [](float x, float y) { return fmaxf(x, y); });
+          bmax[warp][lane] = mx;
+          __syncwarp();
+#pragma unroll
+          for (int q = 0; q < 32; ++q) {
+            const float mq = bmax[warp][q];
+            z[q] = seen || z[q] != -INFINITY ? exp2f(z[q] - mq) : 0.f;
+            t[q] = z[q];
+          }
+          __syncwarp();
+          const float sum = warp_columns(t, lane, [](float x, float y) { return x + y; });
+          float vis;
+          const int wp0 = p0 + 32 * quad;   // the warp's keys
+          if (wp0 >= v0 && wp0 + 32 <= v1) {
+            vis = sum;
+          } else if (wp0 + 32 <= v0 || wp0 >= v1) {
+            vis = 0.f;
+          } else {
+#pragma unroll
+            for (int q = 0; q < 32; ++q) t[q] = in_vis ? z[q] : 0.f;
+            vis = warp_columns(t, lane, [](float x, float y) { return x + y; });
+          }
+          part[gr][quad][lane] = make_float4(mx, sum, vis, 0.f);
+          asm volatile("bar.sync %0, 128;" :: "r"(1 + gr) : "memory");
+          if (quad == 0 && n0 + lane < ncol) {   // the four warps in order
+            const float4 x0 = part[gr][0][lane], x1 = part[gr][1][lane], x2 = part[gr][2][lane],
+                         x3 = part[gr][3][lane];
+            const float mm = fmaxf(fmaxf(x0.x, x1.x), fmaxf(x2.x, x3.x));
+            float s4 = 0.f, vv = 0.f;
+            const float4 xs[4] = {x0, x1, x2, x3};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const float f = xs[q].x == -INFINITY ? 0.f : exp2f(xs[q].x - mm);
+              s4 += xs[q].y * f;
+              vv += xs[q].z * f;
+            }
+            const int n = n0 + lane, r = n / a.G;
+            st[(long long)r * a.L * a.Hq + rh0 + (n - r * a.G)] = make_float4(mm, s4, vv, 0.f);
+          }
+          asm volatile("bar.sync %0, 128;" :: "r"(1 + gr) : "memory");
+        }
+      } else {
+        float s0 = 0.f, s1 = 0.f;
+        for (int n0 = 0; n0 < ncol; n0 += 16) {
+          uint32_t raw[16];
+          tmem_ld16(acc + n0, raw);
+          if (n0 + 16 <= ncol) {
+#pragma unroll
+            for (int j = 0; j < 16; j += 2) {
+              const float2 c0 = cf[gr][n0 + j], c1 = cf[gr][n0 + j + 1];
+              s0 += exp2f(__uint_as_float(raw[j]) * a.qscale - c0.x) * c0.y;
+              s1 += exp2f(__uint_as_float(raw[j + 1]) * a.qscale - c1.x) * c1.y;
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (n0 + j < ncol) s0 += exp2f(__uint_as_float(raw[j]) * a.qscale - cf[gr][n0 + j].x) * cf[gr][n0 + j].y;
+          }
+        }
+        if (in_vis) a.partial[((long long)l * a.Hkv + g) * a.total_vis + m[kRVisOff] + (p - v0)] = s0 + s1;
+        asm volatile("bar.sync %0, 128;" :: "r"(1 + gr) : "memory");   // cf is rewritten next
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&aempty[gr]);
     }
-    a.coef[cb + rh] = make_float2(mx, 1.0f / z);
-    vis_mass += vz / z;
   }
-  // fixed-tree block sum of the visual masses
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) vis_mass += __shfl_xor_sync(0xffffffffu, vis_mass, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = vis_mass;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    float v = threadIdx.x < (int)(blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) a.inv_total[b] = 1.0f / v;
-  }
-}
-
-__global__ void __launch_bounds__(kRowsThreads)
-rows_probs_kernel(const RowsArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char *smem = reinterpret_cast<unsigned char *>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int nkb = a.D / 64, npad = a.npad;
-  unsigned char *sK = smem, *sQ = smem + nkb * (kRowsChunk * 128);
-  float2 *cf = reinterpret_cast<float2 *>(sQ + nkb * (npad * 128));
-  unsigned long long *bar = reinterpret_cast<unsigned long long *>(cf + kRowsMaxN);
-  uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 1);
-  const int2 item = a.items2[blockIdx.x];
-  const int b = item.x, c = item.y, l = blockIdx.y, g = blockIdx.z;
-  const int32_t *m = a.meta + b * kRowsFields;
-  const int seq0 = m[kRSeqStart], P = m[kRSeqLen], v0 = m[kRVisStart], nvis = m[kRNumVis];
-  const int voff = m[kRVisOff], row0 = m[kRRowOff], ncol = m[kRNumRows] * a.G;
-  const int cb = m[kRCoefBase];
-  const int t = threadIdx.x, warp = t >> 5;
-
-  if (t == 0) {
-    mbar_init(bar, 1);
-    fence_mbar_init();
-  }
-  if (warp == 0) tmem_alloc(tslot, a.tmem_probs);
-  stage_keys(sK, a, seq0, P, c, l, g);
-  stage_queries(sQ, a, npad, 0, ncol, row0, l, g);
-  for (int n = t; n < ncol; n += kRowsThreads) {
-    const int r = n / a.G, h = g * a.G + (n - r * a.G);
-    cf[n] = a.coef[cb + ((long long)r * a.L + l) * a.Hq + h];
-  }
-  fence_proxy_async_smem();
-  tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot;
-  if (t == 0) rows_mma(tmem, sK, sQ, npad, nkb, bar);
-  __syncwarp();
-  mbar_wait_bounded(bar, 0, a.err, kErrTimeout);
-  tc_fence_after();
+  if (warp == 0) tmem_dealloc(tmem, tmem_total);
+}
 
-  const int p = c * kRowsChunk + t;
-  float s0 = 0.f, s1 = 0.f;
-  for (int n0 = 0; n0 < ncol; n0 += 16) {
-    uint32_t raw[16];
-    tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)n0, raw);
-#pragma unroll
-    for (int j = 0; j < 16; j += 2) {
-      if (n0 + j < ncol)
-        s0 += exp2f(__uint_as_float(raw[j]) * a.qscale - cf[n0 + j].x) * cf[n0 + j].y;
-      if (n0 + j + 1 < ncol)
-        s1 += exp2f(__uint_as_float(raw[j + 1]) * a.qscale - cf[n0 + j + 1].x) * cf[n0 + j + 1].y;
-    }
-  }
-  // every column's row sits after the visual span, so each visual key is unmasked
-  if (p >= v0 && p < v0 + nvis && p < P)
-    a.partial[((long long)l * a.Hkv + g) * a.total_vis + voff + (p - v0)] = s0 + s1;
-  tc_fence_before();
+// One CTA per (32 (row, layer, head) triples, request): 8 warps take the chunks in turn,
+// lane = triple, then the warps' results are merged in order.
+__global__ void __launch_bounds__(256) rows_merge_kernel(const RowsArgs a) {
+  __shared__ float4 part[8][32];
+  const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int32_t *m = a.meta + b * kRowsFields;
+  const int RH = m[kRNumRows] * a.L * a.Hq, nch = m[kRNumChunks];
+  if ((int)blockIdx.x * 32 >= RH) return;
+  const int rh = blockIdx.x * 32 + lane;
+  const float4 *st = a.stats + stat_base(m) + min(rh, RH - 1);
+  float mx = -INFINITY, z = 0.f, vz = 0.f;
+  auto add = [&](const float4 &v) {   // running (max, sums); chunks past the row hold -inf
+    const float nm = fmaxf(mx, v.x);
+    const float f = v.x == -INFINITY ? 0.f : exp2f(v.x - nm);
+    const float o = mx == -INFINITY ? 0.f : exp2f(mx - nm);
+    z = z * o + v.y * f;
+    vz = vz * o + v.z * f;
+    mx = nm;
+  };
+  for (int c = warp; c < nch; c += 8) add(st[(long long)c * RH]);
+  part[warp][lane] = make_float4(mx, z, vz, 0.f);
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, a.tmem_probs);
+  if (warp != 0) return;
+  mx = -INFINITY;
+  z = vz = 0.f;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) add(part[q][lane]);
+  float mass = 0.f;
+  if (rh < RH) {
+    a.coef[m[kRCoefBase] + rh] = make_float2(mx, 1.0f / z);
+    mass = vz / z;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mass += __shfl_xor_sync(0xffffffffu, mass, o);
+  if (lane == 0) a.mass[(long long)b * a.mass_blocks + blockIdx.x] = mass;
 }
 
 __global__ void __launch_bounds__(kScoreThreads)
 rows_final_kernel(const RowsArgs a) {
+  __shared__ float inv_s;
   const int b = blockIdx.y;
   const int32_t *m = a.meta + b * kRowsFields;
+  if ((int)blockIdx.x * kScoreThreads >= m[kRNumVis]) return;
+  if (threadIdx.x < 32) {   // the request's visual mass: the blocks over the lanes, a fixed tree
+    const int nb = (m[kRNumRows] * a.L * a.Hq + 31) / 32;
+    float t = 0.f;
+    for (int q = threadIdx.x; q < nb; q += 32) t += a.mass[(long long)b * a.mass_blocks + q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) inv_s = 1.0f / t;
+  }
+  __syncthreads();
   const int i = blockIdx.x * kScoreThreads + threadIdx.x;
   if (i >= m[kRNumVis]) return;
   const long long tok = m[kRVisOff] + i;
   float s = 0.f;
   for (int lg = 0; lg < a.L * a.Hkv; ++lg) s += a.partial[(long long)lg * a.total_vis + tok];
-  a.w[tok] = s * a.inv_total[b];
+  a.w[tok] = s * inv_s;
 }
 
 namespace {
 
 struct RowsPlan {
-  int B = 0, L = 0, Hq = 0, Hkv = 0, D = 0, G = 0, npad = 0, mtiles = 0, max_vis = 0;
+  int B = 0, L = 0, Hq = 0, Hkv = 0, D = 0, G = 0, npad = 0, max_vis = 0, mass_blocks = 0;
   long long total_keys = 0, total_vis = 0, total_rows = 0, n_items1 = 0, n_items2 = 0;
   size_t off_meta = 0, off_items1 = 0, off_items2 = 0, off_pos = 0, blob_bytes = 0;
-  size_t off_stats = 0, off_coef = 0, off_inv = 0, off_partial = 0, total_bytes = 0;
+  size_t off_stats = 0, off_coef = 0, off_mass = 0, off_partial = 0, total_bytes = 0;
   std::vector<int32_t> blob;
   float scale = 0.f;
 };
@@ -358,6 +435,7 @@ last_status make_rows_plan(const last_problem *p, const int32_t *cu_rows, const 
     const int nch = (P + kRowsChunk - 1) / kRowsChunk;
     stats += rh * nch;
     rh_total += rh;
+    pl->mass_blocks = std::max(pl->mass_blocks, (int)((rh + 31) / 32));
     pl->n_items1 += nch;
     if (N > 0)
       pl->n_items2 += (p->vis_start[b] + N - 1) / kRowsChunk - p->vis_start[b] / kRowsChunk + 1;
@@ -367,7 +445,6 @@ last_status make_rows_plan(const last_problem *p, const int32_t *cu_rows, const 
     return rows_fail(LAST_ERR_UNSUPPORTED, "query rows x (num_q_heads / num_kv_heads) must be <= 256");
   if (rh_total > 0x7fffffffLL) return rows_fail(LAST_ERR_UNSUPPORTED, "too many query rows in all");
   pl->npad = std::max(16, (max_cols + 15) / 16 * 16);
-  pl->mtiles = (max_cols + kRowsThreads - 1) / kRowsThreads;
   pl->total_keys = p->cu_seqlens[B];
   pl->total_vis = p->cu_vis[B];
   pl->total_rows = cu_rows[B];
@@ -385,8 +462,8 @@ last_status make_rows_plan(const last_problem *p, const int32_t *cu_rows, const 
   o = alignr(o + sizeof(float) * 4 * (size_t)std::max<long long>(stats, 1));
   pl->off_coef = o;
   o = alignr(o + sizeof(float) * 2 * (size_t)std::max<long long>(rh_total, 1));
-  pl->off_inv = o;
-  o = alignr(o + sizeof(float) * std::max(B, 1));
+  pl->off_mass = o;
+  o = alignr(o + sizeof(float) * (size_t)std::max(B, 1) * pl->mass_blocks);
   pl->off_partial = o;
   o = alignr(o + sizeof(float) * (size_t)pl->L * pl->Hkv * (size_t)std::max<long long>(pl->total_vis, 1));
   pl->total_bytes = o;
@@ -429,14 +506,6 @@ last_status make_rows_plan(const last_problem *p, const int32_t *cu_rows, const 
   }
   for (long long r = 0; r < pl->total_rows; ++r) pos[r] = row_pos[r];
   return LAST_OK;
-}
-
-// Dynamic shared memory of a 128-thread kernel holding `cols` TMEM columns: the
-// operands, and at least enough that at most 512 / cols CTAs share an SM, so every
-// CTA's TMEM allocation is granted at once.
-size_t tmem_safe_smem(size_t operands, uint32_t cols) {
-  const size_t per_sm = 228 * 1024;
-  return std::max(operands, per_sm / (512 / cols + 1) + 1);
 }
 
 // One query row per request: the row at position pos attends keys 0 .. pos, which
@@ -507,49 +576,66 @@ extern "C" last_status last_scores_rows(const last_problem *p, const int32_t *cu
   if (pl.total_vis == 0 || pl.B == 0) return LAST_OK;
 
   RowsArgs a;
-  a.q = static_cast<const __nv_bfloat16 *>(q_rows);
-  a.k = static_cast<const __nv_bfloat16 *>(k);
+  std::memset(&a, 0, sizeof a);
   a.meta = reinterpret_cast<const int32_t *>(wsc + pl.off_meta);
   a.items1 = reinterpret_cast<const int2 *>(wsc + pl.off_items1);
   a.items2 = reinterpret_cast<const int2 *>(wsc + pl.off_items2);
   a.row_pos = reinterpret_cast<const int32_t *>(wsc + pl.off_pos);
   a.stats = reinterpret_cast<float4 *>(wsc + pl.off_stats);
   a.coef = reinterpret_cast<float2 *>(wsc + pl.off_coef);
-  a.inv_total = reinterpret_cast<float *>(wsc + pl.off_inv);
+  a.mass = reinterpret_cast<float *>(wsc + pl.off_mass);
   a.partial = reinterpret_cast<float *>(wsc + pl.off_partial);
   a.w = w_out;
   a.total_keys = pl.total_keys;
   a.total_vis = pl.total_vis;
   a.L = pl.L; a.Hq = pl.Hq; a.Hkv = pl.Hkv; a.D = pl.D; a.G = pl.G; a.npad = pl.npad;
-  a.tmem_stats = 128;
-  uint32_t tp = 32;
-  while ((int)tp < pl.npad) tp *= 2;
-  a.tmem_probs = tp;
+  a.mass_blocks = pl.mass_blocks;
+  uint32_t cols = 32;
+  while ((int)cols < pl.npad) cols *= 2;
+  a.tmem_cols = cols;
+  a.ngroup = (int)std::min<uint32_t>(kRowsGroups, 512 / cols);
+  a.qbox = std::min(pl.npad / pl.G, 256);
   a.qscale = pl.scale * 1.4426950408889634f;
   a.err = reinterpret_cast<unsigned *>(wsc);
   auto fail_launch = [](cudaError_t err, const char *what) {
     return rows_fail(LAST_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(err));
   };
-
-  const int nkb = pl.D / 64;
-  const size_t op = 1024 + (size_t)2 * nkb * kRowsChunk * 128 + 64;
-  const size_t smem1 = tmem_safe_smem(op, a.tmem_stats);
-  if ((e = cudaFuncSetAttribute(rows_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem1)) != cudaSuccess)
-    return fail_launch(e, "rows stats");
-  rows_stats_kernel<<<dim3((unsigned)pl.n_items1, pl.L, pl.Hkv * pl.mtiles), kRowsThreads, smem1, s>>>(a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return fail_launch(e, "rows stats launch");
-  rows_merge_kernel<<<pl.B, 1024, 0, s>>>(a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return fail_launch(e, "rows merge launch");
-  if (pl.n_items2 > 0) {
-    const size_t op2 = 1024 + (size_t)nkb * kRowsChunk * 128 + (size_t)nkb * pl.npad * 128 +
-                       sizeof(float2) * kRowsMaxN + 64;
-    const size_t smem2 = tmem_safe_smem(op2, a.tmem_probs);
-    if ((e = cudaFuncSetAttribute(rows_probs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem2)) != cudaSuccess)
-      return fail_launch(e, "rows probs");
-    rows_probs_kernel<<<dim3((unsigned)pl.n_items2, pl.L, pl.Hkv), kRowsThreads, smem2, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return fail_launch(e, "rows probs launch");
+  {
+    const uint64_t kd[2] = {(uint64_t)pl.Hkv * pl.D, (uint64_t)pl.L * pl.total_keys};
+    const uint64_t ks[1] = {(uint64_t)pl.Hkv * pl.D * 2};
+    const uint32_t kb[2] = {64, kRowsChunk};
+    const uint64_t qd[3] = {(uint64_t)pl.D, (uint64_t)pl.L * pl.Hq, (uint64_t)pl.total_rows};
+    const uint64_t qs[2] = {(uint64_t)pl.D * 2, (uint64_t)pl.L * pl.Hq * pl.D * 2};
+    const uint32_t qb[3] = {64, (uint32_t)pl.G, (uint32_t)a.qbox};
+    if (!encode_bf16_map(&a.kmap, k, 2, kd, ks, kb) || !encode_bf16_map(&a.qmap, q_rows, 3, qd, qs, qb))
+      return rows_fail(LAST_ERR_CUDA, "multi-row scoring: the tensor maps cannot be encoded");
+  }
+  int dev = 0, sms = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  // as many stages as fit; more than half of an SM in all cases, so that one CTA holds
+  // an SM's tensor memory
+  const size_t stage = (size_t)(pl.D / 64) * (kRowsChunk + pl.npad) * 128;
+  const size_t fixed = 16 * 1024 + 1024;   // the kernel's own arrays (15 KB) and the alignment
+  a.nstage = (int)std::min<size_t>(kRowsMaxStages, ((size_t)optin - fixed) / stage);
+  const size_t smem = std::max<size_t>(a.nstage * stage + 1024, 116 * 1024);
+  for (int pass = 0; pass < 2; ++pass) {
+    void *fn = pass == 0 ? (void *)rows_pass_kernel<true> : (void *)rows_pass_kernel<false>;
+    const long long n = (pass == 0 ? pl.n_items1 : pl.n_items2) * pl.L * pl.Hkv;
+    if (n > 0x7fffffffLL) return rows_fail(LAST_ERR_UNSUPPORTED, "too many key chunks in all");
+    if (n > 0) {
+      a.n_items = (int)n;
+      if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        return fail_launch(e, "rows pass");
+      void *args[] = {&a};
+      e = cudaLaunchKernel(fn, dim3((unsigned)std::min<long long>(n, sms)), dim3(kPassThreads), args, smem, s);
+      if (e != cudaSuccess) return fail_launch(e, "rows pass launch");
+    }
+    if (pass == 0) {
+      rows_merge_kernel<<<dim3(pl.mass_blocks, pl.B), 256, 0, s>>>(a);
+      if ((e = cudaGetLastError()) != cudaSuccess) return fail_launch(e, "rows merge launch");
+    }
   }
   const int tiles = (pl.max_vis + kScoreThreads - 1) / kScoreThreads;
   rows_final_kernel<<<dim3(tiles, pl.B), kScoreThreads, 0, s>>>(a);

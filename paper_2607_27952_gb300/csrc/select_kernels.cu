@@ -2,6 +2,7 @@
 // map and launch.  The kernel itself is in select_impl.cuh; its instantiations
 // are in select_f32.cu, select_bf16.cu and select_bf16_tc.cu.
 #include "select_impl.cuh"
+#include "tensor_map.h"
 
 #include <algorithm>
 #include <cmath>
@@ -120,17 +121,29 @@ int active_clusters(void *fn, int csize, size_t smem, int threads) {
   return active;
 }
 
-// X as a [rows][dv] bf16 tensor, 64-element x box_rows boxes, 128-byte swizzle.
-bool encode_x_map(CUtensorMap *m, const void *x, long long rows, int dv, int box_rows) {
+bool encode_bf16_map(CUtensorMap *m, const void *base, int rank, const uint64_t *dims,
+                     const uint64_t *strides, const uint32_t *box) {
   EncodeTiledFn fn = encode_tiled();
-  if (fn == nullptr || rows <= 0) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)dv, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)dv * 2};
-  cuuint32_t box[2] = {(cuuint32_t)kTcBK, (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(x), dims, strides, box, estr,
+  if (fn == nullptr) return false;
+  cuuint64_t d[3], st[2];
+  cuuint32_t bx[3], es[3];
+  for (int i = 0; i < rank; ++i) {
+    if (dims[i] == 0) return false;
+    d[i] = dims[i];
+    bx[i] = box[i];
+    es[i] = 1;
+    if (i + 1 < rank) st[i] = strides[i];
+  }
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void *>(base), d, st, bx, es,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// X as a [rows][dv] bf16 tensor, 64-element x box_rows boxes, 128-byte swizzle.
+bool encode_x_map(CUtensorMap *m, const void *x, long long rows, int dv, int box_rows) {
+  const uint64_t dims[2] = {(uint64_t)dv, (uint64_t)(rows > 0 ? rows : 0)}, strides[1] = {(uint64_t)dv * 2};
+  const uint32_t box[2] = {(uint32_t)kTcBK, (uint32_t)box_rows};
+  return encode_bf16_map(m, x, 2, dims, strides, box);
 }
 
 namespace {

@@ -106,3 +106,15 @@ def test_many_rows_full_width():
     cu, pos, q = make_rows(wl, "all", np.random.default_rng(9), m_rows=64)
     assert int(np.diff(cu).max()) == 64
     check(wl, cu, pos, q)
+
+
+@pytest.mark.parametrize("hq,hkv,D,m_rows,n_vis,n_text,n_before", [
+    (9, 3, 64, 43, [129, 255, 257], [60, 47, 50], [0, 127, 128]),   # 129 columns: two epilogue groups
+    (8, 1, 256, 32, [128, 1], [40, 34], [1, 5]),                    # 256 columns, one stage
+    (4, 4, 128, 5, [2000, 31, 640], [7, 129, 8], [128, 0, 63]),     # more items than stages and CTAs
+])
+def test_chunk_edges_and_column_counts(hq, hkv, D, m_rows, n_vis, n_text, n_before):
+    wl = custom(name="edges", seed=71, batch=len(n_vis), n_vis=n_vis, n_text=n_text, n_before=n_before,
+                num_layers=2, num_q_heads=hq, num_kv_heads=hkv, head_dim=D, feat_dim=64, dtype="bf16",
+                keep=[1] * len(n_vis), n_planted=1)
+    check(wl, *make_rows(wl, "all", np.random.default_rng(3), m_rows=m_rows))
