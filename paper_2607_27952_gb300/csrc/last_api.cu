@@ -158,17 +158,19 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
     return kb > 1 && kb < n ? (long long)n * (gram_ld(n) / 32) : 0;
   };
   long long units = 0;
-  if (sel_scratch)
+  const bool gram_ok = p->feat_dim >= 8 && p->feat_dim % 8 == 0 && p->feat_dim <= kMaxFeatDim;
+  if (gram_ok)
     for (int b = 0; b < B; ++b) units += gram_units(b);
-  // Used where the contraction (about 1.1 PFLOP/s over the lower triangle) costs less
-  // than the rounds over X that it replaces: those accept about 16 picks a round and
-  // take about 100 us each, and the longest request's rounds set the call's time.
-  // Eight requests of 16384 x 2048: 3.7 ms against 16.6 ms at k = 2048, 8.5 ms at 1024;
-  // the line lies near k = 700.
-  double gram_s = 0.0;
-  if (sel_scratch)
-    for (int b = 0; b < B; ++b) gram_s += (double)gram_units(b) * 32.0 * p->feat_dim / 1.1e15;
-  pl->gram = units > 0 && units * 128 <= kGramMaxBytes && gram_s <= 6e-6 * pl->max_keep;
+  // Used where the contraction over the lower triangle (about 1.1 PFLOP/s on tensor
+  // cores, 20 T fma/s in the canonical order) costs less than the rounds over X that it
+  // replaces: those accept about 16 picks a round and take about 100 us each, and the
+  // longest request's rounds set the call's time.  Eight requests of 16384 x 2048: 3.0 ms
+  // against 16.6 ms at k = 2048, 8.5 ms at 1024; the line lies near k = 700.
+  const double fmas = 0.5 * (double)units * 32.0 * p->feat_dim;
+  const double tensor_s = 2.0 * fmas / 1.1e15, exact_s = fmas / 20e12;
+  pl->gram_exact = p->dtype == LAST_DTYPE_F32 || exact_s <= kGramExactSeconds;
+  pl->gram = units > 0 && units * 128 <= kGramMaxBytes &&
+             (pl->gram_exact ? exact_s : tensor_s) <= 6e-6 * pl->max_keep;
   if (pl->gram) {
     pl->off_rn = o;
     o = align_up(o + sizeof(float) * (size_t)pl->total_vis);
@@ -192,7 +194,10 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
     if (pl->gram) {
       m[kGramOff] = (int32_t)gram_off;
       gram_off += gram_units(b);
-      if (gram_units(b) > 0) pl->gram_tiles += gram_tiles(p->cu_vis[b + 1] - p->cu_vis[b], gram_long(pl->max_vis));
+      if (gram_units(b) > 0) {
+        const int n = p->cu_vis[b + 1] - p->cu_vis[b];
+        pl->gram_tiles += pl->gram_exact ? gram_exact_tiles(n, p->dtype == LAST_DTYPE_F32) : gram_tiles(n, gram_long(pl->max_vis));
+      }
     }
     m[kRootOff] = (int32_t)root_off;
     if (sel_scratch) root_off += root_cap(b);

@@ -36,6 +36,7 @@ constexpr int kSelectWarps = 8;
 constexpr int kGridMaxReq = 4;      // requests of one whole-GPU selection launch
 constexpr int kGridMaxCtas = 256;   // CTAs of one whole-GPU selection launch at most
 constexpr int kGatherThreads = 256;
+constexpr double kGramExactSeconds = 20e-6;   // bf16 batches up to this take the canonical matrix
 constexpr long long kGramMaxBytes = 12LL << 30;   // Gram matrices of one call at most
 
 // Device error flags (first word of the workspace).
@@ -66,7 +67,7 @@ struct Plan {
   // base_bytes excludes the first two (Top-k and the gather do not use them).
   size_t off_rn = 0, off_gram = 0, off_tile0 = 0, base_bytes = 0;
   int gram_tiles = 0;
-  bool gram = false;
+  bool gram = false, gram_exact = false;   // exact: in the canonical order, on CUDA cores
   // host staging (error word, meta rows, score items, selection order) in ws order
   std::vector<int32_t> host_blob;
   size_t blob_bytes = 0;  // bytes from off_meta to the end of the order array
@@ -98,6 +99,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
                                void *x_out, char *ws, cudaStream_t s, bool *done);
 // Tiles of the Gram kernel for one request; floats per row of its matrix.
 int gram_tiles(int n_tokens, bool pair);
+int gram_exact_tiles(int n_tokens, bool f32);
 // Whether CTA pairs compute the matrices (the longest request decides).
 bool gram_long(int max_vis);
 #ifdef __CUDACC__

@@ -1,8 +1,9 @@
-// Eq. 9-12 (Sec. 3.4): the greedy selection of bf16 features from a Gram matrix.
+// Eq. 9-12 (Sec. 3.4): the greedy selection from a Gram matrix.
 //
 // Three launches.  norms_kernel: 1/|x_i| of every token (canonical order).
 // gram_kernel or gram_pair_kernel: every request's dot products x_i . x_j on the tensor
-// cores, fp32, to the workspace (lower triangle computed, mirrored on the way out).
+// cores, fp32, to the workspace (lower triangle computed, mirrored on the way out); or
+// gram_exact_kernel: the same in the canonical order (fp32 features, small batches).
 // select_gram_kernel: the greedy, one thread-block cluster of C CTAs per request,
 // in rounds that accept a batch of consecutive picks at once and give exactly the
 // sequential Eq. 10-11 sequence:
@@ -479,6 +480,143 @@ __global__ void __launch_bounds__(256) norms_kernel(const char *x, float *rn, in
   }
 }
 
+// The same matrix in the canonical order on CUDA cores: every distance the greedy reads
+// from it is then exact.  For fp32 features (the tensor cores' tf32 would leave almost
+// every pair open) and for bf16 batches small enough that the evaluations it saves the
+// greedy outweigh it.  A warp's 32 lanes are the canonical order's: each holds the
+// partial sums of 8 x 8 pairs over its own coordinate groups, rows staged 256
+// coordinates at a time (three buffers), and the lanes' sums are added by the canonical
+// butterfly with the pairs dealt out on the way (62 shuffles for 64 pairs instead of
+// 320).  Bound by the fmas and the shared-memory reads that feed them: 15 T fma/s in fp32
+// on 4096 x 1024, 21 in bf16.  A CTA takes 32 x 32 pairs in fp32, whose copies limit
+// narrower tiles (six requests of 800 x 1000: 231 us at 32 x 16, 147 at 32 x 32), and 32 x
+// 16 in bf16, which only comes here in small batches that must be spread over the SMs
+// (one image of 576 x 2048: 27 against 32 us).
+constexpr int kExRows = 32, kExBufs = 3;
+template <typename T> constexpr int kExCols = sizeof(T) == 4 ? 32 : 16;
+int gram_exact_tiles(int n_tokens, bool f32) {
+  const int R = (n_tokens + kExRows - 1) / kExRows;
+  return f32 ? R * (R + 1) / 2 : R * (R + 1);
+}
+
+struct GramExactArgs {
+  const char *x;
+  float *gram;
+  const int32_t *meta;
+  const int32_t *tile0;
+  int B, dv, row_bytes;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(16 * kExCols<T>, kExRows / kExCols<T>) gram_exact_kernel(const GramExactArgs a) {
+  constexpr int kCols = kExCols<T>, kThreads = 16 * kCols, kPer = kExRows / kCols;   // kPer column blocks a row block
+  constexpr int kVec = (int)sizeof(T) / 2;            // 16-byte pieces per 8 coordinates
+  constexpr int kRowBytes = 256 * (int)sizeof(T);     // a row's staged part
+  constexpr int kBuf = (kExRows + kCols) * kRowBytes;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int lo = 0, hi = a.B - 1;
+  const int tile = blockIdx.x;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (a.tile0[mid] <= tile) lo = mid; else hi = mid - 1;
+  }
+  const int rem = tile - a.tile0[lo];
+  // row block ti has kPer (ti + 1) column blocks
+  int ti = (int)((sqrtf(8.0f * (float)(rem / kPer) + 1.0f) - 1.0f) * 0.5f);
+  while (kPer * (ti * (ti + 1) / 2) > rem) --ti;
+  while (kPer * ((ti + 1) * (ti + 2) / 2) <= rem) ++ti;
+  const int tj = rem - kPer * (ti * (ti + 1) / 2);
+  const int32_t *m = a.meta + lo * kMetaFields;
+  const int N = m[kNumVis], ld = gram_ld(N);
+  float *G = a.gram + (long long)m[kGramOff] * 32;
+  const char *xreq = a.x + (long long)m[kVisOff] * a.row_bytes;
+  const int i0 = ti * kExRows, j0 = tj * kCols;
+  const uint32_t sbase = smem_addr(smem);
+  const int nchunk = (a.dv + 255) / 256;
+
+  // a thread copies the same 16-byte piece of every (threads / pieces per row)-th row:
+  // piece q is lane q / kVec's part q % kVec.  fp32 lanes read every other piece; swapping
+  // the two pieces of every second group of four lanes spreads them over all banks.
+  constexpr int kPieces = 32 * kVec, kStep = kThreads / kPieces;
+  const int q0 = tid % kPieces, r0 = tid / kPieces, col0 = (q0 / kVec) * 8;
+  const char *src0 = xreq + 16 * q0;
+  const int swap = kVec == 2 ? (lane >> 2) & 1 : 0;
+  const uint32_t dst_q = sbase + r0 * kRowBytes + 16 * (kVec == 2 ? q0 ^ ((q0 >> 3) & 1) : q0);
+  auto stage = [&](int c) {
+    const uint32_t dst = dst_q + (c % kExBufs) * kBuf;
+    const char *src = src0 + (size_t)c * kRowBytes;
+    const bool in = 256 * c + col0 < a.dv;
+#pragma unroll
+    for (int i = 0; i < (kExRows + kCols) / kStep; ++i) {
+      const int r = r0 + i * kStep;   // (a step never straddles the two operands)
+      const int t = min(i * kStep < kExRows ? i0 + r : j0 + r - kExRows, N - 1);
+      if (in)
+        cp_async16(dst + i * kStep * kRowBytes, src + (size_t)(uint32_t)t * (uint32_t)a.row_bytes);
+      else
+        asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" :: "r"(dst + i * kStep * kRowBytes), "r"(0u) : "memory");
+    }
+    cp_async_commit();
+  };
+  float acc[64];
+#pragma unroll
+  for (int q = 0; q < 64; ++q) acc[q] = 0.f;
+  constexpr int kWj = kCols / 8;   // warps along the columns
+  const uint32_t row_i = 8 * (warp / kWj), row_j = kExRows + 8 * (warp % kWj);
+  stage(0);
+  if (nchunk > 1) stage(1);
+  else cp_async_commit();
+  for (int c = 0; c < nchunk; ++c) {
+    cp_async_wait<1>();
+    __syncthreads();   // chunk c has landed; its predecessor's buffer is free
+    if (c + 2 < nchunk) stage(c + 2);
+    else cp_async_commit();
+#pragma unroll 1
+    for (int h = 0; h < kVec; ++h) {
+      const uint32_t base = sbase + (c % kExBufs) * kBuf + 16 * (lane * kVec + (h ^ swap));
+      U4 xi[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) xi[i] = lds32(base + (row_i + i) * kRowBytes);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const U4 xj = lds32(base + (row_j + j) * kRowBytes);
+        const uint32_t jw[4] = {xj.x, xj.y, xj.z, xj.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const uint32_t iw = q == 0 ? xi[i].x : q == 1 ? xi[i].y : q == 2 ? xi[i].z : xi[i].w;
+            float &s = acc[i * 8 + j];
+            if constexpr (sizeof(T) == 2) {
+              s = fma_bf16_lo(iw, jw[q], s);
+              s = fma_bf16_hi(iw, jw[q], s);
+            } else {
+              s = __fmaf_rn(__uint_as_float(iw), __uint_as_float(jw[q]), s);
+            }
+          }
+      }
+    }
+  }
+  // butterfly over the lanes (offsets 16 .. 1); at each step a lane keeps half of the
+  // pairs, so lane l ends with pairs 2 l, 2 l + 1: row l / 4, columns 2 (l % 4) ..
+#pragma unroll
+  for (int o = 16, n = 32; o > 0; o >>= 1, n >>= 1) {
+#pragma unroll
+    for (int q = 0; q < n; ++q) {
+      const float send = (lane & o) ? acc[q] : acc[q + n];
+      const float keep = (lane & o) ? acc[q + n] : acc[q];
+      acc[q] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, o));
+    }
+  }
+  const int i = i0 + (int)row_i + (lane >> 2), j = j0 + 8 * (warp % kWj) + 2 * (lane & 3);
+  if (i < N) {
+    if (j < ld) *reinterpret_cast<float2 *>(G + (long long)i * ld + j) = make_float2(acc[0], acc[1]);
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      if (j + r < N) G[(long long)(j + r) * ld + i] = acc[r];
+  }
+}
+
 struct GramSelArgs {
   const char *x;
   const float *w, *rn, *gram;
@@ -544,7 +682,9 @@ __device__ __forceinline__ uint32_t key_high(float w, float delta) {
   return (uint32_t)(argmax_key(__fmul_rn(w, delta), 0) >> 32);
 }
 
-template <int NCH>
+// EX: the matrix holds canonical dot products (gram_exact_kernel, eps = 0): every
+// distance is final, nothing is pending and no row is read before the epilogue.
+template <int NCH, bool EX>
 __global__ void __launch_bounds__(kGthreads, 1)
 select_gram_kernel(const __grid_constant__ GramSelArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -717,7 +857,9 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
             bt &= bt - 1;
             const float2 cc = cen[j0 + j];
             const float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(__ldg(G + crow[j0 + j] + t), ri), cc.y));
-            if (!in_range || ((wide >> j) & 1u) || d != d) {
+            if constexpr (EX) {
+              hi = fminf(hi, d);   // NaN leaves it
+            } else if (!in_range || ((wide >> j) & 1u) || d != d) {
               now |= 1u << j;
             } else if (!(__fsub_rd(d, eps) >= hi)) {
               const uint32_t c = __float_as_uint(cc.x);
@@ -735,34 +877,41 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
               }
             }
           }
-          p0_s[li] = p0;
-          p1_s[li] = p1;
-          id_s[li] = ids;
-          ks[li] = key_high(w_s[li], fminf(e, __fadd_ru(fminf(p0, p1), eps)));
+          if constexpr (EX) {
+            e_s[li] = hi;
+            ks[li] = key_high(w_s[li], hi);
+          } else {
+            p0_s[li] = p0;
+            p1_s[li] = p1;
+            id_s[li] = ids;
+            ks[li] = key_high(w_s[li], fminf(e, __fadd_ru(fminf(p0, p1), eps)));
+          }
         }
         __syncwarp();
         // the whole warp per token to evaluate
-        for (unsigned todo = __ballot_sync(0xffffffffu, now != 0u); todo != 0u; todo &= todo - 1) {
-          const int src = __ffs(todo) - 1;
-          const int lt = __shfl_sync(0xffffffffu, li, src);
-          uint32_t bt = __shfl_sync(0xffffffffu, now, src);
-          U4 xv[NCH], xc[NCH];
-          load_row(__shfl_sync(0xffffffffu, t, src), xv);
-          const float rt = __shfl_sync(0xffffffffu, ri, src);
-          float e = e_s[lt];
-          while (bt) {
-            const int j = __ffs(bt) - 1;
-            bt &= bt - 1;
-            const float2 cc = cen[j0 + j];
-            load_row(__float_as_int(cc.x), xc);
-            e = fminf(e, distance(xv, xc, rt, cc.y));
+        if constexpr (!EX) {
+          for (unsigned todo = __ballot_sync(0xffffffffu, now != 0u); todo != 0u; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const int lt = __shfl_sync(0xffffffffu, li, src);
+            uint32_t bt = __shfl_sync(0xffffffffu, now, src);
+            U4 xv[NCH], xc[NCH];
+            load_row(__shfl_sync(0xffffffffu, t, src), xv);
+            const float rt = __shfl_sync(0xffffffffu, ri, src);
+            float e = e_s[lt];
+            while (bt) {
+              const int j = __ffs(bt) - 1;
+              bt &= bt - 1;
+              const float2 cc = cen[j0 + j];
+              load_row(__float_as_int(cc.x), xc);
+              e = fminf(e, distance(xv, xc, rt, cc.y));
+            }
+            __syncwarp();
+            if (lane == 0) {
+              e_s[lt] = e;
+              ks[lt] = key_high(w_s[lt], fminf(e, __fadd_ru(fminf(p0_s[lt], p1_s[lt]), eps)));
+            }
+            __syncwarp();
           }
-          __syncwarp();
-          if (lane == 0) {
-            e_s[lt] = e;
-            ks[lt] = key_high(w_s[lt], fminf(e, __fadd_ru(fminf(p0_s[lt], p1_s[lt]), eps)));
-          }
-          __syncwarp();
         }
       }
     };
@@ -903,22 +1052,24 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       const unsigned long long Up = nc > kGlist ? misc[20] : U;
       unsigned long long need = 0ull;   // this warp's share of the CTA's members
       int before = 0;
+      if constexpr (!EX) {
 #pragma unroll
-      for (int h = 0; h < kGper; ++h) {
-        const int u = lane + 32 * h;
-        const bool mine = u < nL && owned((int)(mem[u].idx >> 5)) &&
-                          !(mem[u].p0 == INFINITY && mem[u].p1 == INFINITY);
-        const unsigned bal = __ballot_sync(0xffffffffu, mine);
-        const int at = before + __popc(bal & ((1u << lane) - 1u));
-        need |= (unsigned long long)__ballot_sync(0xffffffffu, mine && at % kGwarps == warp) << (32 * h);
-        before += __popc(bal);
-      }
-      // their rows start towards L2
-      for (unsigned long long n = need; n != 0ull; n &= n - 1) {
-        const GramEntry &me = mem[__ffsll((long long)n) - 1];
-        if (lane * 128 < rb) {
-          prefetch_l2(xreq + (long long)me.idx * rb + lane * 128);
-          if (me.p0 != INFINITY) prefetch_l2(xreq + (long long)(me.ids & 0xffffu) * rb + lane * 128);
+        for (int h = 0; h < kGper; ++h) {
+          const int u = lane + 32 * h;
+          const bool mine = u < nL && owned((int)(mem[u].idx >> 5)) &&
+                            !(mem[u].p0 == INFINITY && mem[u].p1 == INFINITY);
+          const unsigned bal = __ballot_sync(0xffffffffu, mine);
+          const int at = before + __popc(bal & ((1u << lane) - 1u));
+          need |= (unsigned long long)__ballot_sync(0xffffffffu, mine && at % kGwarps == warp) << (32 * h);
+          before += __popc(bal);
+        }
+        // their rows start towards L2
+        for (unsigned long long n = need; n != 0ull; n &= n - 1) {
+          const GramEntry &me = mem[__ffsll((long long)n) - 1];
+          if (lane * 128 < rb) {
+            prefetch_l2(xreq + (long long)me.idx * rb + lane * 128);
+            if (me.p0 != INFINITY) prefetch_l2(xreq + (long long)(me.ids & 0xffffu) * rb + lane * 128);
+          }
         }
       }
       // 3. pairwise distances from the Gram matrix (NaN: outside the certificate): a warp
@@ -945,16 +1096,19 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
             const int u = pu[i][h], v = pv[i][h];
             if (u < v && v < nL) {
               const float ru = mem[u].r, rv = mem[v].r;
-              float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[i][h], ru), rv));
-              if (!tri_in_range(ru) || !tri_in_range(rv)) d = __int_as_float(0x7fffffff);
-              pm[u * kGpairLd + v] = pm[v * kGpairLd + u] = d;
+              // pm[centre][token]
+              float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[i][h], rv), ru)), dt = d;
+              if constexpr (EX) dt = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[i][h], ru), rv));
+              else if (!tri_in_range(ru) || !tri_in_range(rv)) d = dt = __int_as_float(0x7fffffff);
+              pm[u * kGpairLd + v] = d;
+              pm[v * kGpairLd + u] = dt;
             }
           }
       }
       // the members' pending centres in the canonical order, by the CTA that owns the
       // member, which keeps the result and sends it to every CTA: every member's delta
       // is exact from here on
-      {
+      if constexpr (!EX) {
         for (; need != 0ull; need &= need - 1) {
           const int u = __ffsll((long long)need) - 1;
           const GramEntry me = mem[u];
@@ -981,8 +1135,10 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
           }
           if (lane < C) st_cluster_v2f(map_shared(&res[u], lane), make_float2(__uint_as_float(kh), e));
         }
+        csync();
+      } else {
+        __syncthreads();
       }
-      csync();
       // 4. replay the greedy on the list (warp 0; lane u holds members u, u + 32, ..).
       // A member's delta lies in [lo, hi]: exact until an accepted centre's distance
       // reaches below hi + eps; such centres are kept in `pend` and evaluated only when
@@ -998,7 +1154,7 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
           id[h] = 0u;
           e[h] = wv[h] = 0.f;
           if (u < nL) {
-            const bool was = mem[u].p0 != INFINITY || mem[u].p1 != INFINITY;   // evaluated just now
+            const bool was = !EX && (mem[u].p0 != INFINITY || mem[u].p1 != INFINITY);   // evaluated just now
             const float2 rv = res[u];
             kh[h] = was ? __float_as_uint(rv.x) : mem[u].kh;
             e[h] = was ? rv.y : mem[u].e;
@@ -1024,7 +1180,7 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
           for (int h = kGper - 1; h >= 0; --h) {
             win[h] = __ballot_sync(0xffffffffu, kh[h] == mx);
             leads += __popc(win[h]);
-            const unsigned open = __ballot_sync(0xffffffffu, kh[h] == mx && pend[h] != 0ull);
+            const unsigned open = EX ? 0u : __ballot_sync(0xffffffffu, kh[h] == mx && pend[h] != 0ull);
             bl = win[h] ? __ffs(win[h]) - 1 + 32 * h : bl;
             inexact = win[h] ? open != 0u : inexact;
           }
@@ -1038,14 +1194,15 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
 #pragma unroll
             for (int h = 0; h < kGper; ++h) {
               const unsigned w = __ballot_sync(0xffffffffu, kh[h] == mx && id[h] == low);
-              const unsigned open = __ballot_sync(0xffffffffu, kh[h] == mx && id[h] == low && pend[h] != 0ull);
+              const unsigned open =
+                  EX ? 0u : __ballot_sync(0xffffffffu, kh[h] == mx && id[h] == low && pend[h] != 0ull);
               if (w) {
                 bl = __ffs(w) - 1 + 32 * h;
                 inexact = open != 0u;
               }
             }
           }
-          if (inexact) {
+          if (!EX && inexact) {
             // accepted as it is only if its lower key leads every other upper key
             const int src = bl & 31;
             unsigned long long bp = 0ull;
@@ -1077,7 +1234,7 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
                 const int j = __ffsll((long long)bp) - 1;
                 bp &= bp - 1;
                 const int cj = acc_s[j];
-                if (__fsub_rd(pm[bl * kGpairLd + cj], eps) >= bhi) continue;   // excluded since
+                if (__fsub_rd(pm[cj * kGpairLd + bl], eps) >= bhi) continue;   // excluded since
                 load_row((int)mem[cj].idx, xc);
                 be = fminf(be, distance(xv, xc, mem[bl].r, mem[cj].r));
               }
@@ -1100,11 +1257,15 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
           for (int h = 0; h < kGper; ++h) {
             const int u = lane + 32 * h;
             const float d = pm[bl * kGpairLd + u];
-            const float dlo = __fsub_rd(d, eps), dhi = __fadd_ru(d, eps);
-            const bool hit = !(dlo >= hi[h]);   // NaN too
-            pend[h] |= hit ? bit : 0ull;
-            lo[h] = hit ? (d == d ? fminf(lo[h], dlo) : -INFINITY) : lo[h];
-            hi[h] = hit ? fminf(hi[h], dhi) : hi[h];   // NaN keeps hi
+            if constexpr (EX) {
+              hi[h] = fminf(hi[h], d);
+            } else {
+              const float dlo = __fsub_rd(d, eps), dhi = __fadd_ru(d, eps);
+              const bool hit = !(dlo >= hi[h]);   // NaN too
+              pend[h] |= hit ? bit : 0ull;
+              lo[h] = hit ? (d == d ? fminf(lo[h], dlo) : -INFINITY) : lo[h];
+              hi[h] = hit ? fminf(hi[h], dhi) : hi[h];   // NaN keeps hi
+            }
             kh[h] = kh[h] == 0u || u == bl ? 0u : key_high(wv[h], hi[h]);
           }
           // posted; every eighth centre releases a batch to the workers
@@ -1199,13 +1360,13 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
 
 namespace {
 
-template <int NCH>
+template <typename T, int NCH>
 void pick_nch(int nch, void **sel, void **norm) {
   if (nch == NCH) {
-    *sel = (void *)select_gram_kernel<NCH>;
-    *norm = (void *)norms_kernel<__nv_bfloat16, NCH>;
+    if constexpr (sizeof(T) == 2) *sel = (void *)select_gram_kernel<NCH, false>;
+    *norm = (void *)norms_kernel<T, NCH>;
   } else if constexpr (NCH > 1) {
-    pick_nch<NCH - 1>(nch, sel, norm);
+    pick_nch<T, NCH - 1>(nch, sel, norm);
   }
 }
 
@@ -1237,7 +1398,10 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int rb = pl.dv * pl.elem;
   void *sel_fn = nullptr, *norm_fn = nullptr;
-  pick_nch<8>((pl.dv + 255) / 256, &sel_fn, &norm_fn);
+  const bool f32 = pl.dtype == LAST_DTYPE_F32;
+  if (f32) pick_nch<float, 8>((pl.dv + 255) / 256, &sel_fn, &norm_fn);
+  else pick_nch<__nv_bfloat16, 8>((pl.dv + 255) / 256, &sel_fn, &norm_fn);
+  if (pl.gram_exact) sel_fn = (void *)select_gram_kernel<1, true>;
 
   // The cluster size with the shortest schedule: requests go, most work first, to the
   // next free cluster; a request takes about k / 16 + 2 rounds of 27K cycles, 4.6K more
@@ -1273,7 +1437,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
 
   GramArgs g;
   std::memset(&g, 0, sizeof g);
-  if (!encode_x_map(&g.tmap, x, pl.total_vis, pl.dv)) return cudaSuccess;
+  if (!pl.gram_exact && !encode_x_map(&g.tmap, x, pl.total_vis, pl.dv)) return cudaSuccess;
   g.gram = reinterpret_cast<float *>(ws + pl.off_gram);
   g.meta = reinterpret_cast<const int32_t *>(ws + pl.off_meta);
   g.tile0 = reinterpret_cast<const int32_t *>(ws + pl.off_tile0);
@@ -1293,6 +1457,19 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
     void *nargs[] = {&xc, &rn, &dv, &row, &total};
     const int ngrid = (int)std::min<long long>((pl.total_vis + 7) / 8, (long long)sms * 8);
     if ((e = cudaLaunchKernel(norm_fn, dim3(ngrid), dim3(256), nargs, 0, s)) != cudaSuccess) return e;
+    if (pl.gram_exact) {
+      GramExactArgs x1 = {};
+      x1.x = static_cast<const char *>(x);
+      x1.gram = g.gram; x1.meta = g.meta; x1.tile0 = g.tile0;
+      x1.B = pl.B; x1.dv = pl.dv; x1.row_bytes = rb;
+      void *fn = f32 ? (void *)gram_exact_kernel<float> : (void *)gram_exact_kernel<__nv_bfloat16>;
+      const int cols = f32 ? kExCols<float> : kExCols<__nv_bfloat16>;
+      const size_t smem = (size_t)kExBufs * (kExRows + cols) * 256 * pl.elem;
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      void *args[] = {&x1};
+      if ((e = cudaLaunchKernel(fn, dim3(pl.gram_tiles), dim3(16 * cols), args, smem, s)) != cudaSuccess) return e;
+    } else {
     // the matrix needs no norms: its kernel starts beside the norms' and ends after them
     void *fn = pair ? (void *)gram_pair_kernel : (void *)gram_kernel;
     const size_t smem = 192 * 1024 + 1024;
@@ -1316,6 +1493,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
     cfg.numAttrs = 2;
     void *args[] = {&g};
     if ((e = cudaLaunchKernelExC(&cfg, fn, args)) != cudaSuccess) return e;
+    }
   }
   GramSelArgs a;
   std::memset(&a, 0, sizeof a);
@@ -1325,7 +1503,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   a.meta = g.meta;
   a.order = reinterpret_cast<const int32_t *>(ws + pl.off_order);
   a.dv = pl.dv; a.row_bytes = rb; a.csize = sh.C; a.mc = sh.mc; a.slots = sh.slots; a.words = sh.words;
-  a.eps = gram_distance_eps(pl.dv, chunk);
+  a.eps = pl.gram_exact ? 0.f : gram_distance_eps(pl.dv, chunk);
   a.err = g.err;
   e = cudaFuncSetAttribute(sel_fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(sel_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);

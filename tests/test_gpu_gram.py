@@ -1,6 +1,7 @@
-"""The greedy from a Gram matrix (select_gram.cu) at the sizes where it can go wrong:
-around the 128-row and 256-column tiles (of one CTA and of pairs) and the 32-token blocks, one token more than
-the cluster's warps hold, feature widths that end inside a K block, every budget from
+"""The greedy from a Gram matrix (select_gram.cu; on tensor cores, or in the canonical
+order for fp32 and small batches) at the sizes where it can go wrong: around the
+128-row and 256-column tiles (of one CTA and of pairs) and the 32-token blocks, one token
+more than the cluster's warps hold, feature widths that end inside a K block, every budget from
 one pick to all but one, exact ties, zero rows and rows outside the certificate's norm
 range.  Indices and rows are exact against the oracle."""
 import numpy as np
@@ -14,9 +15,9 @@ from workloads import bf16_bits_to_f32, custom, f32_to_bf16_bits
 pytestmark = pytest.mark.gpu
 
 
-def _wl(n_vis, keep, d_v, seed=5, **kw):
+def _wl(n_vis, keep, d_v, seed=5, dtype="bf16", **kw):
     return custom(name="gram", seed=seed, batch=len(n_vis), n_vis=n_vis, n_text=4, num_layers=1,
-                  num_q_heads=4, num_kv_heads=2, head_dim=64, feat_dim=d_v, dtype="bf16", keep=keep,
+                  num_q_heads=4, num_kv_heads=2, head_dim=64, feat_dim=d_v, dtype=dtype, keep=keep,
                   n_clusters=kw.pop("n_clusters", 12), n_planted=3, **kw)
 
 
@@ -36,6 +37,7 @@ def _run(wl, x=None, w=None):
     return w, idx.cpu().numpy(), to_host_bits(xs)
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("d_v", [8, 72, 520, 1536, 2048])
 @pytest.mark.parametrize("n_vis,keep", [
     ([1, 31, 33, 127, 129], [1, 30, 2, 64, 40]),
@@ -43,22 +45,23 @@ def _run(wl, x=None, w=None):
     ([545, 640, 2049], [100, 0, 130]),
     ([8200, 90, 257], [60, 20, 60]),       # CTA pairs
 ])
-def test_selection_equals_the_oracle(n_vis, keep, d_v):
-    wl = _wl(n_vis, keep, d_v)
+def test_selection_equals_the_oracle(n_vis, keep, d_v, dtype):
+    wl = _wl(n_vis, keep, d_v, dtype=dtype)
     w, idx, xs = _run(wl)
     assert_selection_equal(wl, w, idx, range(wl.batch))
     assert_gather_equal(wl, idx, xs, range(wl.batch))
 
 
-def test_ties_zero_rows_and_extreme_norms():
-    n, d = 300, 512
-    wl = _wl([n], [150], d)
-    x = bf16_bits_to_f32(wl.x).copy()
+@pytest.mark.parametrize("dtype,n", [("bf16", 300), ("bf16", 1900), ("f32", 300)])
+def test_ties_zero_rows_and_extreme_norms(dtype, n):
+    d = 512   # 300 tokens: canonical matrix, 1900: tensor cores
+    wl = _wl([n], [150], d, dtype=dtype)
+    x = (bf16_bits_to_f32(wl.x) if dtype == "bf16" else wl.x).copy()
     x[10:60] = x[9]                      # exact duplicates
     x[60:70] = 0.0
     x[70:110] *= np.float32(2.0) ** -70   # outside the certificate's norm range
     x[110:150] *= np.float32(2.0) ** 55
-    wl.x = f32_to_bf16_bits(x)
+    wl.x = f32_to_bf16_bits(x) if dtype == "bf16" else x
     w = np.full(n, 1.0 / n, dtype=np.float32)
     w[:5] = 0.0
     w, idx, _ = _run(wl, w=w)
