@@ -18,9 +18,10 @@
 //      tokens, eight centres at a time as the replay posts them.
 // The Gram distances d~ are only known to within eps, the decisions are canonical, so
 // a token carries an interval: the minimum e over the centres evaluated so far, and up
-// to two pending centres whose d~ lies within eps of being the minimum.  Tokens are
+// to four pending centres whose d~ lies within eps of being the minimum.  Tokens are
 // ranked by the upper end; a member of the list has its pending centres evaluated in
-// the canonical order (by the CTA that owns it; a second cluster barrier), and during
+// the canonical order (by the CTA that owns it, which sends the member's values to the
+// others; a second cluster barrier), and during
 // the replay a member is evaluated again only when the order of the picks depends on
 // it.  A token far from the lead is never evaluated at all: evaluating every pair that
 // the certificate leaves open, at the moment it appears, took 185K of 400K cycles a
@@ -57,7 +58,8 @@ namespace {
 
 constexpr int kGwarps = 16;
 constexpr int kGthreads = kGwarps * 32;
-constexpr int kGwork = kGwarps - 1;        // warps 1.. own the tokens, warp 0 replays the greedy
+constexpr bool kGspare = false;            // warp 0 alone on its scheduler: warps 4, 8, 12 own nothing
+constexpr int kGwork = kGspare ? 12 : kGwarps - 1;   // worker warps own the tokens, warp 0 replays
 constexpr int kGtok = kGwork * 32;
 constexpr int kGbatch = 8;                 // accepted centres handed to the workers at a time
 constexpr int kGlist = 64;                 // candidate list: two members per lane of the replay
@@ -513,6 +515,7 @@ __global__ void __launch_bounds__(16 * kExCols<T>, kExRows / kExCols<T>) gram_ex
   constexpr int kVec = (int)sizeof(T) / 2;            // 16-byte pieces per 8 coordinates
   constexpr int kRowBytes = 256 * (int)sizeof(T);     // a row's staged part
   constexpr int kBuf = (kExRows + kCols) * kRowBytes;
+  asm volatile("griddepcontrol.launch_dependents;");   // the greedy waits for this grid's end
   extern __shared__ __align__(128) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int lo = 0, hi = a.B - 1;
@@ -615,6 +618,7 @@ __global__ void __launch_bounds__(16 * kExCols<T>, kExRows / kExCols<T>) gram_ex
     for (int r = 0; r < 2; ++r)
       if (j + r < N) G[(long long)(j + r) * ld + i] = acc[r];
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the norms too are done when this grid is
 }
 
 struct GramSelArgs {
@@ -628,20 +632,14 @@ struct GramSelArgs {
   unsigned *err;
 };
 
-// A published candidate: upper key (high word), token, w~, 1/|x|, the evaluated
-// minimum e, and up to two centres whose distance is only known to within eps.
-struct GramEntry {
-  uint32_t idx;
-  float w, r;
-  uint32_t ids;            // centre of p0 | centre of p1 << 16
-  uint32_t kh;
-  float e, p0, p1;
-};
-static_assert(sizeof(GramEntry) == 32, "two 16-byte stores publish an entry");
+// Centres of a token whose distance is only known to within eps.  With two, tokens of
+// tight clusters were evaluated again and again as a third came near: 2 / 4 took 2.53 /
+// 2.44 ms on 128 requests of 256..4096, 1.29 / 1.20 on one video request.
+constexpr int kGpend = 4;
 
 // Shared memory of select_gram_kernel (host sizing and device carve-up alike).
 struct GramSelSmem {
-  size_t ks, w, r, e, p0, p1, ids, hot, sel, pkey, pub, ckey, cidx, pm, mem, res, top, acc, cen,
+  size_t ks, w, r, e, hi, p, ids, hot, sel, pkey, pwr, ckey, cidx, pm, lidx, lr, res, top, acc, cen,
       crow, bars, misc, total;
 };
 __host__ __device__ inline GramSelSmem gram_sel_smem(int slots, int words, int csize, int mc) {
@@ -652,18 +650,19 @@ __host__ __device__ inline GramSelSmem gram_sel_smem(int slots, int words, int c
   s.w = o; o += 4 * cap;
   s.r = o; o += 4 * cap;
   s.e = o; o += 4 * cap;
-  s.p0 = o; o += 4 * cap;
-  s.p1 = o; o += 4 * cap;
-  s.ids = o; o += 4 * cap;
+  s.hi = o; o += 4 * cap;                         // upper end of delta
+  s.p = o; o += 4 * kGpend * cap;                 // pending centres: distance
+  s.ids = o; o += 2 * kGpend * cap;               // and token
   s.hot = o; o += 4 * cap;                        // tokens a batch may lower: slot, centres
   s.sel = o; o += align16(4 * (size_t)words);     // selected bits of the whole request
   s.pkey = o; o += (size_t)2 * kGwork * csize * (mc + 1) * 8;   // published keys
-  s.pub = o; o += (size_t)2 * kGwork * csize * (mc + 1) * sizeof(GramEntry);
+  s.pwr = o; o += (size_t)2 * kGwork * csize * (mc + 1) * 8;    // and their w~, 1/|x|
   s.ckey = o = align16(o); o += 8 * (kGcand + 2);
   s.cidx = o; o += 2 * kGcand;
   s.pm = o; o += align16(4 * kGlist * kGpairLd);  // the list's pairwise distances
-  s.mem = o; o += sizeof(GramEntry) * kGlist;
-  s.res = o; o += 8 * kGlist;                     // members evaluated by their owners: key, delta
+  s.lidx = o; o += 4 * kGlist;                    // the list: token, 1/|x|
+  s.lr = o; o += 4 * kGlist;
+  s.res = o = align16(o); o += 16 * kGlist;       // key and delta (from its owner), w~, 1/|x|
   s.top = o; o += 8 * kGwarps * 16;               // a warp's leading keys
   s.acc = o; o += 4 * kGmaxAccept;
   s.cen = o; o += 8 * kGmaxAccept;                // accepted centres: token, 1/|x|
@@ -690,6 +689,9 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int C = a.csize, rank = (int)cluster_ctarank();
+  // a programmatic dependent of the canonical matrix's kernel: nothing is read before it
+  // (and what precedes it) has completed
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int b = a.order[cluster_id_x()];
   const int32_t *m = a.meta + b * kMetaFields;
   const int voff = m[kVisOff], N = m[kNumVis], koff = m[kKeepOff], K = m[kNumKeep];
@@ -703,22 +705,25 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       return;
     }
   }
+  const int widx = !kGspare ? warp - 1 : (warp & 3) ? (warp >> 2) * 3 + (warp & 3) - 1 : -1;   // worker or -1
   uint32_t *ks = reinterpret_cast<uint32_t *>(smem + S.ks);
   float *w_s = reinterpret_cast<float *>(smem + S.w);
   float *r_s = reinterpret_cast<float *>(smem + S.r);
   float *e_s = reinterpret_cast<float *>(smem + S.e);
-  float *p0_s = reinterpret_cast<float *>(smem + S.p0);
-  float *p1_s = reinterpret_cast<float *>(smem + S.p1);
-  uint32_t *id_s = reinterpret_cast<uint32_t *>(smem + S.ids);
-  uint32_t *hot = reinterpret_cast<uint32_t *>(smem + S.hot) + (warp - 1) * a.slots * 32;   // workers
+  float *hi_s = reinterpret_cast<float *>(smem + S.hi);
+  const int cap = a.slots * kGtok;
+  float *p_s = reinterpret_cast<float *>(smem + S.p);            // [kGpend][cap]
+  uint16_t *id_s = reinterpret_cast<uint16_t *>(smem + S.ids);   // [kGpend][cap]
+  uint32_t *hot = reinterpret_cast<uint32_t *>(smem + S.hot) + widx * a.slots * 32;   // workers
   uint32_t *sel = reinterpret_cast<uint32_t *>(smem + S.sel);
-  GramEntry *pub = reinterpret_cast<GramEntry *>(smem + S.pub);
   unsigned long long *pkey = reinterpret_cast<unsigned long long *>(smem + S.pkey);
   unsigned long long *ckey = reinterpret_cast<unsigned long long *>(smem + S.ckey);
-  uint16_t *cidx = reinterpret_cast<uint16_t *>(smem + S.cidx);
   float *pm = reinterpret_cast<float *>(smem + S.pm);
-  GramEntry *mem = reinterpret_cast<GramEntry *>(smem + S.mem);
-  float2 *res = reinterpret_cast<float2 *>(smem + S.res);
+  int *lidx = reinterpret_cast<int *>(smem + S.lidx);
+  float *lr = reinterpret_cast<float *>(smem + S.lr);
+  float2 *pwr = reinterpret_cast<float2 *>(smem + S.pwr);
+  uint16_t *cidx = reinterpret_cast<uint16_t *>(smem + S.cidx);
+  float4 *res = reinterpret_cast<float4 *>(smem + S.res);
   unsigned long long *top_s = reinterpret_cast<unsigned long long *>(smem + S.top) + warp * 16;
   int *acc_s = reinterpret_cast<int *>(smem + S.acc);
   float2 *cen = reinterpret_cast<float2 *>(smem + S.cen);
@@ -735,9 +740,9 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
   const float *G = a.gram + (long long)m[kGramOff] * 32;
   const int P = kGwork * C;                           // publishing warps of the cluster
   const int step = C * kGwork;                        // blocks between a warp's slots
-  const int blk0 = rank + C * (warp - 1);             // a worker's first block
-  const int nslot = warp == 0 ? 0 : (nblk - blk0 + step - 1) / step;   // and its blocks (<= a.slots)
-  const int li0 = tid - 32;                           // a worker thread's first token slot
+  const int blk0 = rank + C * widx;             // a worker's first block
+  const int nslot = widx < 0 ? 0 : (nblk - blk0 + step - 1) / step;   // and its blocks (<= a.slots)
+  const int li0 = widx * 32 + lane;                           // a worker thread's first token slot
   // block k (< 2^12): owner CTA and slot in shared memory, by multiplication
   const uint32_t inv_c = (0xffffffffu / (uint32_t)C) + 1u, inv_step = (0xffffffffu / (uint32_t)step) + 1u;
   auto over_c = [&](int k) { return C == 1 ? k : (int)__umulhi((uint32_t)k, inv_c); };
@@ -755,10 +760,12 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
     const bool in = t < N;
     w_s[li] = in ? wreq[t] : 0.f;
     r_s[li] = in && K < N ? rreq[t] : 0.f;
-    e_s[li] = INFINITY;
-    p0_s[li] = INFINITY;
-    p1_s[li] = INFINITY;
-    id_s[li] = 0u;
+    hi_s[li] = INFINITY;
+    if constexpr (!EX) {
+      e_s[li] = INFINITY;
+#pragma unroll
+      for (int q = 0; q < kGpend; ++q) p_s[q * cap + li] = INFINITY;
+    }
     ks[li] = in ? 1u : 0u;   // live; the first update sets the key
   }
 
@@ -796,9 +803,9 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
 
     // A worker folds the accepted centres cen[j0 .. j0 + n) (n <= kGbatch) into its
     // tokens.  A centre with d~ - eps at or above the token's upper bound cannot lower
-    // its delta.  Any other becomes one of the token's two pending centres; entries that
-    // a new upper bound excludes leave.  Pairs outside the certificate's norm range, NaN
-    // and a third pending centre are evaluated at once.
+    // its delta.  Any other becomes one of the token's pending centres; entries that a new
+    // upper bound excludes leave.  Pairs outside the certificate's norm range, NaN and a
+    // centre too many are evaluated at once.
     auto update = [&](int j0, int n) {
       const uint32_t all = (1u << n) - 1u;
       // centres whose pairs the certificate does not cover
@@ -824,7 +831,7 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
         for (int z = 0; z < 4; ++z) {
           if (s0 + z >= nslot) break;
           const int li = (s0 + z) * kGtok + li0;
-          const float ri = r_s[li], hi = fminf(e_s[li], __fadd_ru(fminf(p0_s[li], p1_s[li]), eps));
+          const float ri = r_s[li], hi = hi_s[li];
           const float thr = __fdiv_rn(1.0f - eps - hi - 1e-6f, ri);
           uint32_t low = tri_in_range(ri) ? wide : all;
 #pragma unroll
@@ -849,9 +856,10 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
           t = 32 * (blk0 + z * step) + (li & 31);
           ri = r_s[li];
           const bool in_range = tri_in_range(ri);
-          const float e = e_s[li];
-          float p0 = p0_s[li], p1 = p1_s[li], hi = fminf(e, __fadd_ru(fminf(p0, p1), eps));
-          uint32_t ids = id_s[li];
+          float hi = hi_s[li], pp[kGpend];
+          if constexpr (!EX)
+#pragma unroll
+            for (int q = 0; q < kGpend; ++q) pp[q] = p_s[q * cap + li];
           while (bt) {
             const int j = __ffs(bt) - 1;
             bt &= bt - 1;
@@ -862,29 +870,25 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
             } else if (!in_range || ((wide >> j) & 1u) || d != d) {
               now |= 1u << j;
             } else if (!(__fsub_rd(d, eps) >= hi)) {
-              const uint32_t c = __float_as_uint(cc.x);
               hi = fminf(hi, __fadd_ru(d, eps));
-              if (__fsub_rd(p0, eps) >= hi) p0 = INFINITY;
-              if (__fsub_rd(p1, eps) >= hi) p1 = INFINITY;
-              if (p0 == INFINITY) {
-                p0 = d;
-                ids = (ids & 0xffff0000u) | c;
-              } else if (p1 == INFINITY) {
-                p1 = d;
-                ids = (ids & 0xffffu) | (c << 16);
-              } else {
-                now |= 1u << j;
+              bool placed = false;
+#pragma unroll
+              for (int q = 0; q < kGpend; ++q) {
+                if (__fsub_rd(pp[q], eps) >= hi) pp[q] = INFINITY;
+                if (!placed && pp[q] == INFINITY) {
+                  pp[q] = d;
+                  id_s[q * cap + li] = (uint16_t)__float_as_uint(cc.x);
+                  placed = true;
+                }
               }
+              if (!placed) now |= 1u << j;
             }
           }
-          if constexpr (EX) {
-            e_s[li] = hi;
-            ks[li] = key_high(w_s[li], hi);
-          } else {
-            p0_s[li] = p0;
-            p1_s[li] = p1;
-            id_s[li] = ids;
-            ks[li] = key_high(w_s[li], fminf(e, __fadd_ru(fminf(p0, p1), eps)));
+          hi_s[li] = hi;
+          ks[li] = key_high(w_s[li], hi);
+          if constexpr (!EX) {
+#pragma unroll
+            for (int q = 0; q < kGpend; ++q) p_s[q * cap + li] = pp[q];
           }
         }
         __syncwarp();
@@ -906,9 +910,11 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
               e = fminf(e, distance(xv, xc, rt, cc.y));
             }
             __syncwarp();
-            if (lane == 0) {
+            if (lane == 0) {   // (hi holds d~ + eps of these centres already)
+              const float hi = fminf(e, hi_s[lt]);
               e_s[lt] = e;
-              ks[lt] = key_high(w_s[lt], fminf(e, __fadd_ru(fminf(p0_s[lt], p1_s[lt]), eps)));
+              hi_s[lt] = hi;
+              ks[lt] = key_high(w_s[lt], hi);
             }
             __syncwarp();
           }
@@ -934,19 +940,19 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       __syncthreads();
     }
     int taken = 1;
-    if (taken < K && warp > 0) update(0, 1);
+    if (taken < K && widx >= 0) update(0, 1);
     csync();   // every CTA of the cluster runs before the first remote write
 
     // ---- rounds (Eq. 10-11) ----
     const int ent = a.mc + 1;
     for (int round = 0; taken < K; ++round) {
       const int par = round & 1;
-      GramEntry *pubp = pub + (size_t)par * P * ent;
       unsigned long long *keyp = pkey + (size_t)par * P * ent;
+      float2 *pwrp = pwr + (size_t)par * P * ent;
       // 1. this warp's best live tokens by upper key, best first, into top_s: each lane
       // queues its three best.  A lane whose third is taken may hide a fourth, which is
       // below it: the third then becomes the bound.
-      if (warp > 0) {
+      if (widx >= 0) {
         unsigned long long k1 = 0ull, k2 = 0ull, k3 = 0ull, bound = 0ull;
         for (int s = 0; s < nslot; ++s) {
           const uint32_t v = ks[s * kGtok + li0];
@@ -985,19 +991,12 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
         const int esh = ent <= 4 ? 2 : ent <= 8 ? 3 : 4, e = lane & ((1 << esh) - 1);
         if (e < ent) {
           const unsigned long long kk = top_s[e];
-          uint4 v0 = make_uint4(0u, 0u, 0u, 0u), v1 = v0;
-          if (kk != 0ull) {
-            const int t = key_index(kk), li = slot_of(t);
-            v0 = make_uint4((uint32_t)t, __float_as_uint(w_s[li]), __float_as_uint(r_s[li]), id_s[li]);
-            v1 = make_uint4(ks[li], __float_as_uint(e_s[li]), __float_as_uint(p0_s[li]),
-                            __float_as_uint(p1_s[li]));
-          }
-          const int slot = (rank * kGwork + warp - 1) * ent + e;
+          const int slot = (rank * kGwork + widx) * ent + e;
+          const int li = slot_of(key_index(kk));   // (kk == 0: unused)
+          const float2 wr = kk != 0ull ? make_float2(w_s[li], r_s[li]) : make_float2(0.f, 0.f);
           for (int q = lane >> esh; q < C; q += 32 >> esh) {
             st_cluster_u64(map_shared(&keyp[slot], q), kk);
-            const uint32_t addr = map_shared(&pubp[slot], q);
-            st_cluster_v4u(addr, v0);
-            st_cluster_v4u(addr + 16, v1);
+            st_cluster_v2f(map_shared(&pwrp[slot], q), wr);
           }
         }
       }
@@ -1018,8 +1017,8 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
           base = __shfl_sync(0xffffffffu, base, 0);
           if (up) {
             const int pos = base + __popc(bal & ((1u << lane) - 1u));
-            cidx[pos] = (uint16_t)e;
             ckey[pos] = kk;
+            cidx[pos] = (uint16_t)e;
           }
         }
       }
@@ -1039,8 +1038,16 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
           pos += (x.x > kk ? 1 : 0) + (x.y > kk ? 1 : 0);
         }
         if (c < nc) {
-          if (pos < kGlist) mem[pos] = pubp[cidx[c]];
-          else if (pos == kGlist) misc[20] = kk;
+          if (pos < kGlist) {
+            const float2 wr = pwrp[cidx[c]];
+            lidx[pos] = key_index(kk);
+            lr[pos] = wr.y;
+            res[pos].z = wr.x;
+            res[pos].w = wr.y;
+            if constexpr (EX) res[pos].x = __uint_as_float((uint32_t)(kk >> 32));   // final: no owner is asked
+          } else if (pos == kGlist) {
+            misc[20] = kk;
+          }
         }
       }
       __syncthreads();
@@ -1050,102 +1057,124 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       }
       const int nL = min(nc, kGlist);
       const unsigned long long Up = nc > kGlist ? misc[20] : U;
-      unsigned long long need = 0ull;   // this warp's share of the CTA's members
-      int before = 0;
+      unsigned long long need = 0ull;   // this warp's share of the CTA's members to evaluate
       if constexpr (!EX) {
+        int before = 0;
 #pragma unroll
         for (int h = 0; h < kGper; ++h) {
           const int u = lane + 32 * h;
-          const bool mine = u < nL && owned((int)(mem[u].idx >> 5)) &&
-                            !(mem[u].p0 == INFINITY && mem[u].p1 == INFINITY);
+          const bool mine = u < nL && owned(lidx[min(u, nL - 1)] >> 5);
           const unsigned bal = __ballot_sync(0xffffffffu, mine);
           const int at = before + __popc(bal & ((1u << lane) - 1u));
-          need |= (unsigned long long)__ballot_sync(0xffffffffu, mine && at % kGwarps == warp) << (32 * h);
-          before += __popc(bal);
-        }
-        // their rows start towards L2
-        for (unsigned long long n = need; n != 0ull; n &= n - 1) {
-          const GramEntry &me = mem[__ffsll((long long)n) - 1];
-          if (lane * 128 < rb) {
-            prefetch_l2(xreq + (long long)me.idx * rb + lane * 128);
-            if (me.p0 != INFINITY) prefetch_l2(xreq + (long long)(me.ids & 0xffffu) * rb + lane * 128);
-          }
-        }
-      }
-      // 3. pairwise distances from the Gram matrix (NaN: outside the certificate): a warp
-      // takes rows u and kGlist - 1 - u together, 63 pairs
-      {
-        constexpr int kRows = kGlist / 2 / kGwarps;
-        float g[kRows][kGper];
-        int pu[kRows][kGper], pv[kRows][kGper];
+          // a member without a pending centre is exact: sent as it is
+          bool open = false;
+          if (mine && at % kGwarps == warp) {
+            const int li = slot_of(lidx[u]);
 #pragma unroll
-        for (int i = 0; i < kRows; ++i)
-#pragma unroll
-          for (int h = 0; h < kGper; ++h) {
-            const int u = warp + i * kGwarps, x = lane + 32 * h, len = kGlist - 1 - u;
-            pu[i][h] = x < len ? u : len;
-            pv[i][h] = x < len ? u + 1 + x : x + 1;
-            g[i][h] = 0.f;
-            if (pv[i][h] < nL && pu[i][h] < pv[i][h])
-              g[i][h] = __ldg(G + (long long)mem[pu[i][h]].idx * ld + mem[pv[i][h]].idx);
-          }
-#pragma unroll
-        for (int i = 0; i < kRows; ++i)
-#pragma unroll
-          for (int h = 0; h < kGper; ++h) {
-            const int u = pu[i][h], v = pv[i][h];
-            if (u < v && v < nL) {
-              const float ru = mem[u].r, rv = mem[v].r;
-              // pm[centre][token]
-              float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[i][h], rv), ru)), dt = d;
-              if constexpr (EX) dt = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[i][h], ru), rv));
-              else if (!tri_in_range(ru) || !tri_in_range(rv)) d = dt = __int_as_float(0x7fffffff);
-              pm[u * kGpairLd + v] = d;
-              pm[v * kGpairLd + u] = dt;
+            for (int q = 0; q < kGpend; ++q) open |= p_s[q * cap + li] != INFINITY;
+            if (!open) {
+              const float2 v = make_float2(__uint_as_float(ks[li]), e_s[li]);
+              for (int q = 0; q < C; ++q) st_cluster_v2f(map_shared(&res[u], q), v);
             }
           }
+          need |= (unsigned long long)__ballot_sync(0xffffffffu, open) << (32 * h);
+          before += __popc(bal);
+        }
       }
-      // the members' pending centres in the canonical order, by the CTA that owns the
-      // member, which keeps the result and sends it to every CTA: every member's delta
-      // is exact from here on
+      // the rows to evaluate start towards L2
+      if constexpr (!EX)
+        for (unsigned long long n = need; n != 0ull; n &= n - 1) {
+          const int t = lidx[__ffsll((long long)n) - 1], li = slot_of(t);
+          if (lane * 128 < rb) {
+            prefetch_l2(xreq + (long long)t * rb + lane * 128);
+#pragma unroll
+            for (int q = 0; q < kGpend; ++q)
+              if (p_s[q * cap + li] != INFINITY)
+                prefetch_l2(xreq + (long long)id_s[q * cap + li] * rb + lane * 128);
+          }
+        }
+      // 3. pairwise distances from the Gram matrix (NaN: outside the certificate): a warp
+      // takes rows u and kGlist - 1 - u together, 63 pairs; the loads are in flight while
+      // members are evaluated
+      constexpr int kRows = kGlist / 2 / kGwarps;
+      float g[kRows][kGper];
+      auto pair_of = [&](int i, int h, int *u, int *v) {
+        const int r = warp + i * kGwarps, x = lane + 32 * h, len = kGlist - 1 - r;
+        *u = x < len ? r : len;
+        *v = x < len ? r + 1 + x : x + 1;
+        return *u < *v && *v < nL;
+      };
+#pragma unroll
+      for (int i = 0; i < kRows; ++i)
+#pragma unroll
+        for (int h = 0; h < kGper; ++h) {
+          int u, v;
+          g[i][h] = pair_of(i, h, &u, &v) ? __ldg(G + (long long)lidx[u] * ld + lidx[v]) : 0.f;
+        }
+      // the CTA that owns a member evaluates its pending centres in the canonical order,
+      // keeps the result and sends (key, delta) to every CTA: every member's delta is exact
+      // from here on
       if constexpr (!EX) {
         for (; need != 0ull; need &= need - 1) {
-          const int u = __ffsll((long long)need) - 1;
-          const GramEntry me = mem[u];
-          const int c0 = (int)(me.ids & 0xffffu), c1 = (int)(me.ids >> 16);
-          const float rc0 = me.p0 != INFINITY ? rreq[c0] : 0.f, rc1 = me.p1 != INFINITY ? rreq[c1] : 0.f;
+          const int u = __ffsll((long long)need) - 1, t = lidx[u], li = slot_of(t);
+          float e = e_s[li];
+          const float w = w_s[li], r = r_s[li];
+          // nearest first: a centre whose d~ - eps is at or above e cannot lower it
           U4 xv[NCH], xc[NCH];
-          load_row((int)me.idx, xv);
-          float e = me.e;
-          if (me.p0 != INFINITY) {
-            load_row(c0, xc);
-            e = fminf(e, distance(xv, xc, me.r, rc0));
+          load_row(t, xv);
+          float pq = INFINITY;
+          int first = 0;
+#pragma unroll
+          for (int q = 0; q < kGpend; ++q)
+            if (p_s[q * cap + li] < pq) {
+              pq = p_s[q * cap + li];
+              first = q;
+            }
+#pragma unroll 1
+          for (int it = 0; it < kGpend; ++it) {
+            const int q = it == 0 ? first : it <= first ? it - 1 : it;
+            const float pd = p_s[q * cap + li];
+            if (pd == INFINITY || __fsub_rd(pd, eps) >= e) continue;
+            const int c = id_s[q * cap + li];
+            const float rc = rreq[c];
+            load_row(c, xc);
+            e = fminf(e, distance(xv, xc, r, rc));
           }
-          if (me.p1 != INFINITY) {
-            load_row(c1, xc);
-            e = fminf(e, distance(xv, xc, me.r, rc1));
-          }
-          const uint32_t kh = key_high(me.w, e);
+          const uint32_t kh = key_high(w, e);
+          __syncwarp();
           if (lane == 0) {
-            const int li = slot_of((int)me.idx);
             e_s[li] = e;
-            p0_s[li] = INFINITY;
-            p1_s[li] = INFINITY;
+            hi_s[li] = e;
             ks[li] = kh;
           }
+          if (lane < kGpend) p_s[lane * cap + li] = INFINITY;
           if (lane < C) st_cluster_v2f(map_shared(&res[u], lane), make_float2(__uint_as_float(kh), e));
         }
-        csync();
-      } else {
-        __syncthreads();
       }
+#pragma unroll
+      for (int i = 0; i < kRows; ++i)
+#pragma unroll
+        for (int h = 0; h < kGper; ++h) {
+          int u, v;
+          if (pair_of(i, h, &u, &v)) {
+            const float ru = lr[u], rv = lr[v];
+            // pm[centre][token]
+            float d = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[i][h], rv), ru)), dt = d;
+            if constexpr (EX) dt = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(g[i][h], ru), rv));
+            else if (!tri_in_range(ru) || !tri_in_range(rv)) d = dt = __int_as_float(0x7fffffff);
+            pm[u * kGpairLd + v] = d;
+            pm[v * kGpairLd + u] = dt;
+          }
+        }
+      if constexpr (EX) __syncthreads();
+      else csync();
       // 4. replay the greedy on the list (warp 0; lane u holds members u, u + 32, ..).
-      // A member's delta lies in [lo, hi]: exact until an accepted centre's distance
+      // A member's delta is at most hi, and exact until an accepted centre's distance
       // reaches below hi + eps; such centres are kept in `pend` and evaluated only when
       // the member's place in the order depends on it.
       if (warp == 0) {
         uint32_t kh[kGper], id[kGper];   // upper key (high word), token
-        float e[kGper], hi[kGper], lo[kGper], wv[kGper];
+        float e[kGper], hi[kGper], wv[kGper];
         unsigned long long pend[kGper];
 #pragma unroll
         for (int h = 0; h < kGper; ++h) {
@@ -1154,19 +1183,31 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
           id[h] = 0u;
           e[h] = wv[h] = 0.f;
           if (u < nL) {
-            const bool was = !EX && (mem[u].p0 != INFINITY || mem[u].p1 != INFINITY);   // evaluated just now
-            const float2 rv = res[u];
-            kh[h] = was ? __float_as_uint(rv.x) : mem[u].kh;
-            e[h] = was ? rv.y : mem[u].e;
-            id[h] = mem[u].idx;
-            wv[h] = mem[u].w;
+            const float4 v = res[u];
+            kh[h] = __float_as_uint(v.x);
+            e[h] = v.y;
+            wv[h] = v.z;
+            id[h] = (uint32_t)lidx[u];
           }
-          hi[h] = lo[h] = e[h];
+          hi[h] = e[h];
           pend[h] = 0ull;
         }
         const uint32_t up_hi = (uint32_t)(Up >> 32);
         int nA = 0;
         const int most = min(K - taken, kGmaxAccept);
+        // picks [j0, j0 + n) as centres for the workers (n < kGbatch ends the round)
+        auto post = [&](int j0, int n) {
+          if (lane < n) {
+            const int u = acc_s[j0 + lane], t = lidx[u];
+            cen[j0 + lane] = make_float2(__int_as_float(t), lr[u]);
+            crow[j0 + lane] = (uint32_t)t * (uint32_t)ld;   // N^2 < 2^32 (the matrix is at most 12 GiB)
+          }
+          __syncwarp();
+          if (lane == 0) {
+            cnt[4 + j0 / kGbatch] = n;
+            mbar_arrive(&bars[j0 / kGbatch]);
+          }
+        };
         while (nA < most) {
           // the member with the largest upper key (equal values: the lowest token)
           uint32_t lk = kh[0];
@@ -1206,87 +1247,81 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
             // accepted as it is only if its lower key leads every other upper key
             const int src = bl & 31;
             unsigned long long bp = 0ull;
-            uint32_t bkl = 0u, bid = 0u;
-            float bhi = 0.f, be = 0.f;
             uint32_t second = 0u;   // best other upper key (high word)
+            float bhi = 0.f, be = 0.f;
 #pragma unroll
             for (int h = 0; h < kGper; ++h) {
               if (lane + 32 * h == bl) {
                 bp = pend[h];
-                bkl = lo[h] == -INFINITY ? 0u : key_high(wv[h], lo[h]);
                 bhi = hi[h];
                 be = e[h];
-                bid = id[h];
               } else {
                 second = max(second, kh[h]);
               }
             }
-            bkl = __shfl_sync(0xffffffffu, bkl, src);
+            bp = shfl_u64(bp, src);
+            be = __shfl_sync(0xffffffffu, be, src);
             second = __reduce_max_sync(0xffffffffu, second);
-            if (!(bkl > up_hi && bkl > second)) {
-              bp = shfl_u64(bp, src);
-              bid = __shfl_sync(0xffffffffu, bid, src);
+            // the lower end: e or the nearest pending centre less eps (NaN: none)
+            const float bw = res[bl].z;
+            uint32_t low = key_high(bw, be);
+#pragma unroll
+            for (int h = 0; h < kGmaxAccept / 32; ++h) {
+              const int j = lane + 32 * h;
+              if ((bp >> j) & 1ull) {
+                const float d = __fsub_rd(pm[acc_s[j] * kGpairLd + bl], eps);
+                low = min(low, d == d ? key_high(bw, d) : 0u);
+              }
+            }
+            low = __reduce_min_sync(0xffffffffu, low);
+            if (!(low > up_hi && low > second)) {
               bhi = __shfl_sync(0xffffffffu, bhi, src);
-              be = __shfl_sync(0xffffffffu, be, src);
               U4 xv[NCH], xc[NCH];
-              load_row((int)bid, xv);
+              load_row(lidx[bl], xv);
               while (bp) {
                 const int j = __ffsll((long long)bp) - 1;
                 bp &= bp - 1;
                 const int cj = acc_s[j];
                 if (__fsub_rd(pm[cj * kGpairLd + bl], eps) >= bhi) continue;   // excluded since
-                load_row((int)mem[cj].idx, xc);
-                be = fminf(be, distance(xv, xc, mem[bl].r, mem[cj].r));
+                load_row(lidx[cj], xc);
+                be = fminf(be, distance(xv, xc, res[bl].w, res[cj].w));
               }
 #pragma unroll
               for (int h = 0; h < kGper; ++h)
-                if (32 * h <= bl && bl < 32 * (h + 1)) {
-                  if (lane == src) {
-                    pend[h] = 0ull;
-                    e[h] = hi[h] = lo[h] = be;
-                    kh[h] = key_high(wv[h], be);
-                  }
+                if (lane + 32 * h == bl) {
+                  pend[h] = 0ull;
+                  e[h] = hi[h] = be;
+                  kh[h] = key_high(wv[h], be);
                 }
               continue;
             }
           }
-          const uint32_t bidx = mem[bl].idx;
-          const float brn = mem[bl].r;
           const unsigned long long bit = 1ull << nA;
 #pragma unroll
           for (int h = 0; h < kGper; ++h) {
             const int u = lane + 32 * h;
             const float d = pm[bl * kGpairLd + u];
-            if constexpr (EX) {
-              hi[h] = fminf(hi[h], d);
+            if (EX) {   // w min(delta, d) = min(w delta, w d); NaN has the largest key
+              kh[h] = kh[h] == 0u || u == bl ? 0u : min(kh[h], key_high(wv[h], d));
+              continue;
             } else {
-              const float dlo = __fsub_rd(d, eps), dhi = __fadd_ru(d, eps);
-              const bool hit = !(dlo >= hi[h]);   // NaN too
-              pend[h] |= hit ? bit : 0ull;
-              lo[h] = hit ? (d == d ? fminf(lo[h], dlo) : -INFINITY) : lo[h];
-              hi[h] = hit ? fminf(hi[h], dhi) : hi[h];   // NaN keeps hi
+              if (!(__fsub_rd(d, eps) >= hi[h])) pend[h] |= bit;   // NaN too
+              hi[h] = fminf(hi[h], __fadd_ru(d, eps));             // (above hi unless pending; NaN keeps it)
             }
             kh[h] = kh[h] == 0u || u == bl ? 0u : key_high(wv[h], hi[h]);
           }
-          // posted; every eighth centre releases a batch to the workers
-          if (lane == 0) {
-            acc_s[nA] = bl;
-            cen[nA] = make_float2(__uint_as_float(bidx), brn);
-            crow[nA] = bidx * (uint32_t)ld;   // N^2 < 2^32 (the matrix is at most 12 GiB)
-            if (nA % kGbatch == kGbatch - 1) {
-              cnt[4 + nA / kGbatch] = kGbatch;
-              mbar_arrive(&bars[nA / kGbatch]);
-            }
-          }
+          if (lane == 0) acc_s[nA] = bl;
           __syncwarp();
           ++nA;
+          if (nA % kGbatch == 0) post(nA - kGbatch, kGbatch);
         }
         if (lane == 0) cnt[2] = nA;
-        if (lane >= nA / kGbatch && lane < kGmaxAccept / kGbatch) {
-          cnt[4 + lane] = lane == nA / kGbatch ? nA % kGbatch : 0;
-          mbar_arrive(&bars[lane]);
+        if (nA < kGmaxAccept) {
+          post(nA / kGbatch * kGbatch, nA % kGbatch);
+          // the batches that this round does not reach complete too: one phase a round
+          if (lane > nA / kGbatch && lane < kGmaxAccept / kGbatch) mbar_arrive(&bars[lane]);
         }
-      } else {
+      } else if (widx >= 0) {
         // 5. meanwhile the workers fold the accepted centres into their tokens
         for (int i = 0; i < kGmaxAccept / kGbatch; ++i) {
           mbar_wait_bounded(&bars[i], par, a.err, kErrTimeout);
@@ -1298,7 +1333,7 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       __syncthreads();
       const int nA = cnt[2];
       if (tid < nA) {
-        const int gi = (int)mem[acc_s[tid]].idx, k = gi >> 5;
+        const int gi = lidx[acc_s[tid]], k = gi >> 5;
         atomicOr(&sel[k], 1u << (gi & 31));
         if (owned(k)) ks[slot_of(gi)] = 0u;
       }
@@ -1310,7 +1345,7 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
 
   // ---- Eq. 12: ascending positions from the request's selected bits; every CTA
   // writes the indices and rows of its own blocks ----
-  int2 *out = reinterpret_cast<int2 *>(smem + S.e);   // (token, position) of the kept tokens, over e and p0
+  int2 *out = reinterpret_cast<int2 *>(smem + S.e);   // (token, position) of the kept tokens, over e and hi
   int *wsum = reinterpret_cast<int *>(misc);
   if (tid == 0) cnt[0] = 0;
   int run = 0;
@@ -1467,32 +1502,42 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
       const size_t smem = (size_t)kExBufs * (kExRows + cols) * 256 * pl.elem;
       e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(pl.gram_tiles);
+      cfg.blockDim = dim3(16 * cols);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = s;
+      cudaLaunchAttribute attr[1];   // beside the norms' kernel, as below
+      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[0].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
       void *args[] = {&x1};
-      if ((e = cudaLaunchKernel(fn, dim3(pl.gram_tiles), dim3(16 * cols), args, smem, s)) != cudaSuccess) return e;
+      if ((e = cudaLaunchKernelExC(&cfg, fn, args)) != cudaSuccess) return e;
     } else {
-    // the matrix needs no norms: its kernel starts beside the norms' and ends after them
-    void *fn = pair ? (void *)gram_pair_kernel : (void *)gram_kernel;
-    const size_t smem = 192 * 1024 + 1024;
-    static_assert(kGramStages * kGramStageBytes == 192 * 1024 && kPairStages * kPairStageBytes == 192 * 1024,
-                  "the ring of either kernel");
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(pair ? 2 * std::min(sms / 2, pl.gram_tiles) : std::min(sms, pl.gram_tiles));
-    cfg.blockDim = dim3(kGramThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = pair ? 2 : 1;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    void *args[] = {&g};
-    if ((e = cudaLaunchKernelExC(&cfg, fn, args)) != cudaSuccess) return e;
+      // the matrix needs no norms: its kernel starts beside the norms' and ends after them
+      void *fn = pair ? (void *)gram_pair_kernel : (void *)gram_kernel;
+      const size_t smem = 192 * 1024 + 1024;
+      static_assert(kGramStages * kGramStageBytes == 192 * 1024 && kPairStages * kPairStageBytes == 192 * 1024,
+                    "the ring of either kernel");
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(pair ? 2 * std::min(sms / 2, pl.gram_tiles) : std::min(sms, pl.gram_tiles));
+      cfg.blockDim = dim3(kGramThreads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = s;
+      cudaLaunchAttribute attr[2];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = pair ? 2 : 1;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[1].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 2;
+      void *args[] = {&g};
+      if ((e = cudaLaunchKernelExC(&cfg, fn, args)) != cudaSuccess) return e;
     }
   }
   GramSelArgs a;
@@ -1513,13 +1558,16 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   cfg.blockDim = dim3(kGthreads);
   cfg.dynamicSmemBytes = sh.smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = sh.C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  // (behind the tensor-core kernels an early start cost 1% on long requests)
+  cfg.numAttrs = pl.gram_exact ? 2 : 1;
   void *args[] = {&a};
   *done = true;
   return cudaLaunchKernelExC(&cfg, sel_fn, args);
