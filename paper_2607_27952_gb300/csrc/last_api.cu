@@ -163,14 +163,18 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
     for (int b = 0; b < B; ++b) units += gram_units(b);
   // Used where the contraction over the lower triangle (about 1.1 PFLOP/s on tensor
   // cores, 20 T fma/s in the canonical order) costs less than the rounds over X that it
-  // replaces: those accept about 16 picks a round and take about 100 us each, and the
-  // longest request's rounds set the call's time.  Eight requests of 16384 x 2048: 3.0 ms
-  // against 16.6 ms at k = 2048, 8.5 ms at 1024; the line lies near k = 700.
+  // replaces.  bf16, matrix / rounds over X, us: 8 requests of 16384 x 2048 at k = 32 3169 /
+  // 3102, 64 3337 / 3707, 400 3622 / 7732; one of them at k = 8 456 / 1404; 16 of 4096 x
+  // 1536 at 8 475 / 937; 64 of 576 x 2048 at 4 148 / 387: the line lies near 0.12 ms a pick
+  // for matrices of several ms and below any budget for small ones.  fp32: 576 x 1024 at
+  // k = 2 39 / 30, 4 43 / 46; two of 2048 at 32 350 / 319, 64 378 / 598; four of 4096 at
+  // 128 2456 / 1585; 10000 at 128 3551 / 3313: 6 us a pick.
   const double fmas = 0.5 * (double)units * 32.0 * p->feat_dim;
   const double tensor_s = 2.0 * fmas / 1.1e15, exact_s = fmas / 20e12;
-  pl->gram_exact = p->dtype == LAST_DTYPE_F32 || exact_s <= kGramExactSeconds;
+  const bool f32 = p->dtype == LAST_DTYPE_F32;
+  pl->gram_exact = f32 || exact_s <= kGramExactSeconds;
   pl->gram = units > 0 && units * 128 <= kGramMaxBytes &&
-             (pl->gram_exact ? exact_s : tensor_s) <= 6e-6 * pl->max_keep;
+             (f32 ? exact_s <= 6e-6 * pl->max_keep : tensor_s <= std::max(0.8e-3, 1.2e-4 * pl->max_keep));
   if (pl->gram) {
     pl->off_rn = o;
     o = align_up(o + sizeof(float) * (size_t)pl->total_vis);

@@ -7,6 +7,7 @@ range.  Indices and rows are exact against the oracle."""
 import numpy as np
 import pytest
 
+import oracle
 import paper_2607_27952_gb300 as last
 from gpu_util import (assert_gather_equal, assert_selection_equal, oracle_selection,
                       problem_of, to_dev, to_host_bits)
@@ -66,3 +67,27 @@ def test_ties_zero_rows_and_extreme_norms(dtype, n):
     w[:5] = 0.0
     w, idx, _ = _run(wl, w=w)
     assert np.array_equal(idx, np.sort(oracle_selection(wl, w, 0)))
+
+
+@pytest.mark.parametrize("batch,k", [(13, 200), (8, 20)])
+def test_batches_past_the_matrix_keep_the_rounds_over_x(batch, k):
+    """13 requests of 16384 tokens are past the matrices' 12 GiB, 8 with 20 picks are
+    cheaper without them: the clustered kernel that streams X (and skips rows) takes both.
+    One request's features repeated, other weights per request."""
+    import torch
+    n, d = 16384, 2048
+    rng = np.random.default_rng(8)
+    x = rng.standard_normal((n // 512, 512, d), dtype=np.float32)
+    x[1:] *= 0.05
+    x = f32_to_bf16_bits(np.cumsum(x, 0).reshape(n, d))
+    w = (1.0 + 0.01 * rng.random((batch, n))).astype(np.float32)
+    prob = last.Problem(batch=batch, num_layers=0, num_q_heads=0, num_kv_heads=0, head_dim=0, feat_dim=d,
+                        dtype="bf16", cu_seqlens=None, vis_start=None, cu_vis=np.arange(batch + 1) * n,
+                        cu_keep=np.arange(batch + 1) * k)
+    ws = last.workspace(prob, "cuda:0")
+    idx = torch.full((batch * k,), -7, dtype=torch.int32, device="cuda:0")
+    last.last_select(prob, torch.from_numpy(w).cuda(), to_dev(x, torch.device("cuda:0")).repeat(batch, 1), idx, ws)
+    last.last_poll(ws)
+    got = idx.cpu().numpy().reshape(batch, k)
+    for b in (0, batch - 1):
+        assert np.array_equal(got[b], np.sort(oracle.select_fp32(x, w[b], k)))
