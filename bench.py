@@ -503,7 +503,7 @@ def earlier_capture(kernel_source, workload, select_ms, hbm):
 
 
 def selection_roofline(wl, select_ms, hbm, bf16_peak, traffic):
-    """Roofline of select_kernel against real resources.  `achieved` is the DRAM
+    """Roofline of the selection against real resources.  `achieved` is the DRAM
     rate: bytes per launch recorded by ncu for this workload and kernel source
     (`traffic`), else the compulsory bytes (a lower bound on what crosses DRAM),
     over the event time; `tensor_frac` is the greedy's full distance contraction
@@ -512,7 +512,7 @@ def selection_roofline(wl, select_ms, hbm, bf16_peak, traffic):
     comp = select_compulsory_bytes(wl)
     dram = traffic if traffic is not None else comp
     achieved = dram / sec / 1e9
-    return {"bound": "hbm", "kernel": "select_kernel", "achieved": achieved, "peak": hbm,
+    return {"bound": "hbm", "kernel": "norms + gram + select_gram kernels (last_select)", "achieved": achieved, "peak": hbm,
             "unit": "GB/s", "frac": achieved / hbm, "traffic": traffic,
             "achieved_basis": ("ncu dram__bytes_read.sum + dram__bytes_write.sum per launch"
                                if traffic is not None else
@@ -575,7 +575,7 @@ def measure_config(name, budget, rank, dev, last, seconds, hbm, bf16_peak):
     sc = statistics.mean(e[0].elapsed_time(e[1]) for e in ev)
     se = statistics.mean(e[1].elapsed_time(e[2]) for e in ev)
     key = f"{name}-{budget}"
-    traffic = measured_traffic("select_impl.cuh", key)
+    traffic = measured_traffic("select_gram.cu", key)
     rl = selection_roofline(wl, se, hbm, bf16_peak, traffic)
     sc_gbs = score_bytes(wl) / (sc / 1e3) / 1e9
     out = {"workload": workload_desc(wl, budget, name)["workload"], "dtype": workload_dtype(wl),
@@ -586,7 +586,7 @@ def measure_config(name, budget, rank, dev, last, seconds, hbm, bf16_peak):
            "select_dram_frac": rl["frac"] if traffic is not None else None,
            "select_compulsory_frac": rl["compulsory_frac"],
            "select_tensor_frac": rl["tensor_frac"], "select_dram_bytes": traffic}
-    out |= earlier_capture("select_impl.cuh", key, se, hbm)
+    out |= earlier_capture("select_gram.cu", key, se, hbm)
     del q, k, x, w, idx, xs, ws
     torch.cuda.empty_cache()
     return out
@@ -708,18 +708,18 @@ def main():
         "config": workload_desc(wl, args.budget, args.workload) | {"parallelism": f"replicas x{world}"},
         "visual_tokens_scored_per_s": tokens_per_s,
         # per step: scoring (logits + tokens, or the four multi-row passes) and the
-        # selection (select_kernel, or topk_kernel + gather_kernel)
+        # selection (norms, Gram matrix and greedy, or topk_kernel + gather_kernel)
         "gpu_launches": (scoring_kernels(wl, None if rows is None else rows_host[0]) +
-                         (2 if topk else 1)) * K,
+                         (2 if topk else 3)) * K,
         "kernels": {"scores_ms": scores_ms, "select_ms": select_ms,
                     "scores_ms_median": statistics.median(scores_all),
                     "select_ms_median": statistics.median(select_all),
                     "scores_GBps": sc_gbs, "scores_hbm_frac": sc_gbs / hbm},
         "roofline": selection_roofline(wl, select_ms, hbm, bf16_peak,
-                                       measured_traffic("select_impl.cuh", key))
+                                       measured_traffic("select_gram.cu", key))
                     | {"peak_note": f"{pk_kind} HBM copy bandwidth (of {pk_kind}); tensor peak: "
                                     f"{pk_kind} cuBLAS bf16 burst"}
-                    | earlier_capture("select_impl.cuh", key, select_ms, hbm),
+                    | earlier_capture("select_gram.cu", key, select_ms, hbm),
         "clocks": clocks,
         "prune_bytes_moved": {"compulsory_bytes": comp, "greedy_feature_bytes": greedy,
                               "compulsory_frac": comp / (total_ms / K / 1e3) / 1e9 / hbm,
@@ -767,7 +767,7 @@ def main():
             per[f"{name}-{bud}"] = measure_config(name, bud, rank, dev, last,
                                                   args.per_config_seconds, hbm, bf16_peak)
         line["per_config"] = per
-        line["gpu_launches"] += 3 * sum(v["steps"] for v in per.values())
+        line["gpu_launches"] += 5 * sum(v["steps"] for v in per.values())
     if rank == 0:
         print(json.dumps(line), flush=True)
     if world > 1:
