@@ -45,6 +45,8 @@ struct ScoreArgs {
 
 constexpr int kSegBatch = 8;        // 16-byte loads in flight per lane
 constexpr int kRowsPerTask = 16;    // keys of one warp task (two lanes per key)
+constexpr int kScoreWarps = kScoreThreads / 32;
+constexpr int kStatHeads = 2;       // heads whose statistics a warp forms together
 
 template <typename T, int G>
 __global__ void __launch_bounds__(kScoreThreads, 3)
@@ -174,39 +176,57 @@ score_logits_kernel(const ScoreArgs a) {
     }
     __syncthreads();
 
-    // per-head chunk statistics: max, sums of 2^(z - max) over all and over visual keys
+    // per-head chunk statistics: max, sums of 2^(z - max) over all and over visual keys,
+    // and the visual logits.  The phase is a chain of shared-memory reads and shuffles, no
+    // key load is in flight in it: two heads a warp side by side (their chains overlap) and
+    // the logits stored from the same pass, without an index division per element.  32
+    // requests x 2880 keys x 4 layers, both scoring kernels: 133 -> 121 us, one head at a
+    // time against two; four 131 us (heads past the last are formed twice).
     const int vlo = max(p_begin, v0), vhi = min(p_begin + nk, v0 + nvis);
-    for (int h = warp; h < Hq; h += kScoreThreads / 32) {
-      float mx = -INFINITY;
-      for (int kk = lane; kk < nk; kk += 32) mx = fmaxf(mx, zbuf[kk * ldz + h]);
+    for (int h0 = warp; h0 < Hq; h0 += kScoreWarps * kStatHeads) {
+      float mx[kStatHeads], sum[kStatHeads], vis[kStatHeads];
+      int hh[kStatHeads];   // past the last head: the first one again, not stored
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      float sum = 0.f, vis = 0.f;
+      for (int u = 0; u < kStatHeads; ++u) {
+        hh[u] = h0 + u * kScoreWarps < Hq ? h0 + u * kScoreWarps : h0;
+        mx[u] = -INFINITY;
+        sum[u] = vis[u] = 0.f;
+      }
+      for (int kk = lane; kk < nk; kk += 32)
+#pragma unroll
+        for (int u = 0; u < kStatHeads; ++u) mx[u] = fmaxf(mx[u], zbuf[kk * ldz + hh[u]]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < kStatHeads; ++u) mx[u] = fmaxf(mx[u], __shfl_xor_sync(0xffffffffu, mx[u], o));
       for (int kk = lane; kk < nk; kk += 32) {
-        const float e = exp2f(zbuf[kk * ldz + h] - mx);
-        sum += e;
         const int p = p_begin + kk;
-        if (p >= vlo && p < vhi) vis += e;
+        const bool v = p >= vlo && p < vhi;
+        float *zl = a.zlog + (long long)l * Hq * a.total_vis + voff + (p - v0);
+#pragma unroll
+        for (int u = 0; u < kStatHeads; ++u) {
+          const float z = zbuf[kk * ldz + hh[u]];
+          const float e = exp2f(z - mx[u]);
+          sum[u] += e;
+          if (v) {
+            vis[u] += e;
+            if (h0 + u * kScoreWarps < Hq) zl[(long long)hh[u] * a.total_vis] = z;
+          }
+        }
       }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        vis += __shfl_xor_sync(0xffffffffu, vis, o);
-      }
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < kStatHeads; ++u) {
+          sum[u] += __shfl_xor_sync(0xffffffffu, sum[u], o);
+          vis[u] += __shfl_xor_sync(0xffffffffu, vis[u], o);
+        }
       if (lane == 0)
-        a.stats[((long long)l * Hq + h) * a.total_chunks + cbase + chunk] =
-            make_float4(mx, sum, vis, 0.f);
-    }
-
-    // visual logits of this chunk
-    const int nv = vhi - vlo;
-    if (nv > 0) {
-      for (int idx = tid; idx < nv * Hq; idx += kScoreThreads) {
-        const int h = idx / nv, i = idx - h * nv;
-        const int p = vlo + i;
-        a.zlog[((long long)l * Hq + h) * a.total_vis + voff + (p - v0)] =
-            zbuf[(p - p_begin) * ldz + h];
-      }
+#pragma unroll
+        for (int u = 0; u < kStatHeads; ++u)
+          if (h0 + u * kScoreWarps < Hq)
+            a.stats[((long long)l * Hq + hh[u]) * a.total_chunks + cbase + chunk] =
+                make_float4(mx[u], sum[u], vis[u], 0.f);
     }
   }
   // the token kernel (launched as a programmatic dependent) may start its

@@ -141,6 +141,19 @@ def test_feature_widths(dv):
     assert_gather_equal(wl, idx, xs, range(wl.batch))
 
 
+@pytest.mark.parametrize("heads,kv", [(1, 1), (9, 3), (17, 17), (24, 4), (25, 5)])
+def test_head_counts_around_the_statistics_pairs(heads, kv):
+    """A warp forms the statistics of heads h and h + 8 together: counts below, at and past
+    whole pairs, chunks that end inside a warp's stride."""
+    wl = custom(name=f"heads{heads}", seed=70 + heads, batch=3, n_vis=[130, 33, 250],
+                n_text=[3, 1, 7], n_before=[0, 1, 5], num_layers=2, num_q_heads=heads,
+                num_kv_heads=kv, head_dim=64, feat_dim=64, dtype="bf16", keep=[2, 1, 3],
+                n_clusters=4, n_planted=2)
+    w_ref = oracle.scores(wl.q, wl.k, wl.cu_seqlens, wl.vis_start, wl.cu_vis,
+                          num_kv_heads=wl.num_kv_heads, scale=wl.scale)
+    assert_scores_close(DeviceWorkload(wl).scores(), w_ref, wl)
+
+
 def test_identical_and_orthogonal_features():
     """Special cases with textbook answers run through the kernels."""
     import torch
