@@ -751,8 +751,8 @@ def main():
         line["config"]["source"] = f"{args.source} ({int(cu[-1])} query rows, Table 4)"
         line["kernels"]["scores_tensor_TFLOPs"] = flops / (scores_ms / 1e3) / 1e12
         if topk and scoring_kernels(wl, cu) == 4:
-            line["roofline"]["kernel"] = ("rows_stats_kernel+rows_merge_kernel+"
-                                          "rows_probs_kernel+rows_final_kernel")
+            line["roofline"]["kernel"] = ("rows_pass_kernel+rows_merge_kernel+"
+                                          "rows_pass_kernel+rows_final_kernel")
     if e2e is not None:
         line["e2e"] = e2e
     if rank == 0 and not args.no_cpu_baseline:
