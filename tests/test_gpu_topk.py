@@ -1,5 +1,9 @@
 """GPU parity of the Top-k selection variant (Table 5) against the oracle,
 through the C ABI: kept indices and gathered rows bit-exact on identical scores."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -172,3 +176,27 @@ def test_threshold_ties_and_shared_leading_bits(n, kind):
         last.last_select_topk(prob, torch.from_numpy(w).cuda(), idx, last.workspace(prob, "cuda:0"))
         want = np.sort(np.argsort(-w, kind="stable")[:k])
         assert np.array_equal(idx.cpu().numpy(), want)
+
+
+_FIRST_CALL = """
+import sys
+import numpy as np, torch
+import paper_2607_27952_gb300 as last
+n = int(sys.argv[1]); k = n // 5
+w = np.random.default_rng(n).random(n).astype(np.float32)
+prob = last.Problem(batch=1, num_layers=0, num_q_heads=0, num_kv_heads=0, head_dim=0, feat_dim=8,
+                    dtype="bf16", cu_seqlens=None, vis_start=None, cu_vis=[0, n], cu_keep=[0, k])
+idx = torch.full((k,), -7, dtype=torch.int32, device="cuda:0")
+last.last_select_topk(prob, torch.from_numpy(w).cuda(), idx, last.workspace(prob, "cuda:0"))
+assert np.array_equal(idx.cpu().numpy(), np.sort(np.argsort(-w, kind="stable")[:k]))
+"""
+
+
+@pytest.mark.parametrize("n", [10172, 10240, 11000, 12288])
+def test_first_call_of_a_process_around_the_default_shared_memory(n):
+    """Scores and the kernel's own arrays pass the 48 KB default together from 10173
+    tokens on, the scores alone from 12289: the first Top-k call of a process (no earlier
+    one has raised the limit) runs at all of them."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FIRST_CALL, str(n)], cwd=root, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
