@@ -1324,7 +1324,11 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       } else if (widx >= 0) {
         // 5. meanwhile the workers fold the accepted centres into their tokens
         for (int i = 0; i < kGmaxAccept / kGbatch; ++i) {
-          mbar_wait_bounded(&bars[i], par, a.err, kErrTimeout);
+          // an expired wait (the call is reported as failed): nothing that the replay may
+          // not have posted is read, cen and crow would be offsets into the matrix.  The
+          // rounds go on, in step with the cluster, and end after at most K picks.
+          const bool posted = mbar_wait_bounded(&bars[i], par, a.err, kErrTimeout);
+          if (!__all_sync(0xffffffffu, posted)) break;
           const int n = cnt[4 + i];
           if (n > 0) update(i * kGbatch, n);
           if (n < kGbatch) break;
