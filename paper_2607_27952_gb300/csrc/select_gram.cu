@@ -982,6 +982,7 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
             k3 = 0ull;
           }
         }
+        __syncwarp();   // the winners' entries, before lane 0 reads and rewrites the last one
         if (nslot > 3 && __any_sync(0xffffffffu, left == 0)) {
           bound = warp_max_u64(bound);
           if (lane == 0) top_s[a.mc] = max(top_s[a.mc], bound);

@@ -91,3 +91,25 @@ def test_batches_past_the_matrix_keep_the_rounds_over_x(batch, k):
     got = idx.cpu().numpy().reshape(batch, k)
     for b in (0, batch - 1):
         assert np.array_equal(got[b], np.sort(oracle.select_fp32(x, w[b], k)))
+
+
+def test_best_tokens_on_one_lane_of_every_warp():
+    """A lane queues its three best tokens, the third of them taken bounds the rest.  Every
+    token of weight sits on the same lane (tokens are dealt in blocks of 32), and so many
+    requests run on one CTA each, whose warps hold four or five blocks."""
+    import torch
+    batch, n, d, k = 150, 2100, 512, 40
+    rng = np.random.default_rng(9)
+    x = f32_to_bf16_bits(rng.standard_normal((n, d), dtype=np.float32))
+    at = np.arange(n)
+    w = np.where(at % 32 == 5, 1.0 + rng.random((batch, n)), 1e-3 * rng.random((batch, n))).astype(np.float32)
+    prob = last.Problem(batch=batch, num_layers=0, num_q_heads=0, num_kv_heads=0, head_dim=0, feat_dim=d,
+                        dtype="bf16", cu_seqlens=None, vis_start=None, cu_vis=np.arange(batch + 1) * n,
+                        cu_keep=np.arange(batch + 1) * k)
+    ws = last.workspace(prob, "cuda:0")
+    idx = torch.full((batch * k,), -7, dtype=torch.int32, device="cuda:0")
+    last.last_select(prob, torch.from_numpy(w).cuda(), to_dev(x, torch.device("cuda:0")).repeat(batch, 1), idx, ws)
+    last.last_poll(ws)
+    got = idx.cpu().numpy().reshape(batch, k)
+    for b in (0, 70, batch - 1):
+        assert np.array_equal(got[b], np.sort(oracle.select_fp32(x, w[b], k)))
