@@ -221,6 +221,11 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, uint3
   atomicOr(err, flag);
   return false;
 }
+// After a wait has expired: lets asynchronous work in flight finish before its CTA exits
+// (`never`: an initialised barrier that nothing completes).  Bounded like every wait.
+__device__ __forceinline__ void wait_out(unsigned long long *never) {
+  for (int i = 0; i < 1 << 14; ++i) mbar_try_wait(never, 0);
+}
 
 // ---- tcgen05 (5th-generation tensor cores), TMA tensor loads ----
 // Shared-memory matrix descriptor for a K-major operand stored in the 128-byte

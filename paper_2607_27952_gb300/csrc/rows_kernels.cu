@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) rows_pass_kernel(const __grid
   __shared__ unsigned long long full[kRowsMaxStages], empty[kRowsMaxStages];
   __shared__ unsigned long long afull[kRowsGroups], aempty[kRowsGroups], never;
   __shared__ uint32_t tslot;
+  __shared__ volatile int gave_up;   // a role's wait has expired
   __shared__ float4 part[kRowsGroups][4][32];   // pass 1: the warps' statistics of 32 columns
   __shared__ float2 cf[kRowsGroups][kRowsMaxN]; // pass 2: the item's (max, 1 / Z)
   __shared__ float bmax[kRowsGroups * 4][32];   // pass 1: a warp's column maxima
@@ -118,6 +119,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) rows_pass_kernel(const __grid
     }
     mbar_init(&never, 1);
     fence_mbar_init();
+    gave_up = 0;
   }
   const uint32_t tmem_total = a.tmem_cols * (uint32_t)ngroup;
   if (warp == 0) tmem_alloc(&tslot, tmem_total);
@@ -127,7 +129,10 @@ __global__ void __launch_bounds__(kPassThreads, 1) rows_pass_kernel(const __grid
   const uint32_t tmem = tslot;
   bool dead = false;   // after one expired wait a role's others return at once
   auto twait = [&](unsigned long long *bar, uint32_t par) -> bool {
-    if (!dead && !mbar_wait_bounded(bar, par, a.err, kErrTimeout)) dead = true;
+    if (!dead && !mbar_wait_bounded(bar, par, a.err, kErrTimeout)) {
+      dead = true;
+      gave_up = 1;
+    }
     return !dead;
   };
   const int2 *items = STATS ? a.items1 : a.items2;
@@ -164,9 +169,6 @@ __global__ void __launch_bounds__(kPassThreads, 1) rows_pass_kernel(const __grid
           ph ^= 1u;
         }
       }
-      // an aborted call: time for the last copies to land before the CTA may exit
-      if (dead)
-        for (int i = 0; i < 1 << 14; ++i) mbar_try_wait(&never, 0);
     }
   } else if (warp == 4 * kRowsGroups + 1) {
     if (lane == 0) {
@@ -308,6 +310,10 @@ __global__ void __launch_bounds__(kPassThreads, 1) rows_pass_kernel(const __grid
     }
   }
   __syncthreads();
+  if (gave_up) {   // an aborted call: time for copies and MMAs in flight before the CTA may exit
+    if (threadIdx.x == 0) wait_out(&never);
+    __syncthreads();
+  }
   tc_fence_after();
   if (warp == 0) tmem_dealloc(tmem, tmem_total);
 }

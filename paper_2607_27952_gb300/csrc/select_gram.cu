@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   __shared__ unsigned long long full[kGramStages], empty[kGramStages], afull[2], aempty[2], never;
   __shared__ uint32_t tslot;   // TMEM base
+  __shared__ volatile int gave_up;   // a role's wait has expired
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nkb = tc_kblocks(a.dv);
   if (threadIdx.x == 0) {
@@ -170,6 +171,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
     }
     mbar_init(&never, 1);
     fence_mbar_init();
+    gave_up = 0;
   }
   if (warp == 0) tmem_alloc(&tslot, 512);
   tc_fence_before();
@@ -179,7 +181,10 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
   // a role's waits: after one has expired the others return at once and the call reports it
   bool dead = false;
   auto twait = [&](unsigned long long *bar, uint32_t par) -> bool {
-    if (!dead && !mbar_wait_bounded(bar, par, a.err, kErrTimeout)) dead = true;
+    if (!dead && !mbar_wait_bounded(bar, par, a.err, kErrTimeout)) {
+      dead = true;
+      gave_up = 1;
+    }
     return !dead;
   };
   // tile -> (request, row block, column block)
@@ -228,9 +233,6 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
           }
         }
       }
-      // an aborted call: time for the last copies to land before the CTA may exit
-      if (dead)
-        for (int i = 0; i < 1 << 14; ++i) mbar_try_wait(&never, 0);
     }
   } else if (warp == 9) {
     if (lane == 0) {
@@ -297,6 +299,10 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_kernel(const __grid_cons
     }
   }
   __syncthreads();
+  if (gave_up) {   // an aborted call: time for copies and MMAs in flight before the CTA may exit
+    if (threadIdx.x == 0) wait_out(&never);
+    __syncthreads();
+  }
   tc_fence_after();
   if (warp == 0) tmem_dealloc(tmem, 512);
   asm volatile("griddepcontrol.wait;" ::: "memory");   // the norms too are done when this grid is
@@ -320,6 +326,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_pair_kernel(const __grid
   // full, aempty: of the even CTA (its barriers count both CTAs); empty, afull: each CTA's
   __shared__ unsigned long long full[kPairStages], empty[kPairStages], afull[2], aempty[2], never;
   __shared__ uint32_t tslot;   // TMEM base
+  __shared__ volatile int gave_up;   // a role's wait has expired, in either CTA
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const int nkb = tc_kblocks(a.dv);
@@ -334,6 +341,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_pair_kernel(const __grid
     }
     mbar_init(&never, 1);
     fence_mbar_init();
+    gave_up = 0;
   }
   if (warp == 0) tmem_alloc_pair(&tslot, 512);
   tc_fence_before();
@@ -342,7 +350,10 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_pair_kernel(const __grid
   const uint32_t tmem = tslot;
   bool dead = false;
   auto twait = [&](unsigned long long *bar, uint32_t par) -> bool {
-    if (!dead && !mbar_wait_bounded(bar, par, a.err, kErrTimeout)) dead = true;
+    if (!dead && !mbar_wait_bounded(bar, par, a.err, kErrTimeout)) {
+      dead = true;
+      for (int r = 0; r < 2; ++r) st_cluster_s32(map_shared(const_cast<int *>(&gave_up), r), 1);
+    }
     return !dead;
   };
   auto decode = [&](int tile, int *b_, int *ti, int *tj) {
@@ -393,10 +404,6 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_pair_kernel(const __grid
           }
         }
       }
-      // an aborted call: time for the last copies to land (their barrier may be the
-      // other CTA's) before the CTA may exit
-      if (dead)
-        for (int i = 0; i < 1 << 14; ++i) mbar_try_wait(&never, 0);
     }
   } else if (warp == 9) {
     if (lane == 0 && rank == 0) {
@@ -462,6 +469,11 @@ __global__ void __launch_bounds__(kGramThreads, 1) gram_pair_kernel(const __grid
   __syncwarp();
   tc_fence_before();
   cluster_sync();   // both CTAs are done with either's barriers, operands and accumulators
+  if (gave_up) {   // an aborted call: time for copies and MMAs in flight before either may exit
+    if (threadIdx.x == 0) wait_out(&never);
+    __syncwarp();
+    cluster_sync();
+  }
   tc_fence_after();
   if (warp == 0) tmem_dealloc_pair(tmem, 512);
   asm volatile("griddepcontrol.wait;" ::: "memory");
