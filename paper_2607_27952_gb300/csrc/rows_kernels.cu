@@ -243,12 +243,12 @@ __global__ void __launch_bounds__(kPassThreads, 1) rows_pass_kernel(const __grid
 #pragma unroll
           for (int q = 0; q < 32; ++q) t[q] = z[q];
           const float mx = warp_columns(t, lane, [](float x, float y) { return fmaxf(x, y); });
-          bmax[warp][lane] = mx;
+          // (a column without a finite logit here is left at zero, not at 2^(-inf + inf))
+          bmax[warp][lane] = mx == -INFINITY ? 0.f : mx;
           __syncwarp();
 #pragma unroll
           for (int q = 0; q < 32; ++q) {
-            const float mq = bmax[warp][q];
-            z[q] = seen || z[q] != -INFINITY ? exp2f(z[q] - mq) : 0.f;
+            z[q] = exp2f(z[q] - bmax[warp][q]);
             t[q] = z[q];
           }
           __syncwarp();

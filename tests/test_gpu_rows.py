@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import oracle
-from workloads import config, custom, query_rows
+from workloads import config, custom, f32_to_bf16_bits, query_rows
 
 from gpu_util import SCORE_ATOL, SCORE_RTOL, problem_of, to_dev
 
@@ -118,3 +118,19 @@ def test_chunk_edges_and_column_counts(hq, hkv, D, m_rows, n_vis, n_text, n_befo
                 num_layers=2, num_q_heads=hq, num_kv_heads=hkv, head_dim=D, feat_dim=64, dtype="bf16",
                 keep=[1] * len(n_vis), n_planted=1)
     check(wl, *make_rows(wl, "all", np.random.default_rng(3), m_rows=m_rows))
+
+
+@pytest.mark.parametrize("masked", [(32, 64), (128, 256), (32, 256)])
+def test_keys_whose_logits_are_minus_infinity(masked):
+    """Visual keys whose products overflow to -inf take no part in the softmax, also where they
+    fill a warp's 32 keys or a whole 128-key chunk that every row sees."""
+    wl = custom(name="inf", seed=72, batch=1, n_vis=[400], n_text=[8], num_layers=1, num_q_heads=4,
+                num_kv_heads=2, head_dim=64, feat_dim=64, dtype="bf16", keep=[1], n_planted=1)
+    cu, pos, q = make_rows(wl, "all", np.random.default_rng(4), m_rows=6)
+    big, low = f32_to_bf16_bits(np.float32([3e38, -3e38]))
+    v0 = int(wl.vis_start[0])
+    wl.k[..., 0] = 0
+    wl.k[:, v0 + masked[0]:v0 + masked[1], :, 0] = low
+    q[..., 0] = big
+    w = check(wl, cu, pos, q)
+    assert (w[masked[0]:masked[1]] == 0).all() and (np.delete(w, np.arange(*masked)) > 0).all()
