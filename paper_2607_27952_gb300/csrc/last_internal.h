@@ -106,6 +106,11 @@ bool gram_long(int max_vis);
 __host__ __device__
 #endif
 inline int gram_ld(int n_tokens) { return (n_tokens + 31) / 32 * 32; }
+// Lets `fn` be launched with `smem` bytes of dynamic shared memory on the current device.
+// The limit belongs to the process, not to the call, and covers the kernel's own arrays too:
+// it is set to all that the device leaves beside those, always the same value, so that
+// host threads launching other shapes of one kernel cannot lower it between them.
+cudaError_t allow_smem(const void *fn, size_t smem);
 // Clusters of `fn` (csize CTAs of `threads`, smem bytes each) resident at once, cached.
 int active_clusters(void *fn, int csize, size_t smem, int threads);
 size_t grid_select_smem(int row_bytes, int tpc);

@@ -648,8 +648,7 @@ extern "C" last_status last_scores_rows(const last_problem *p, const int32_t *cu
     if (n > 0x7fffffffLL) return rows_fail(LAST_ERR_UNSUPPORTED, "too many key chunks in all");
     if (n > 0) {
       a.n_items = (int)n;
-      if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return fail_launch(e, "rows pass");
+      if ((e = allow_smem(fn, smem)) != cudaSuccess) return fail_launch(e, "rows pass");
       void *args[] = {&a};
       e = cudaLaunchKernel(fn, dim3((unsigned)std::min<long long>(n, sms)), dim3(kPassThreads), args, smem, s);
       if (e != cudaSuccess) return fail_launch(e, "rows pass launch");

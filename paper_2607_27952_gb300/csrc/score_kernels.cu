@@ -396,11 +396,8 @@ cudaError_t launch_scores(const Plan &pl, const void *q, const void *k, float *w
   void *fn = pl.dtype == LAST_DTYPE_BF16 ? pick_logits<__nv_bfloat16>(pl.G)
                                          : pick_logits<float>(pl.G);
   const size_t smem = logits_smem(pl);
-  cudaError_t e;
-  if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  cudaError_t e = allow_smem(fn, smem);
+  if (e != cudaSuccess) return e;
   int slots = 0;
   if ((e = resident_slots(fn, smem, &slots)) != cudaSuccess) return e;
   const long long items = (long long)pl.total_chunks * pl.L;
@@ -410,11 +407,7 @@ cudaError_t launch_scores(const Plan &pl, const void *q, const void *k, float *w
   if (e != cudaSuccess) return e;
   const int max_tiles = (pl.max_vis + kTokenTile - 1) / kTokenTile;
   const size_t tsmem = sizeof(float) * 3 * pl.L * pl.Hq;
-  if (tsmem > 48 * 1024) {
-    e = cudaFuncSetAttribute(score_tokens_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tsmem);
-    if (e != cudaSuccess) return e;
-  }
+  if ((e = allow_smem((const void *)score_tokens_kernel, tsmem)) != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(max_tiles, pl.B);
   cfg.blockDim = dim3(kScoreThreads);

@@ -1517,7 +1517,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
       void *fn = f32 ? (void *)gram_exact_kernel<float> : (void *)gram_exact_kernel<__nv_bfloat16>;
       const int cols = f32 ? kExCols<float> : kExCols<__nv_bfloat16>;
       const size_t smem = (size_t)kExBufs * (kExRows + cols) * 256 * pl.elem;
-      e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = allow_smem(fn, smem);
       if (e != cudaSuccess) return e;
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(pl.gram_tiles);
@@ -1537,7 +1537,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
       const size_t smem = 192 * 1024 + 1024;
       static_assert(kGramStages * kGramStageBytes == 192 * 1024 && kPairStages * kPairStageBytes == 192 * 1024,
                     "the ring of either kernel");
-      e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      e = allow_smem(fn, smem);
       if (e != cudaSuccess) return e;
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(pair ? 2 * std::min(sms / 2, pl.gram_tiles) : std::min(sms, pl.gram_tiles));
@@ -1568,7 +1568,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   a.eps = pl.gram_exact ? 0.f : gram_distance_eps(pl.dv, chunk);
   a.err = g.err;
   e = cudaFuncSetAttribute(sel_fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(sel_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
+  if (e == cudaSuccess) e = allow_smem(sel_fn, sh.smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(sh.C * pl.B);

@@ -609,7 +609,7 @@ cudaError_t launch_select_grid(const Plan &pl, const float *w, const void *x, in
   for (int b = 0; b < pl.B; ++b) a.req[b] = b;
   const size_t smem = grid_smem(rb, tpc).total;
   if (tpc == 0 || smem > (size_t)optin) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   a.x = x; a.w = w; a.idx_out = idx_out; a.x_out = x_out;
   a.meta = reinterpret_cast<const int32_t *>(ws + pl.off_meta);

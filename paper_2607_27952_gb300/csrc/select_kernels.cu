@@ -86,6 +86,19 @@ EncodeTiledFn encode_tiled() {
 
 }  // namespace
 
+cudaError_t allow_smem(const void *fn, size_t smem) {
+  // within the default of 48 KB with the kernel's own arrays (11 KB at most)
+  if (smem <= 32 * 1024) return cudaSuccess;
+  int dev = 0, optin = 0;
+  cudaFuncAttributes at;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, fn);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              optin - (int)at.sharedSizeBytes);
+}
+
 // Clusters of `fn` (csize CTAs of `threads`, smem bytes each) resident at once, cached per
 // (device, kernel, cluster size, shared memory); 0 if it cannot be placed.
 int active_clusters(void *fn, int csize, size_t smem, int threads) {
@@ -101,7 +114,7 @@ int active_clusters(void *fn, int csize, size_t smem, int threads) {
   }
   int active = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
+      allow_smem(fn, smem) == cudaSuccess) {
     cudaLaunchConfig_t q = {};
     q.gridDim = dim3(csize);
     q.blockDim = dim3(threads);
@@ -329,7 +342,7 @@ cudaError_t launch_select(const Plan &pl, const float *w, const void *x, int32_t
   }
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
 
   a.x = x; a.w = w; a.idx_out = idx_out; a.x_out = x_out;

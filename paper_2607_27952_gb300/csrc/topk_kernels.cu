@@ -160,13 +160,10 @@ cudaError_t launch_topk(const Plan &pl, const float *w, int32_t *idx_out, char *
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   // cache every request's scores when they fit beside the kernel's own arrays (8.3 KB)
-  const int most = std::min<int>(kTopkCacheTokens, std::max(0, (optin - 12 * 1024) / 4));
-  const int cache = std::min(most, pl.max_vis);
+  const int cache = std::min<int>(std::min(kTopkCacheTokens, pl.max_vis),
+                                  std::max(0, (optin - 12 * 1024) / 4));
   const size_t smem = sizeof(float) * (size_t)cache;
-  // The limit holds for the kernel's own arrays and the cache together (48 KB unless
-  // raised), and is the process's: always the same value, the most a call may ask for.
-  cudaError_t e = cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float) * most));
+  cudaError_t e = allow_smem((const void *)topk_kernel, smem);
   if (e != cudaSuccess) return e;
   topk_kernel<<<pl.B, kTopkThreads, smem, s>>>(
       w, reinterpret_cast<const int32_t *>(ws + pl.off_meta), idx_out, cache);

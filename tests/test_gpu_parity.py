@@ -5,6 +5,10 @@ rows bit-exact against the canonical-fp32 oracle selection when run on the same
 scores (ties -> lowest index); end-to-end, an index sequence may leave the
 oracle's only at a near-tie (products within PRODUCT_TIE_RTOL = 2.5e-3).
 """
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -283,3 +287,28 @@ def test_gather_wide_rows():
     got = to_host_bits(out)
     assert np.array_equal(got[:9], oracle.gather(wl.x[:40], idx[:9]))
     assert np.array_equal(got[9:], oracle.gather(wl.x[40:115], idx[9:]))
+
+
+_FIRST_SCORES = """
+import sys
+sys.path.insert(0, "tests")
+import oracle
+from gpu_util import DeviceWorkload, assert_scores_close
+from workloads import custom
+layers, heads = int(sys.argv[1]), int(sys.argv[2])
+wl = custom(name="pairs", seed=75, batch=1, n_vis=[50], n_text=[3], num_layers=layers, num_q_heads=heads,
+            num_kv_heads=heads, head_dim=8, feat_dim=64, dtype="bf16", keep=[2], n_clusters=4, n_planted=2)
+w_ref = oracle.scores(wl.q, wl.k, wl.cu_seqlens, wl.vis_start, wl.cu_vis, num_kv_heads=heads, scale=wl.scale)
+assert_scores_close(DeviceWorkload(wl).scores(), w_ref, wl)
+"""
+
+
+@pytest.mark.parametrize("layers,heads", [(62, 66), (63, 65), (32, 128), (17, 241)])
+def test_first_call_of_a_process_around_the_default_shared_memory(layers, heads):
+    """4092, 4095, 4096 and 4097 (layer, q-head) pairs: at two of them the token kernel's tables
+    pass the default 48 KB only together with its own words, in a process whose first
+    scoring call this is (no earlier one has raised the limit)."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FIRST_SCORES, str(layers), str(heads)], cwd=root,
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
