@@ -24,8 +24,8 @@
  *
  * Conventions shared by every entry point
  *   - All tensors are DEVICE pointers (caller-allocated, e.g. torch tensors),
- *     except those of last_prune_host; the library allocates no device memory.  Scratch lives in a caller
- *     workspace of at least last_workspace_size() bytes (256-byte aligned).
+ *     except those of last_prune_host; the library allocates no device memory.  Scratch
+ *     lives in a caller workspace (256-byte aligned), sized by last_workspace_size().
  *   - The offset arrays in last_problem are HOST arrays; each call validates
  *     them and copies a small plan into the workspace on `stream`.
  *   - Calls are asynchronous on `stream` (a cudaStream_t; NULL = legacy
@@ -88,7 +88,7 @@ typedef enum {
   LAST_OK = 0,
   LAST_ERR_INVALID_ARG = 1,          /* shape/offset/pointer check failed (host) */
   LAST_ERR_UNSUPPORTED = 2,          /* valid but outside the compiled limits */
-  LAST_ERR_WORKSPACE_TOO_SMALL = 3,  /* ws_bytes < last_workspace_size() */
+  LAST_ERR_WORKSPACE_TOO_SMALL = 3,  /* ws_bytes below what the call needs at least */
   LAST_ERR_CUDA = 4,                 /* a CUDA runtime call failed */
   LAST_ERR_DEVICE_INDEX = 5,         /* last_poll: a caller index was out of range */
   LAST_ERR_TIMEOUT = 6               /* last_poll: a bounded device wait expired; outputs invalid */
@@ -117,13 +117,26 @@ typedef struct {
   const int32_t *cu_keep;    /* [batch+1] */
 } last_problem;
 
-/* Bytes of device workspace the entry points below need for `p`, except
+/* Bytes of device workspace with which the entry points below run `p` fastest, except
  * last_scores_rows and last_prune_host, which are sized by
  * last_scores_rows_workspace_size and last_host_workspace_size.
- * Returns LAST_ERR_INVALID_ARG / LAST_ERR_UNSUPPORTED for a bad problem. */
+ * Returns LAST_ERR_INVALID_ARG / LAST_ERR_UNSUPPORTED for a bad problem.
+ *
+ * Most of it may be room for the selection's Gram matrices: 4 N_b^2 bytes per request
+ * with 1 < k_b < N_b, up to 12 GiB a call (8 requests of 16384 tokens: 8.6 GB), where
+ * a matrix makes the selection faster.  last_select, last_prune and
+ * last_prune_host also take less: without room for the matrices they read the
+ * features in every round, with the same results, three to four times slower
+ * on such batches.  What a call needs at least grows with its problem, and the size
+ * reported for the same problem with cu_keep = cu_vis (no token to choose, so no
+ * matrix) is always enough, whatever the budgets; so is that of a problem with
+ * more requests, tokens or keys for one with fewer (see last_scores and
+ * last_select_topk for callers that do not select).  LAST_ERR_WORKSPACE_TOO_SMALL
+ * names the least size in last_error_message(). */
 last_status last_workspace_size(const last_problem *p, size_t *bytes);
 
-/* Eq. 6-8.  w_out [cu_vis[batch]] fp32 receives w~ (sums to 1 per request). */
+/* Eq. 6-8.  w_out [cu_vis[batch]] fp32 receives w~ (sums to 1 per request).  The size
+ * reported with cu_keep all zero is enough (the budgets are not used). */
 last_status last_scores(const last_problem *p, const void *q, const void *k, float *w_out,
                         void *ws, size_t ws_bytes, void *stream);
 
@@ -140,7 +153,8 @@ last_status last_select(const last_problem *p, const float *w, const void *x,
  * k_b indices of highest w~ (ties between equal scores go to the lower index;
  * -0 equals +0).  When x_out is not NULL the kept rows of x are also written
  * there (x is then required; feat_dim a positive multiple of 8); x may be NULL
- * otherwise.  The problem's layer/head fields are not used.  Same ownership,
+ * otherwise.  The problem's layer/head fields are not used.  Uses no matrix: like for
+ * last_gather, the size reported with cu_keep = cu_vis is enough.  Same ownership,
  * stream and error rules as last_select.  w must hold no NaN: the kept set is
  * then unspecified (but still k_b distinct valid indices). */
 last_status last_select_topk(const last_problem *p, const float *w, const void *x,
@@ -193,7 +207,8 @@ last_status last_prune(const last_problem *p, const void *q, const void *k, cons
  * on two streams overlaps one call's copies with another's kernels; pageable
  * memory works but the copies then block the host.  The device workspace holds
  * the plan and device copies of q, K, X, w~, the indices and the kept rows:
- * last_host_workspace_size() bytes, 256-byte aligned. */
+ * last_host_workspace_size() bytes, 256-byte aligned, or less when that holds Gram
+ * matrices (see last_workspace_size). */
 last_status last_host_workspace_size(const last_problem *p, size_t *bytes);
 last_status last_prune_host(const last_problem *p, const void *q_host, const void *k_host,
                             const void *x_host, float *w_out_host, int32_t *idx_out_host,
@@ -211,7 +226,8 @@ last_status last_prune_host(const last_problem *p, const void *q_host, const voi
  * graph (the plan is copied from host memory the call releases).  All calls share
  * the array and it keeps the last call's contents: calls whose executions
  * overlap on the GPU race on it.  A problem needing more than 16 MiB of scratch
- * (last_workspace_size) returns LAST_ERR_UNSUPPORTED.  Allocates nothing. */
+ * (last_workspace_size with cu_keep all zero) returns LAST_ERR_UNSUPPORTED.
+ * Allocates nothing. */
 last_status last_scores_noalloc(const last_problem *p, const void *q, const void *k,
                                 float *w_out, void *stream);
 

@@ -196,10 +196,37 @@ def last_workspace_size(problem: Problem) -> int:
     return n.value
 
 
-def workspace(problem: Problem, device="cuda"):
-    """A torch uint8 tensor of last_workspace_size bytes (torch allocations are 512-B aligned)."""
+def _keep_all(problem: Problem) -> Problem:
+    """The same problem with every token kept: its workspace size holds no Gram matrices and is
+    enough for `problem` whatever its budgets."""
+    a, c = problem.arrays, problem.c
+    return Problem(batch=c.batch, num_layers=c.num_layers, num_q_heads=c.num_q_heads,
+                   num_kv_heads=c.num_kv_heads, head_dim=c.head_dim, feat_dim=c.feat_dim,
+                   dtype=problem.dtype, cu_seqlens=a["cu_seqlens"], vis_start=a["vis_start"],
+                   cu_vis=a["cu_vis"], cu_keep=a["cu_vis"], softmax_scale=c.softmax_scale)
+
+
+def _alloc(size, problem: Problem, device):
+    """`size(problem)` bytes on the device; without that much memory free, the smaller
+    workspace with which the selection does without its Gram matrices."""
     import torch
-    return torch.empty(max(last_workspace_size(problem), 256), dtype=torch.uint8, device=device)
+
+    def empty(n):
+        return torch.empty(max(n, 256), dtype=torch.uint8, device=device)
+    n = size(problem)
+    try:
+        return empty(n)
+    except torch.OutOfMemoryError:
+        least = size(_keep_all(problem))
+        if least >= n:
+            raise
+        return empty(least)
+
+
+def workspace(problem: Problem, device="cuda"):
+    """A torch uint8 tensor of last_workspace_size bytes (torch allocations are 512-B aligned),
+    or of the size without the selection's Gram matrices where the device has less free."""
+    return _alloc(last_workspace_size, problem, device)
 
 
 def last_scores(problem: Problem, q, k, w_out, ws, stream=None):
@@ -277,10 +304,8 @@ def last_host_workspace_size(problem: Problem) -> int:
 
 
 def host_workspace(problem: Problem, device="cuda"):
-    """A torch uint8 device tensor of last_host_workspace_size bytes."""
-    import torch
-    return torch.empty(max(last_host_workspace_size(problem), 256), dtype=torch.uint8,
-                       device=device)
+    """A torch uint8 device tensor of last_host_workspace_size bytes, or less (see workspace)."""
+    return _alloc(last_host_workspace_size, problem, device)
 
 
 def last_prune_host(problem: Problem, q, k, x, w_out, idx_out, x_out, ws, stream=None):

@@ -147,9 +147,10 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
   o = align_up(o + (size_t)pl->root_rows * (size_t)((std::max(p->feat_dim, 0) + 63) / 64) * 128);
   pl->off_rtab = o;
   o = align_up(o + (size_t)pl->root_rows * kRootTableCols * sizeof(float));
-  // the whole-GPU selection's published keys, for launches that may take it
+  // the whole-GPU selection's published keys, where launches of few requests may take it
+  // (room for them whatever the batch: what a call needs grows with its problem)
   pl->off_gpub = o;
-  if (B <= kGridMaxReq && pl->max_vis >= kGridMinTokens) o = align_up(o + grid_pub_bytes());
+  if (pl->max_vis >= kGridMinTokens) o = align_up(o + grid_pub_bytes());
   pl->base_bytes = o;
   // The greedy from a Gram matrix: N_b rows of gram_ld(N_b) floats for every request
   // that has a choice to make (1 < k_b < N_b).
@@ -181,7 +182,8 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
     pl->off_gram = o;
     o = align_up(o + (size_t)units * 128);
   }
-  pl->total_bytes = o;
+  pl->min_bytes = pl->base_bytes + (gram_ok && pl->total_keep > 0 ? kGramSmallBytes : 0);
+  pl->total_bytes = std::max(o, pl->min_bytes);
 
   // ---- host staging: [err words][meta][items][order], one copy ----
   pl->blob_bytes = blob_end;
@@ -237,28 +239,32 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
 
 namespace {
 
-last_status check_ws(const Plan &pl, const void *ws, size_t ws_bytes, bool scores_only = false,
-                     bool select = false) {
+last_status check_ws(const void *ws, size_t ws_bytes, size_t need) {
   if (ws == nullptr) return fail(LAST_ERR_INVALID_ARG, "workspace is NULL");
   if ((reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0)
     return fail(LAST_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
-  const size_t need = scores_only ? pl.score_bytes : select ? pl.total_bytes : pl.base_bytes;
   if (ws_bytes < need)
     return fail(LAST_ERR_WORKSPACE_TOO_SMALL, "workspace needs " + std::to_string(need) + " bytes");
   return LAST_OK;
+}
+
+// The selection's workspace: without room for the matrices its rounds read X.
+last_status check_select_ws(Plan *pl, const void *ws, size_t ws_bytes) {
+  if (ws_bytes < pl->total_bytes) pl->gram = false;
+  return check_ws(ws, ws_bytes, pl->min_bytes);
 }
 
 last_status cuda_fail(cudaError_t e, const char *what) {
   return fail(LAST_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-// Device copies of last_prune_host's tensors after the plan workspace, each
-// 256-byte aligned.
+// Device copies of last_prune_host's tensors after the plan workspace (of `plan_bytes`),
+// each 256-byte aligned.
 struct HostLayout {
   size_t q, k, x, w, idx, xo, total;
   size_t q_bytes, k_bytes, x_bytes, w_bytes, idx_bytes, xo_bytes;
 };
-HostLayout host_layout(const Plan &pl) {
+HostLayout host_layout(const Plan &pl, size_t plan_bytes) {
   auto al = [](size_t v) { return (v + kAlign - 1) & ~(size_t)(kAlign - 1); };
   HostLayout h;
   h.q_bytes = (size_t)pl.B * pl.L * pl.Hq * pl.D * pl.elem;
@@ -267,7 +273,7 @@ HostLayout host_layout(const Plan &pl) {
   h.w_bytes = (size_t)pl.total_vis * sizeof(float);
   h.idx_bytes = (size_t)pl.total_keep * sizeof(int32_t);
   h.xo_bytes = (size_t)pl.total_keep * pl.dv * pl.elem;
-  size_t o = al(pl.total_bytes);
+  size_t o = al(plan_bytes);
   h.q = o; o += al(h.q_bytes);
   h.k = o; o += al(h.k_bytes);
   h.x = o; o += al(h.x_bytes);
@@ -307,7 +313,7 @@ last_status last_scores(const last_problem *p, const void *q, const void *k, flo
   Plan pl;
   last_status st = make_plan(p, true, false, &pl);
   if (st != LAST_OK) return st;
-  if ((st = check_ws(pl, ws, ws_bytes, true)) != LAST_OK) return st;
+  if ((st = check_ws(ws, ws_bytes, pl.score_bytes)) != LAST_OK) return st;
   if (pl.total_vis > 0 && (q == nullptr || k == nullptr || w_out == nullptr))
     return fail(LAST_ERR_INVALID_ARG, "q, k and w_out are required");
   if (!aligned16(q) || !aligned16(k)) return fail(LAST_ERR_INVALID_ARG, "q and k must be 16-byte aligned");
@@ -331,7 +337,7 @@ last_status last_select(const last_problem *p, const float *w, const void *x, in
   last_status st = make_plan(p, false, true, &pl);
   if (st != LAST_OK) return st;
   if ((st = check_select_fits(pl)) != LAST_OK) return st;
-  if ((st = check_ws(pl, ws, ws_bytes, false, true)) != LAST_OK) return st;
+  if ((st = check_select_ws(&pl, ws, ws_bytes)) != LAST_OK) return st;
   if (pl.total_keep > 0 && (w == nullptr || x == nullptr || idx_out == nullptr))
     return fail(LAST_ERR_INVALID_ARG, "w, x and idx_out are required");
   if (!aligned16(x) || !aligned16(x_out))
@@ -349,7 +355,7 @@ last_status last_select_topk(const last_problem *p, const float *w, const void *
   Plan pl;
   last_status st = make_plan(p, false, false, &pl);
   if (st != LAST_OK) return st;
-  if ((st = check_ws(pl, ws, ws_bytes)) != LAST_OK) return st;
+  if ((st = check_ws(ws, ws_bytes, pl.base_bytes)) != LAST_OK) return st;
   if (pl.total_keep > 0 && (w == nullptr || idx_out == nullptr))
     return fail(LAST_ERR_INVALID_ARG, "w and idx_out are required");
   if (x_out != nullptr) {
@@ -381,7 +387,7 @@ last_status last_gather(const last_problem *p, const void *x, const int32_t *idx
   if (st != LAST_OK) return st;
   if (p->feat_dim < 8 || p->feat_dim % 8 != 0)
     return fail(LAST_ERR_INVALID_ARG, "feat_dim must be a positive multiple of 8");
-  if ((st = check_ws(pl, ws, ws_bytes)) != LAST_OK) return st;
+  if ((st = check_ws(ws, ws_bytes, pl.base_bytes)) != LAST_OK) return st;
   if (pl.total_keep > 0 && (x == nullptr || idx == nullptr || x_out == nullptr))
     return fail(LAST_ERR_INVALID_ARG, "x, idx and x_out are required");
   if (!aligned16(x) || !aligned16(x_out))
@@ -400,7 +406,7 @@ last_status last_prune(const last_problem *p, const void *q, const void *k, cons
   last_status st = make_plan(p, true, true, &pl);
   if (st != LAST_OK) return st;
   if ((st = check_select_fits(pl)) != LAST_OK) return st;
-  if ((st = check_ws(pl, ws, ws_bytes, false, true)) != LAST_OK) return st;
+  if ((st = check_select_ws(&pl, ws, ws_bytes)) != LAST_OK) return st;
   if (pl.total_vis > 0 && (q == nullptr || k == nullptr || x == nullptr))
     return fail(LAST_ERR_INVALID_ARG, "q, k and x are required");
   if (pl.total_keep > 0 && idx_out == nullptr)
@@ -423,7 +429,7 @@ last_status last_host_workspace_size(const last_problem *p, size_t *bytes) {
   Plan pl;
   last_status st = make_plan(p, true, true, &pl);
   if (st != LAST_OK) return st;
-  *bytes = host_layout(pl).total;
+  *bytes = host_layout(pl, pl.total_bytes).total;
   return LAST_OK;
 }
 
@@ -434,7 +440,11 @@ last_status last_prune_host(const last_problem *p, const void *q, const void *k,
   last_status st = make_plan(p, true, true, &pl);
   if (st != LAST_OK) return st;
   if ((st = check_select_fits(pl)) != LAST_OK) return st;
-  const HostLayout h = host_layout(pl);
+  HostLayout h = host_layout(pl, pl.total_bytes);
+  if (ws_bytes < h.total) {   // no room for the matrices: the rounds read X
+    h = host_layout(pl, pl.min_bytes);
+    pl.gram = false;
+  }
   if (ws == nullptr) return fail(LAST_ERR_INVALID_ARG, "workspace is NULL");
   if ((reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0)
     return fail(LAST_ERR_INVALID_ARG, "workspace must be 256-byte aligned");

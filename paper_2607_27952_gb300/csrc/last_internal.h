@@ -38,6 +38,9 @@ constexpr int kGridMaxCtas = 256;   // CTAs of one whole-GPU selection launch at
 constexpr int kGatherThreads = 256;
 constexpr double kGramExactSeconds = 20e-6;   // bf16 batches up to this take the canonical matrix
 constexpr long long kGramMaxBytes = 12LL << 30;   // Gram matrices of one call at most
+// Matrices up to this always have their room: the least workspace of a selection includes it,
+// so that it grows with the problem whether or not a matrix is used.
+constexpr size_t kGramSmallBytes = 64 << 10;
 
 // Device error flags (first word of the workspace).
 constexpr unsigned kErrGatherIndex = 1u;
@@ -64,8 +67,9 @@ struct Plan {
   size_t off_gbar = 0, off_gpub = 0;
   long long root_rows = 0;
   // selection from a Gram matrix: 1/|x| per token, the matrices, first tile per request.
-  // base_bytes excludes the first two (Top-k and the gather do not use them).
-  size_t off_rn = 0, off_gram = 0, off_tile0 = 0, base_bytes = 0;
+  // base_bytes excludes the first two (Top-k and the gather do not use them).  The selection
+  // takes min_bytes to total_bytes: with less than total_bytes it does without the matrices.
+  size_t off_rn = 0, off_gram = 0, off_tile0 = 0, base_bytes = 0, min_bytes = 0;
   int gram_tiles = 0;
   bool gram = false, gram_exact = false;   // exact: in the canonical order, on CUDA cores
   // host staging (error word, meta rows, score items, selection order) in ws order

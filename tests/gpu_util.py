@@ -2,6 +2,8 @@
 the C ABI, and the comparison rules against the oracle."""
 from __future__ import annotations
 
+import re
+
 import numpy as np
 
 import oracle
@@ -67,14 +69,18 @@ class DeviceWorkload:
         last.last_poll(ws)
         return w.cpu().numpy()
 
-    def select(self, w32: np.ndarray, cu_keep=None):
+    def select(self, w32: np.ndarray, cu_keep=None, path=None):
+        """last_select's indices.  path: None, "matrix" (asserts that the selection used its Gram
+        matrices) or "rounds" (gives it no room for them: every round reads X)."""
         import torch
         prob = problem_of(self.wl, cu_keep)
         _, idx, _ = self.outputs(cu_keep)
-        ws = last.workspace(prob, self.dev)
+        ws = select_workspace(prob, self.dev, path)
         wt = torch.from_numpy(np.ascontiguousarray(w32, dtype=np.float32)).to(self.dev)
         last.last_select(prob, wt, self.x, idx, ws)
         last.last_poll(ws)
+        if path == "matrix":
+            assert_matrix_used(prob, ws)
         return idx.cpu().numpy()
 
 
@@ -157,3 +163,32 @@ def near_tie_divergence(x, w_ref, seq_ref, seq_alt):
         dc = (1.0 - xb[c] @ xb[S].T).min()
         pa, pc = w_ref[a] * da, w_ref[c] * dc
     return t, abs(pa - pc) / max(abs(pa), abs(pc), 1e-300)
+
+
+def least_workspace(prob: last.Problem) -> int:
+    """Bytes that last_select needs at least for `prob` (it names them when given fewer, before
+    it looks at any pointer).  Below last_workspace_size, a call with so many runs the rounds
+    over X: it has no room for the Gram matrices."""
+    try:
+        last.last_select(prob, 256, 256, 256, (256, 256), stream=0)
+    except last.LastError as e:
+        assert e.status == last.LAST_ERR_WORKSPACE_TOO_SMALL, str(e)
+        return int(re.search(r"needs (\d+) bytes", str(e)).group(1))
+    raise AssertionError("a workspace of 256 bytes was accepted")
+
+
+def select_workspace(prob: last.Problem, dev, path=None):
+    """A workspace that has the selection take `path`: "rounds" over X (no room for a matrix),
+    "matrix" (marked, for assert_matrix_used) or None, what it takes by itself."""
+    import torch
+    if path != "rounds":
+        ws = last.workspace(prob, dev)
+        return ws.fill_(0xA5) if path == "matrix" else ws
+    n = least_workspace(prob)
+    assert n < last.last_workspace_size(prob), "matrices so small always have their room"
+    return torch.empty(n, dtype=torch.uint8, device=dev)
+
+
+def assert_matrix_used(prob: last.Problem, ws):
+    """The matrices lie past the least workspace (all but their first 64 KB): written, or not."""
+    assert (ws[least_workspace(prob):] != 0xA5).any(), "the selection did not use a matrix"

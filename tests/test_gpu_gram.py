@@ -9,8 +9,8 @@ import pytest
 
 import oracle
 import paper_2607_27952_gb300 as last
-from gpu_util import (assert_gather_equal, assert_selection_equal, oracle_selection,
-                      problem_of, to_dev, to_host_bits)
+from gpu_util import (DeviceWorkload, assert_gather_equal, assert_selection_equal, least_workspace,
+                      oracle_selection, problem_of, to_dev, to_host_bits)
 from workloads import bf16_bits_to_f32, custom, f32_to_bf16_bits
 
 pytestmark = pytest.mark.gpu
@@ -113,3 +113,31 @@ def test_best_tokens_on_one_lane_of_every_warp():
     got = idx.cpu().numpy().reshape(batch, k)
     for b in (0, 70, batch - 1):
         assert np.array_equal(got[b], np.sort(oracle.select_fp32(x, w[b], k)))
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_without_room_for_the_matrices(dtype):
+    """last_select, last_prune and last_prune_host with the least workspace they take, and with
+    one byte less than the matrices need: the rounds over X give the same picks."""
+    import torch
+    wl = _wl([900, 40, 1300], [130, 40, 70], 256, dtype=dtype)
+    dw, prob, rng = DeviceWorkload(wl), problem_of(wl), np.random.default_rng(3)
+    w = (rng.random(int(wl.cu_vis[-1])) + 0.5).astype(np.float32)
+    want = dw.select(w, path="matrix")
+    assert np.array_equal(dw.select(w, path="rounds"), want)
+    assert_selection_equal(wl, w, want, range(wl.batch))
+    least, full = least_workspace(prob), last.last_workspace_size(prob)
+    w_full, idx_full, xs_full = dw.prune()
+    for n in (least, full - 1):
+        w_out, idx, xs = dw.outputs()
+        ws = torch.empty(n, dtype=torch.uint8, device=dw.dev)
+        last.last_prune(prob, dw.q, dw.k, dw.x, w_out, idx, xs, ws)
+        last.last_poll(ws)
+        assert np.array_equal(idx.cpu().numpy(), idx_full)
+        assert np.array_equal(to_host_bits(xs), xs_full) and np.array_equal(w_out.cpu().numpy(), w_full)
+    host = [t.cpu().pin_memory() for t in (dw.q, dw.k, dw.x)]
+    out = torch.empty(int(wl.cu_keep[-1]), dtype=torch.int32).pin_memory()
+    ws = torch.empty(last.last_host_workspace_size(prob) - full + least, dtype=torch.uint8, device=dw.dev)
+    last.last_prune_host(prob, *host, None, out, None, ws)
+    last.last_poll(ws)
+    assert np.array_equal(out.numpy(), idx_full)
