@@ -158,24 +158,56 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
     const int n = p->cu_vis[b + 1] - p->cu_vis[b], kb = p->cu_keep[b + 1] - p->cu_keep[b];
     return kb > 1 && kb < n ? (long long)n * (gram_ld(n) / 32) : 0;
   };
-  long long units = 0;
+  long long units = 0, tokens = 0;
+  int choices = 0, keep = 2;   // requests with a choice, their tokens and largest budget
   const bool gram_ok = p->feat_dim >= 8 && p->feat_dim % 8 == 0 && p->feat_dim <= kMaxFeatDim;
   if (gram_ok)
-    for (int b = 0; b < B; ++b) units += gram_units(b);
-  // Used where the contraction over the lower triangle (about 1.1 PFLOP/s on tensor
-  // cores, 20 T fma/s in the canonical order) costs less than the rounds over X that it
-  // replaces.  bf16, matrix / rounds over X, us: 8 requests of 16384 x 2048 at k = 32 3169 /
-  // 3102, 64 3337 / 3707, 400 3622 / 7732; one of them at k = 8 456 / 1404; 16 of 4096 x
-  // 1536 at 8 475 / 937; 64 of 576 x 2048 at 4 148 / 387: the line lies near 0.12 ms a pick
-  // for matrices of several ms and below any budget for small ones.  fp32: 576 x 1024 at
-  // k = 2 39 / 30, 4 43 / 46; two of 2048 at 32 350 / 319, 64 378 / 598; four of 4096 at
-  // 128 2456 / 1585; 10000 at 128 3551 / 3313: 6 us a pick.
-  const double fmas = 0.5 * (double)units * 32.0 * p->feat_dim;
-  const double tensor_s = 2.0 * fmas / 1.1e15, exact_s = fmas / 20e12;
+    for (int b = 0; b < B; ++b)
+      if (gram_units(b) > 0) {
+        units += gram_units(b);
+        tokens += p->cu_vis[b + 1] - p->cu_vis[b];
+        keep = std::max(keep, p->cu_keep[b + 1] - p->cu_keep[b]);
+        ++choices;
+      }
   const bool f32 = p->dtype == LAST_DTYPE_F32;
-  pl->gram_exact = f32 || exact_s <= kGramExactSeconds;
-  pl->gram = units > 0 && units * 128 <= kGramMaxBytes &&
-             (f32 ? exact_s <= 6e-6 * pl->max_keep : tensor_s <= std::max(0.8e-3, 1.2e-4 * pl->max_keep));
+  const double pairs = 0.5 * (double)units * 32.0;
+  const double exact_s = pairs * p->feat_dim / 20e12;   // canonical order, 20 T fma/s
+  // ... whose kernel takes whole groups of 256 coordinates and one more for its butterfly
+  const double exact_all_s = pairs * 256.0 * ((std::max(p->feat_dim, 0) + 255) / 256 + 1) / 20e12;
+  // bf16 batches take the canonical matrix where it costs little; measured against the tensor
+  // cores' (us, whole selection, k = N/8): one request of 576 x 2048 85 / 110, four 138 / 122;
+  // of 1100 x 512 126 / 142, of 2000 x 512 210 / 194; narrow rows, 16 of 576 x 64 140 / 111.
+  pl->gram_exact = f32 || (exact_s <= kGramExactSeconds && exact_all_s <= 55e-6);
+  // A matrix is used where it costs less than the rounds over X that it replaces: its bytes
+  // at 5.2 TB/s beside its products (1.1 PFLOP/s, 1.7 in the long chains of requests of
+  // 8192 tokens), and 50 us + 0.9 us a request for what surrounds it.  The rounds cost a
+  // pass that grows with the width and the tokens per CTA and recurs a little with every
+  // doubling of the budget.  Both sides measured, matrix / rounds, us: 8 requests of 16384
+  // x 64 at k = 2 1723 / 303, 256 1864 / 1628; x 2048 at 32 3169 / 2580, 64 3203 / 3378, 256
+  // 3323 / 6006; one of 50000 x 64 at 2 1971 / 564, 32 2096 / 1550, 128 2236 / 2570; two of
+  // 16384 x 256 at 2 489 / 266, 16 528 / 574; 64 of 2048 x 256 at 2 327 / 263, 4 337 / 360; 32
+  // of 2880 x 2048 at 2 630 / 652.  Of the 300 shapes so measured three take the slower side
+  // by more than 6% (13 to 26%).  The second line, in products alone, was drawn first; it
+  // holds back matrices at tiny budgets of wide features.
+  // fp32, canonical order: 576 x 1024 at k = 2 39 / 30, 4 43 / 46; two of 2048 at 32 350 / 319,
+  // 64 378 / 598; four of 4096 at 128 2456 / 1585; 10000 at 128 3551 / 3313; 12000 x 8 at 8 1834
+  // / 455; 8 of 1200 x 64 at 8 203 / 141, 32 220 / 276 (rows narrower than 32 lanes' worth of
+  // coordinates make the rounds slower: 1200 x 8 at 8 207 / 235).
+  bool faster;
+  if (f32) {
+    const double pick = (2.3e-6 + 2.4e-9 * std::min(pl->max_vis, 4096)) * std::max(1.0, 32.0 / std::max(p->feat_dim, 1));
+    faster = exact_all_s <= keep * pick && exact_s <= 6e-6 * keep;
+  } else {
+    const double flops = 2.0 * pairs * ((std::max(p->feat_dim, 0) + 63) / 64 * 64);
+    const double matrix_s = (pl->gram_exact ? exact_all_s
+                                            : std::hypot(8.0 * pairs / 5.2e12, flops / (pl->max_vis >= 8192 ? 1.7e15 : 1.1e15))) +
+                            50e-6 + 0.9e-6 * std::min(choices, 152);
+    const double per_cta = (double)tokens / std::min(152, 16 * std::max(choices, 1));
+    const double rounds_s = (0.20e-3 + 0.28e-3 * p->feat_dim / 1024) * (0.5 + 0.7e-3 * per_cta) *
+                            (1.0 + 0.34 * std::log2(0.5 * keep) + 0.006 * std::max(0, keep - 64));
+    faster = matrix_s <= rounds_s && flops / 1.1e15 <= std::max(0.8e-3, 1.2e-4 * keep);
+  }
+  pl->gram = units > 0 && units * 128 <= kGramMaxBytes && faster;
   if (pl->gram) {
     pl->off_rn = o;
     o = align_up(o + sizeof(float) * (size_t)pl->total_vis);

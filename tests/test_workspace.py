@@ -106,3 +106,39 @@ def test_python_workspaces_do_without_the_matrices_when_memory_is_short(monkeypa
     assert last.host_workspace(prob, "meta").numel() < 2 << 30
     with pytest.raises(torch.OutOfMemoryError):   # no smaller one to fall back on
         last.workspace(_problem(1000, 16384, 16384), "meta")
+
+
+@pytest.mark.parametrize("dtype,batch,n,dv,k,matrix_us,rounds_us", [
+    ("bf16", 8, 16384, 64, 2, 1723, 303), ("bf16", 8, 16384, 256, 64, 1925, 943),
+    ("bf16", 8, 16384, 1024, 32, 2247, 1411), ("bf16", 8, 16384, 1024, 256, 2372, 3241),
+    ("bf16", 8, 16384, 2048, 256, 3323, 6006), ("bf16", 1, 50000, 64, 2, 1971, 564),
+    ("bf16", 1, 50000, 256, 32, 2153, 1575), ("bf16", 1, 50000, 64, 256, 2338, 3214),
+    ("bf16", 2, 16384, 64, 4, 491, 390), ("bf16", 2, 16384, 512, 64, 603, 1044),
+    ("bf16", 64, 2048, 64, 2, 317, 254), ("bf16", 64, 2048, 64, 32, 365, 604),
+    ("bf16", 64, 2048, 2048, 64, 720, 2512), ("bf16", 128, 2048, 64, 2, 556, 400),
+    ("bf16", 16, 4096, 256, 2, 278, 208), ("bf16", 16, 4096, 1024, 32, 393, 734),
+    ("bf16", 32, 2880, 512, 2, 331, 273), ("bf16", 32, 2880, 2048, 8, 648, 978),
+    ("bf16", 256, 576, 64, 2, 216, 322), ("bf16", 16, 576, 64, 2, 98, 110),
+    ("f32", 1, 4096, 8, 2, 245, 120), ("f32", 8, 1200, 64, 8, 203, 141), ("f32", 8, 1200, 64, 32, 220, 276),
+    ("f32", 1, 12000, 8, 8, 1834, 455), ("f32", 1, 4096, 256, 32, 268, 308), ("f32", 8, 1200, 512, 32, 298, 228),
+    ("f32", 1, 576, 1024, 2, 39, 30), ("f32", 1, 4096, 8, 32, 284, 877),
+])
+def test_a_matrix_is_used_where_it_was_measured_faster(dtype, batch, n, dv, k, matrix_us, rounds_us):
+    """The matrix's bytes count as well as its products: narrow features at small budgets are
+    cheaper in rounds over X.  Both sides as measured on a GB300; a matrix shows in the
+    reported size."""
+    prob = _problem(batch, n, k, dtype, dv=dv)
+    assert (last.last_workspace_size(prob) > least_workspace(prob)) == (matrix_us < rounds_us)
+
+
+def test_only_requests_with_a_choice_count():
+    """A request that keeps all its tokens needs no matrix and says nothing about the budgets
+    of those that do."""
+    cu = np.array([0, 16384, 32768, 33768])
+
+    def size(keep_all):
+        prob = last.Problem(batch=3, num_layers=0, num_q_heads=0, num_kv_heads=0, head_dim=0, feat_dim=64,
+                            dtype="bf16", cu_seqlens=None, vis_start=None, cu_vis=cu,
+                            cu_keep=[0, 2, 4, 4 + keep_all])
+        return last.last_workspace_size(prob) - least_workspace(prob)
+    assert size(0) == size(1000) == 0
