@@ -207,7 +207,7 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
                             (1.0 + 0.34 * std::log2(0.5 * keep) + 0.006 * std::max(0, keep - 64));
     faster = matrix_s <= rounds_s && flops / 1.1e15 <= std::max(0.8e-3, 1.2e-4 * keep);
   }
-  pl->gram = units > 0 && units * 128 <= kGramMaxBytes && faster;
+  pl->gram = units > 0 && units * 128 <= kGramMaxBytes && faster && gram_select_fits(pl->max_vis);
   if (pl->gram) {
     pl->off_rn = o;
     o = align_up(o + sizeof(float) * (size_t)pl->total_vis);

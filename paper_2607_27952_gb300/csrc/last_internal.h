@@ -33,6 +33,8 @@ constexpr int kMaxFeatDim = 2048;    // selection keeps x_j in 64 fp32 registers
 constexpr int kRootsPerRequest = 1024;   // root rows per request (the selection's kMaxRoots)
 constexpr int kRootTableCols = 32;       // bound-table columns per root (the selection's kMaxAccept)
 constexpr int kSelectWarps = 8;
+// Opt-in shared memory per CTA of the sm_100 class, for checks made before a device is at hand.
+constexpr int kSmemOptinSm100 = 232448;
 constexpr int kGridMaxReq = 4;      // requests of one whole-GPU selection launch
 constexpr int kGridMaxCtas = 256;   // CTAs of one whole-GPU selection launch at most
 constexpr int kGatherThreads = 256;
@@ -101,6 +103,8 @@ cudaError_t launch_select_grid(const Plan &pl, const float *w, const void *x, in
 // launched, when the requests do not fit it.
 cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, int32_t *idx_out,
                                void *x_out, char *ws, cudaStream_t s, bool *done);
+// Whether some cluster size holds the per-token state of requests of up to max_vis tokens.
+bool gram_select_fits(int max_vis);
 // Tiles of the Gram kernel for one request; floats per row of its matrix.
 int gram_tiles(int n_tokens, bool pair);
 int gram_exact_tiles(int n_tokens, bool f32);

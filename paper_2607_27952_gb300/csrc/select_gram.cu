@@ -1441,6 +1441,13 @@ SelShape shape_for(int c, int max_vis, int optin) {
 
 }  // namespace
 
+bool gram_select_fits(int max_vis) {
+  if (max_vis > 0xffff) return false;   // (token ids of 16 bits)
+  for (int c = kMaxCluster; c >= 1; --c)
+    if (shape_for(c, max_vis, kSmemOptinSm100).C != 0) return true;
+  return false;
+}
+
 cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, int32_t *idx_out,
                                void *x_out, char *ws, cudaStream_t s, bool *done) {
   *done = false;
@@ -1485,7 +1492,7 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
       best = end;
     }
   }
-  if (sh.C == 0 || pl.max_vis > 0xffff) return cudaSuccess;   // too long for a cluster: the caller's other paths
+  if (sh.C == 0 || !gram_select_fits(pl.max_vis)) return cudaSuccess;   // the caller's other paths
 
   GramArgs g;
   std::memset(&g, 0, sizeof g);

@@ -167,10 +167,6 @@ constexpr double kTriMinStreamBytes = 2.0 * 1024 * 1024;
 // the selection keeps each token's nearest root id in 16 bits
 static_assert(kMaxRoots <= 32767, "root ids must fit int16_t");
 
-// Opt-in shared memory per CTA of the sm_100 class, for checks made before a
-// device is at hand.
-constexpr int kSmemOptinSm100 = 232448;
-
 // Token block width of the kernel variant (the shared-memory plan depends on it):
 // 2 for fp32 and the tensor-core update, else 4 unless a CTA owns few tokens.
 int select_tb(int elem, bool tc, int tpc_max) { return (elem == 4 || tc || tpc_max < 64) ? 2 : 4; }

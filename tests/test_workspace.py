@@ -142,3 +142,14 @@ def test_only_requests_with_a_choice_count():
                             cu_keep=[0, 2, 4, 4 + keep_all])
         return last.last_workspace_size(prob) - least_workspace(prob)
     assert size(0) == size(1000) == 0
+
+
+def test_no_matrix_is_reserved_for_requests_too_long_for_a_cluster():
+    """Past about 53 800 tokens no cluster holds a request's per-token state: its matrix (11 to
+    12 GiB) would never be used."""
+    for n in (53000, 54000, 56000, 56700):
+        prob = _problem(1, n, n // 8)
+        used = last.last_workspace_size(prob) - least_workspace(prob) >= 4 * n * n
+        assert used == (n < 53800), n
+    prob = _problem(1, 56700, 56700 // 8)
+    assert last.last_workspace_size(prob) == least_workspace(prob)
