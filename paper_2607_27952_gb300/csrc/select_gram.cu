@@ -45,12 +45,12 @@
 //
 // Arithmetic of every decision is the canonical fp32 of the public header: the kept
 // indices are bit-identical to the sequential definition.
+#include "gram_schedule.h"
 #include "select_impl.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
-#include <functional>
-#include <vector>
 
 namespace last {
 
@@ -1462,31 +1462,23 @@ cudaError_t launch_select_gram(const Plan &pl, const float *w, const void *x, in
   else pick_nch<__nv_bfloat16, 8>((pl.dv + 255) / 256, &sel_fn, &norm_fn);
   if (pl.gram_exact) sel_fn = (void *)select_gram_kernel<1, true>;
 
-  // The cluster size with the shortest schedule: requests go, most work first, to the
-  // next free cluster; a request takes about k / 16 + 2 rounds of 27K cycles, 4.6K more
-  // per block of 32 tokens that a warp holds and 0.4K per CTA (measured: 32K cycles a
-  // round on 576 tokens in two CTAs, 66K on 4096 in one, 42K on 16384 in twelve).
+  // The cluster size with the shortest schedule (about k / 16 + 2 rounds a request).
   // Clusters of two instead of one: 2.88 -> 2.52 ms on 128 requests of 256..4096.
   const int32_t *meta = pl.host_blob.data() + pl.off_meta / 4;
   const int32_t *order = pl.host_blob.data() + pl.off_order / 4;
+  Schedule sched;
+  schedule_begin(&sched, pl.B, [&](int i) {
+    const int32_t *m = meta + order[i] * kMetaFields;
+    return SchedRequest{(m[kNumVis] + 31) / 32, m[kNumKeep] / 16.0 + 2.0};
+  });
   SelShape sh;
   double best = 0.0;
-  std::vector<double> busy;
   for (int c = 1; c <= kMaxCluster; ++c) {
     const SelShape t = shape_for(c, pl.max_vis, optin);
     if (t.C == 0) continue;
     const int active = active_clusters(sel_fn, c, t.smem, kGthreads);
     if (active <= 0) continue;
-    busy.assign(std::min(active, pl.B), 0.0);   // a heap, the next free cluster on top
-    double end = 0.0;
-    for (int i = 0; i < pl.B; ++i) {
-      const int32_t *m = meta + order[i] * kMetaFields;
-      const int slots = ((m[kNumVis] + 31) / 32 + c * kGwork - 1) / (c * kGwork);
-      std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
-      busy.back() += (m[kNumKeep] / 16.0 + 2.0) * (27.0 + 4.6 * slots + 0.4 * c);
-      end = std::max(end, busy.back());
-      std::push_heap(busy.begin(), busy.end(), std::greater<double>());
-    }
+    const double end = schedule_end(&sched, c, active, kGwork, sh.C == 0 ? INFINITY : best);
     if (sh.C == 0 || end < best) {
       sh = t;
       best = end;
