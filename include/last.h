@@ -140,7 +140,7 @@ last_status last_workspace_size(const last_problem *p, size_t *bytes);
 last_status last_scores(const last_problem *p, const void *q, const void *k, float *w_out,
                         void *ws, size_t ws_bytes, void *stream);
 
-/* Eq. 9-12.  w [cu_vis[batch]] fp32 (e.g. from last_scores); idx_out
+/* Eq. 9-12.  w [cu_vis[batch]] fp32, not negative (e.g. from last_scores); idx_out
  * [cu_keep[batch]] receives sort(S_K) per request, request-local.  When x_out
  * is not NULL the kept rows are also written there (the fused form of
  * last_gather). */

@@ -1314,8 +1314,12 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
           for (int h = 0; h < kGper; ++h) {
             const int u = lane + 32 * h;
             const float d = pm[bl * kGpairLd + u];
-            if (EX) {   // w min(delta, d) = min(w delta, w d); NaN has the largest key
-              kh[h] = kh[h] == 0u || u == bl ? 0u : min(kh[h], key_high(wv[h], d));
+            if (EX) {
+              // w min(delta, d) = min(w delta, w d) (NaN has the largest key), or for a weight
+              // below zero their maximum
+              const uint32_t kd = key_high(wv[h], d);
+              const uint32_t to = wv[h] < 0.f ? (d == d ? max(kh[h], kd) : kh[h]) : min(kh[h], kd);
+              kh[h] = kh[h] == 0u || u == bl ? 0u : to;
               continue;
             } else {
               if (!(__fsub_rd(d, eps) >= hi[h])) pend[h] |= bit;   // NaN too

@@ -141,3 +141,23 @@ def test_without_room_for_the_matrices(dtype):
     last.last_prune_host(prob, *host, None, out, None, ws)
     last.last_poll(ws)
     assert np.array_equal(out.numpy(), idx_full)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_weights_below_zero_once_all_tokens_are_candidates(dtype):
+    """Scores are never negative and the rounds rely on keys that only fall; weights below zero
+    are still taken in their order when the tokens left fit the candidate list (canonical
+    matrix: the replay follows w times the smaller distance, whatever w's sign)."""
+    rng = np.random.default_rng(5)
+    n, d = 400, 512
+    x = (rng.standard_normal((60, d))[rng.integers(0, 60, n)] + 0.05 * rng.standard_normal((n, d))).astype(np.float32)
+    x[20:60] = x[19]
+    w = (rng.random(n).astype(np.float32) - np.float32(0.3))
+    wl = _wl([n], [n - 3], d, dtype=dtype)
+    w, idx, _ = _run(wl, w=w, x=_put(wl, x))
+    assert np.array_equal(idx, np.sort(oracle_selection(wl, w, 0)))
+
+
+def _put(wl, x):
+    wl.x = f32_to_bf16_bits(x) if wl.dtype == "bf16" else x
+    return wl.x
