@@ -1,8 +1,10 @@
-"""GPU parity of the selection on inputs chosen against the tensor-core update's
-certificate: the update decides from tensor-core distances only when they are
-provably on one side of delta, and recomputes every other pair in the canonical
-fp32 order, so the kept indices must stay bit-identical to the oracle's even when
-distances are tiny, scores tie, or products cancel."""
+"""GPU parity of the selection on inputs chosen against the certificates of its tensor-core
+distances, on both paths.  The rounds over X (the call is given no room for Gram
+matrices) decide from such distances only when they are provably on one side of delta
+and recompute every other pair in the canonical fp32 order; the rounds over the matrices
+keep an interval and recompute where the order of picks depends on it.  The kept
+indices must stay bit-identical to the oracle's even when distances are tiny, scores
+tie, or products cancel."""
 import numpy as np
 import pytest
 
@@ -47,9 +49,10 @@ def _features(kind, n, dv, rng):
     raise ValueError(kind)
 
 
+@pytest.mark.parametrize("path", ["rounds", "matrix"])
 @pytest.mark.parametrize("dv", [64, 512, 2048])
 @pytest.mark.parametrize("kind", ["near_duplicates", "dynamic_range", "exact_duplicates"])
-def test_certified_update_is_exact(kind, dv):
+def test_certified_update_is_exact(kind, dv, path):
     wl = _workload(dv, [700, 250, 1300], [90, 249, 160], seed=90 + dv)
     rng = np.random.default_rng({"near_duplicates": 1, "dynamic_range": 2,
                                  "exact_duplicates": 3}[kind] * 10000 + dv)
@@ -59,6 +62,6 @@ def test_certified_update_is_exact(kind, dv):
         w32 = np.full(n, 1.0 / 700, np.float32)            # products tie wherever delta ties
     else:
         w32 = rng.dirichlet(np.ones(n)).astype(np.float32)
-    idx = DeviceWorkload(wl).select(w32)
+    idx = DeviceWorkload(wl).select(w32, path=path)
     assert_valid_selection(wl, idx)
     assert_selection_equal(wl, w32, idx, range(wl.batch))

@@ -45,6 +45,8 @@ def _run(wl, x=None, w=None):
     ([255, 256, 257, 513], [254, 1, 100, 60]),
     ([545, 640, 2049], [100, 0, 130]),
     ([8200, 90, 257], [60, 20, 60]),       # CTA pairs
+    # enough for the tensor cores at any width, one CTA a tile
+    ([1900, 255, 256, 257, 513, 127, 129, 33, 700, 96], [90, 200, 3, 100, 60, 64, 20, 2, 50, 95]),
 ])
 def test_selection_equals_the_oracle(n_vis, keep, d_v, dtype):
     wl = _wl(n_vis, keep, d_v, dtype=dtype)

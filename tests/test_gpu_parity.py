@@ -145,6 +145,19 @@ def test_feature_widths(dv):
     assert_gather_equal(wl, idx, xs, range(wl.batch))
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("dv", [8, 264, 1536, 2048])
+def test_feature_widths_in_the_rounds_over_x(dv, dtype):
+    """The same widths in rounds over X (no room for Gram matrices), on larger requests."""
+    wl = custom(name=f"dvx{dv}", seed=60 + dv, batch=3, n_vis=[330, 77, 601], n_text=[3, 3, 3],
+                num_layers=1, num_q_heads=2, num_kv_heads=1, head_dim=64, feat_dim=dv,
+                dtype=dtype, keep=[40, 9, 150], n_clusters=8, n_planted=2)
+    w = np.random.default_rng(dv).dirichlet(np.ones(int(wl.cu_vis[-1]))).astype(np.float32)
+    idx = DeviceWorkload(wl).select(w, path="rounds")
+    assert_valid_selection(wl, idx)
+    assert_selection_equal(wl, w, idx, range(wl.batch))
+
+
 @pytest.mark.parametrize("heads,kv", [(1, 1), (9, 3), (17, 17), (24, 4), (25, 5)])
 def test_head_counts_around_the_statistics_pairs(heads, kv):
     """A warp forms the statistics of heads h and h + 8 together: counts below, at and past

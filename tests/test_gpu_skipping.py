@@ -1,12 +1,14 @@
-"""GPU parity of the selection's row skipping on inputs chosen against its bounds.
+"""GPU parity of the selection on inputs chosen against the row skipping's bounds, on both of
+its paths: the rounds over X, which skip rows (the call is given no room for Gram
+matrices), and the rounds over the matrices, which these calls take by themselves.
 
-The bf16 greedy skips a (token, new centre) pair when the triangle inequality on
+Over X, the bf16 greedy skips a (token, new centre) pair when the triangle inequality on
 the unit sphere proves that the centre cannot lower the token's delta (Eq. 10):
 the bound goes through the token's nearest centre and that centre's root, with
 every computed distance widened by its rounding bound and evaluated with directed
 rounding.  A skipped pair must be one whose canonical fminf would have left delta
-unchanged, so the kept indices stay bit-identical to the oracle's.  The library
-uses the skipping only where a CTA's dense update streams at least 2 MB of rows;
+unchanged, so the kept indices stay bit-identical to the oracle's.  These
+rounds use the skipping only where a CTA's dense update streams at least 2 MB of rows;
 requests of 8192 tokens at d_v = 2048 take it for every cluster size (at most 16
 CTAs of 512 tokens, 2 MB each).
 
@@ -60,8 +62,12 @@ def _workload(batch, n, keep, seed):
                   keep=[keep])
 
 
-def _check_all(wl, w32, idx):
-    assert_valid_selection(wl, idx)
+def _check_all(wl, w32):
+    """Both paths against the oracle, which runs once."""
+    dw = DeviceWorkload(wl)
+    paths = {path: dw.select(w32, path=path) for path in ("rounds", "matrix")}
+    for idx in paths.values():
+        assert_valid_selection(wl, idx)
 
     def run(b):
         v0, v1 = int(wl.cu_vis[b]), int(wl.cu_vis[b + 1])
@@ -70,10 +76,11 @@ def _check_all(wl, w32, idx):
 
     with ThreadPoolExecutor(max_workers=_threads()) as pool:
         for b, want in pool.map(run, range(wl.batch)):
-            got = idx[wl.cu_keep[b]:wl.cu_keep[b + 1]]
-            assert np.array_equal(got, want), (
-                f"request {b}: {np.setdiff1d(got, want).tolist()[:8]} kept by GPU only, "
-                f"{np.setdiff1d(want, got).tolist()[:8]} by oracle only")
+            for path, idx in paths.items():
+                got = idx[wl.cu_keep[b]:wl.cu_keep[b + 1]]
+                assert np.array_equal(got, want), (
+                    f"{path}, request {b}: {np.setdiff1d(got, want).tolist()[:8]} kept by GPU only, "
+                    f"{np.setdiff1d(want, got).tolist()[:8]} by oracle only")
 
 
 def test_skipping_adversarial_features():
@@ -96,8 +103,7 @@ def test_skipping_adversarial_features():
         rows.append(x)
     wl.x = f32_to_bf16_bits(np.concatenate(rows).astype(np.float32))
     w32 = np.concatenate([rng.dirichlet(np.ones(n)) for _ in range(batch)]).astype(np.float32)
-    idx = DeviceWorkload(wl).select(w32)
-    _check_all(wl, w32, idx)
+    _check_all(wl, w32)
 
 
 def test_skipping_root_capacity():
@@ -110,5 +116,4 @@ def test_skipping_root_capacity():
         rows.append(proto[rng.integers(0, 1500, n)] + 0.02 * rng.standard_normal((n, dv)))
     wl.x = f32_to_bf16_bits(np.concatenate(rows).astype(np.float32))
     w32 = np.concatenate([rng.dirichlet(np.ones(n)) for _ in range(batch)]).astype(np.float32)
-    idx = DeviceWorkload(wl).select(w32)
-    _check_all(wl, w32, idx)
+    _check_all(wl, w32)
