@@ -158,17 +158,6 @@ __device__ __forceinline__ void st_cluster_v2f(uint32_t addr, float2 v) {
 __device__ __forceinline__ void st_cluster_s32(uint32_t addr, int v) {
   asm volatile("st.shared::cluster.s32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
 }
-__device__ __forceinline__ U4 ld_cluster_v4(uint32_t addr) {
-  U4 r;
-  asm volatile("ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(addr) : "memory");
-  return r;
-}
-
-__device__ __forceinline__ void st_cluster_v4u(uint32_t addr, uint4 v) {
-  asm volatile("st.shared::cluster.v4.u32 [%0], {%1,%2,%3,%4};"
-               :: "r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
 
 // ---- per-thread async copies (global -> shared), grouped ----
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {

@@ -58,8 +58,7 @@ namespace {
 
 constexpr int kGwarps = 16;
 constexpr int kGthreads = kGwarps * 32;
-constexpr bool kGspare = false;            // warp 0 alone on its scheduler: warps 4, 8, 12 own nothing
-constexpr int kGwork = kGspare ? 12 : kGwarps - 1;   // worker warps own the tokens, warp 0 replays
+constexpr int kGwork = kGwarps - 1;        // worker warps own the tokens, warp 0 replays
 constexpr int kGtok = kGwork * 32;
 constexpr int kGbatch = 8;                 // accepted centres handed to the workers at a time
 constexpr int kGlist = 64;                 // candidate list: two members per lane of the replay
@@ -717,7 +716,7 @@ select_gram_kernel(const __grid_constant__ GramSelArgs a) {
       return;
     }
   }
-  const int widx = !kGspare ? warp - 1 : (warp & 3) ? (warp >> 2) * 3 + (warp & 3) - 1 : -1;   // worker or -1
+  const int widx = warp - 1;   // worker or -1
   uint32_t *ks = reinterpret_cast<uint32_t *>(smem + S.ks);
   float *w_s = reinterpret_cast<float *>(smem + S.w);
   float *r_s = reinterpret_cast<float *>(smem + S.r);
