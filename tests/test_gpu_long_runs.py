@@ -1,9 +1,10 @@
 """Long greedy runs checked in full against the oracle (Eq. 9-11, every step).
 
-The batched rounds, the tensor-core certificate and the triangle-inequality row
-skipping all act at every step of a long greedy run, so the full-budget kept sets
-of the longest configurations are compared bit for bit with the canonical-fp32
-oracle on the GPU's own scores (the selection-on-identical-scores rule):
+The batched rounds and the bounds of their tensor-core distances act at every step of a
+long greedy run, over the Gram matrices (which these batches take) as over X (without
+room for them; there the triangle-inequality row skipping acts too).  So the full-budget
+kept sets of the longest configurations on both paths are compared bit for bit with the
+canonical-fp32 oracle on the GPU's own scores (the selection-on-identical-scores rule):
 
   * video batch (8 x 16384 tokens, k/N = 5%: k = 820) on all 8 requests, and
     k = 2048 (12.5%) on two of them;
@@ -61,6 +62,11 @@ def _oracle_sequences(wl, w32, tasks):
         return dict(pool.map(run, order))
 
 
+def _rounds_over_x(dw, w_gpu, idx, cu_keep=None):
+    """The other path's kept sets, equal to the first one's for every request."""
+    assert np.array_equal(dw.select(w_gpu, cu_keep=cu_keep, path="rounds"), idx)
+
+
 def _check(idx_gpu, cu_keep, b, seq):
     k0, k1 = int(cu_keep[b]), int(cu_keep[b + 1])
     want = oracle.restore_order(np.asarray(seq[:k1 - k0], dtype=np.int32))
@@ -80,6 +86,8 @@ def test_video_full_budget_every_request():
     big = np.arange(wl.batch + 1, dtype=np.int32) * 2048  # k = 2048 (12.5%) for every request
     idx_big = dw.select(w_gpu, cu_keep=big)
     assert_valid_selection(wl, idx_big, cu_keep=big)
+    _rounds_over_x(dw, w_gpu, idx)
+    _rounds_over_x(dw, w_gpu, idx_big, big)
     tasks = [(b, 2048 if b in long_reqs else 820) for b in range(wl.batch)]
     seqs = _oracle_sequences(wl, w_gpu, tasks)
     for b in range(wl.batch):
@@ -93,6 +101,7 @@ def test_high_resolution_eight_requests():
     dw = DeviceWorkload(wl)
     w_gpu, idx, xs = dw.prune()
     assert_valid_selection(wl, idx)
+    _rounds_over_x(dw, w_gpu, idx)
     reqs = list(range(8))
     seqs = _oracle_sequences(wl, w_gpu, [(b, int(wl.cu_keep[b + 1] - wl.cu_keep[b])) for b in reqs])
     for b in reqs:
@@ -105,6 +114,7 @@ def test_dynamic_resolution_sixteen_requests():
     dw = DeviceWorkload(wl)
     w_gpu, idx, xs = dw.prune()
     assert_valid_selection(wl, idx)
+    _rounds_over_x(dw, w_gpu, idx)
     n = np.diff(wl.cu_vis)
     longest = [int(b) for b in np.argsort(-n, kind="stable")[:4]]
     rest = [b for b in range(0, wl.batch, 7) if b not in longest][:12]
