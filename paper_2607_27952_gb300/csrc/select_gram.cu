@@ -36,8 +36,8 @@
 // rounds), of which the replay takes 650 a pick, 40K on 16384 tokens in 12 CTAs (k =
 // 2048, 76 rounds).  Measured against the rounds that stream X (GB300, whole last_prune
 // call): 64 requests of 576 x 2048, k 64/128/192: 1.71 -> 0.39 ms; 32 of 2880, k = 360:
-// 5.27 -> 1.17; 128 of 256..4096 x 1536, k = N/8: 10.3 -> 2.5; 8 of 16384 x 2048, k =
-// 2048: 16.9 -> 5.0 (3.0 of it the Gram matrix).
+// 5.27 -> 1.14; 128 of 256..4096 x 1536, k = N/8: 10.3 -> 2.41; 8 of 16384 x 2048, k =
+// 2048: 16.9 -> 4.83 (3.0 of it the Gram matrix).
 //
 // Tokens are dealt to the cluster in blocks of 32: block k belongs to CTA k % C,
 // worker warp (k / C) % 15, so neighbouring tokens (tiles, frames, near-duplicates) spread
@@ -123,6 +123,9 @@ struct GramArgs {
   int B, dv, total_tiles, chunk_kb;   // chunk_kb: K blocks per accumulation chain
   unsigned *err;
 };
+
+// An epilogue thread adds a tile row's 128 values up in registers: the ten warps are
+// allocated like twelve, 168 registers each, and both kernels spill 40 and 32 bytes.
 
 // Row i, columns j0 .. j0 + 127 of a request's matrix, and the same values as a column
 // when `mirror`.
