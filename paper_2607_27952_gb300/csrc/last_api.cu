@@ -186,9 +186,9 @@ last_status make_plan(const last_problem *p, bool need_scores, bool need_select,
   // x 64 at k = 2 1723 / 303, 256 1864 / 1628; x 2048 at 32 3169 / 2580, 64 3203 / 3378, 256
   // 3323 / 6006; one of 50000 x 64 at 2 1971 / 564, 32 2096 / 1550, 128 2236 / 2570; two of
   // 16384 x 256 at 2 489 / 266, 16 528 / 574; 64 of 2048 x 256 at 2 327 / 263, 4 337 / 360; 32
-  // of 2880 x 2048 at 2 630 / 652.  Of the 300 shapes so measured three take the slower side
-  // by more than 6% (13 to 26%).  The second line, in products alone, was drawn first; it
-  // holds back matrices at tiny budgets of wide features.
+  // of 2880 x 2048 at 2 630 / 652.  Of 361 shapes so measured, fp32 ones included, four take
+  // the slower side by more than 6% (8 to 26%).  The second line, in products alone, keeps
+  // wide features at tiny budgets on the rounds, which is where it was measured.
   // fp32, canonical order: 576 x 1024 at k = 2 39 / 30, 4 43 / 46; two of 2048 at 32 350 / 319,
   // 64 378 / 598; four of 4096 at 128 2456 / 1585; 10000 at 128 3551 / 3313; 12000 x 8 at 8 1834
   // / 455; 8 of 1200 x 64 at 8 203 / 141, 32 220 / 276 (rows narrower than 32 lanes' worth of
